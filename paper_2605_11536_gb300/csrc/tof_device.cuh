@@ -280,6 +280,205 @@ static __device__ __noinline__ bool traverse(const GeomDev& g, float3 o, float3 
     return found;
 }
 
+// ---- traversal of queued rays ----------------------------------------------------------------
+// three-way minimum / maximum (one instruction on sm_100 and later; a NaN operand is dropped, as by
+// fminf / fmaxf)
+static __device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+static __device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+// distances (lo * s - o, hi * s - o) of a slab's two planes, each one rounding, as one packed
+// instruction
+static __device__ __forceinline__ void slab(float lo, float hi, float s, float o, float& ta, float& tb) {
+    asm("{ .reg .b64 p, q, r;\n"
+        "mov.b64 p, {%2, %3};\n"
+        "mov.b64 q, {%4, %4};\n"
+        "mov.b64 r, {%5, %5};\n"
+        "fma.rn.f32x2 p, p, q, r;\n"
+        "mov.b64 {%0, %1}, p; }"
+        : "=f"(ta), "=f"(tb) : "f"(lo), "f"(hi), "f"(s), "f"(-o));
+}
+// entry distances lo0, lo1 of a ray into the boxes of a node's children (above their exit, or beyond
+// `best`: missed) and the children.  The node is read by two 32-byte loads: the lanes of a warp
+// read scattered nodes, each load costs the L1 one wavefront a lane whatever its width, and with
+// four 16-byte loads that data path stood at 76 % of its peak (dynamic gated workload, 512 x 512).
+static __device__ __forceinline__ void node_test(const float4* __restrict__ nodes, int node, float3 id, float3 ood, float best,
+                                                 float& lo0, bool& h0, int& ch0, float& lo1, bool& h1, int& ch1) {
+    const float4* N = nodes + 4 * node;
+    unsigned long long q[8];
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(q[0]), "=l"(q[1]), "=l"(q[2]), "=l"(q[3]) : "l"(N));
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(q[4]), "=l"(q[5]), "=l"(q[6]), "=l"(q[7]) : "l"(N + 2));
+    float v[14];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        v[2 * i] = __uint_as_float((uint32_t)q[i]);
+        v[2 * i + 1] = __uint_as_float((uint32_t)(q[i] >> 32));
+    }
+    float a0, a1, b0, b1, c0, c1;
+    slab(v[0], v[1], id.x, ood.x, a0, a1);
+    slab(v[2], v[3], id.y, ood.y, b0, b1);
+    slab(v[8], v[9], id.z, ood.z, c0, c1);
+    lo0 = fmaxf(max3(fminf(a0, a1), fminf(b0, b1), fminf(c0, c1)), 0.f);
+    h0 = lo0 <= fminf(min3(fmaxf(a0, a1), fmaxf(b0, b1), fmaxf(c0, c1)), best);
+    slab(v[4], v[5], id.x, ood.x, a0, a1);
+    slab(v[6], v[7], id.y, ood.y, b0, b1);
+    slab(v[10], v[11], id.z, ood.z, c0, c1);
+    lo1 = fmaxf(max3(fminf(a0, a1), fminf(b0, b1), fminf(c0, c1)), 0.f);
+    h1 = lo1 <= fminf(min3(fmaxf(a0, a1), fmaxf(b0, b1), fmaxf(c0, c1)), best);
+    ch0 = __float_as_int(v[12]);
+    ch1 = __float_as_int(v[13]);
+}
+
+// a ray's traversal between two rounds
+struct RayState {
+    float3 o, d, id, ood;
+    float tmax, best, b1, b2;
+    int tri, node, sp, budget;
+    bool found;
+    __device__ __forceinline__ void start(float3 o_, float3 d_, float tmax_, int nt) {
+        o = o_; d = d_; tmax = tmax_;
+        id = f3(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
+        ood = f3(o.x * id.x, o.y * id.y, o.z * id.z);
+        best = tmax; tri = 0; b1 = b2 = 0.f; found = false;
+        node = 0; sp = 0;
+        // a valid hierarchy visits each of its nt - 1 internal nodes at most once per ray; the cap
+        // only guards against a malformed one, and running into it is reported in the error word
+        budget = nt + 64;
+    }
+};
+
+// One round of a traversal: up to kRun node visits, whose leaves are collected, then the triangle
+// tests of those leaves; true when the ray is settled.  A warp's lanes reach leaves at different
+// visits (a tenth of the boxes met are leaves), so testing each where it is met runs the
+// triangle code at almost every visit with two or three lanes of 32; collected, the tests of kRun
+// visits share one short loop.  The closest hit does not depend on the order of the tests (closer()),
+// and a hit known later only costs visits.
+template <bool kAny, int kRun>
+static __device__ __forceinline__ bool trav_round(const float4* __restrict__ nodes, const float4* __restrict__ leaf, int nt, RayState& r,
+                                                  int* stack, unsigned& fault) {
+    int pend[2 * kRun];
+    int np = 0;
+    if (nt > 1) {
+#pragma unroll 1
+        for (int step = 0; step < kRun; ++step) {
+            if (--r.budget < 0) {
+                fault |= kErrVisitBudget;
+                r.node = -1;
+                break;
+            }
+            float lo0, lo1;
+            bool h0, h1;
+            int ch0, ch1;
+            node_test(nodes, r.node, r.id, r.ood, r.best, lo0, h0, ch0, lo1, h1, ch1);
+            if (h0 && ch0 < 0) { pend[np++] = ~ch0; h0 = false; }
+            if (h1 && ch1 < 0) { pend[np++] = ~ch1; h1 = false; }
+            if (h0 && h1) {
+                if (r.sp < kStack) stack[r.sp++] = lo0 <= lo1 ? ch1 : ch0;
+                else fault |= kErrStackOverflow;   // the far subtree is skipped: reported in the error word
+                r.node = lo0 <= lo1 ? ch0 : ch1;
+            } else if (h0) {
+                r.node = ch0;
+            } else if (h1) {
+                r.node = ch1;
+            } else {
+                if (r.sp == 0) {
+                    r.node = -1;
+                    break;
+                }
+                r.node = stack[--r.sp];
+            }
+        }
+    } else {
+        r.node = -1;
+        if (nt == 1) pend[np++] = 0;
+    }
+#pragma unroll 1
+    for (int k = 0; k < np; ++k) {
+        float t, u, w;
+        int orig;
+        if (tri_test(leaf, pend[k], r.o, r.d, r.best, t, u, w, orig) && (r.found || t < r.tmax) && closer(r.found, t, orig, r.best, r.tri)) {
+            r.best = t; r.tri = orig; r.b1 = u; r.b2 = w; r.found = true;
+            if (kAny) return true;
+        }
+    }
+    return r.node < 0;
+}
+
+// The n rays of a queue, traced by a persistent grid: Q::load(i, o, d, tmax) reads ray i, Q::done(ray)
+// takes its answer.  kAny: whether anything is hit; else the closest hit.
+//
+// Bound by issue (the min / max of the slab tests and the divergence of a warp's rays), the L1's data path
+// (node_test) and, with few rays, by the longest ray's chain of node visits.
+// * A round has 8 node visits (of 1, 2, 4, 8, 12, 16: 3.45, 3.21, 3.13, 3.02, 2.98, 2.97 ms a frame, but a few
+//   us longer for short queues from 12 on; leaves tested where they were met: 3.11).
+// * A lane whose ray is settled takes another one between two rounds once a quarter of its warp waits; the
+//   warp draws its rays from the queue 32 at a time, one atomic for them (`fetch`).
+// * A queue shorter than the grid's lanes is shared out evenly without an atomic, at least min_rays to a
+//   warp: a kernel alone on the GPU (4) runs a few rays in many warps instead of diverging in a few
+//   (64 x 64 frame 218 -> 206 us); beside other kernels the issue slots of full warps count more (32; 4 cost
+//   5 % of a batch of 32 views).
+// Both together, and the 32-byte node loads: dynamic gated 512 x 512 frame 3.14 -> 2.92 ms, its visibility
+// kernels 826 -> 710 us; 1024 x 1024 12.0 -> 11.2 ms.
+constexpr int kQueueRun = 8;
+constexpr uint32_t kAloneRays = 4;
+template <bool kAny, class Q>
+static __device__ __forceinline__ void trace_queue(const GeomDev& g, uint32_t n, uint32_t* fetch, uint32_t min_rays, Q& q) {
+    const float4* __restrict__ nodes = g.nodes;
+    const float4* __restrict__ leaf = g.leaf;
+    const int nt = g.nt;
+    unsigned* const err = g.err;
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t chunk = min(32u, max(min_rays, (n + warps - 1) / warps));
+    const uint32_t lanes = 0xFFFFFFFFu >> (32u - chunk);
+    const int refill = max(1, (int)chunk / 4);
+    unsigned fault = 0u;
+    bool has = false;
+    // the warp's rays not yet on a lane: its share of a short queue, else drawn as they are needed
+    uint32_t pool = 0, pool_end = 0;
+    bool drained = n <= warps * chunk;
+    if (drained) {
+        pool = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * chunk;
+        pool_end = min(pool + chunk, n);
+        if (pool >= n) return;
+    }
+    RayState r;
+    int stack[kStack];
+    while (true) {
+        const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !has) & lanes;
+        if (__popc(idle) >= refill) {
+            if (pool == pool_end && !drained) {
+                if (lane == 0) pool = atomicAdd(fetch, chunk);
+                pool = __shfl_sync(0xFFFFFFFFu, pool, 0);
+                pool_end = min(pool + chunk, n);
+                if (pool >= n) { drained = true; pool_end = pool; }
+            }
+            if (drained && idle == lanes && pool == pool_end) break;
+            const uint32_t rank = (uint32_t)__popc(idle & ((1u << lane) - 1u));
+            const uint32_t take = min((uint32_t)__popc(idle), pool_end - pool);
+            if (!has && ((lanes >> lane) & 1u) && rank < take) {
+                float3 o, d;
+                float tmax;
+                q.load(pool + rank, o, d, tmax);
+                r.start(o, d, tmax, nt);
+                has = true;
+            }
+            pool += take;
+        }
+        if (has && trav_round<kAny, kQueueRun>(nodes, leaf, nt, r, stack, fault)) {
+            q.done(r);
+            has = false;
+        }
+    }
+    if (fault && err) atomicOr(err, fault);
+}
+
 static __device__ __forceinline__ bool trace_from(const GeomDev& g, const Surf& s, float3 d, float eps, Surf& hit) {
     float3 o = offset_point(s.p, s.n, d, eps);
     int tri; float b1, b2, t;

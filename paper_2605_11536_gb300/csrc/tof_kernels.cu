@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(128) tree_select_kernel(const __grid_constant_
 //   tw_start_kernel   one thread per path: vertex 1 (the G-buffer hit), its NEE candidate, the
 //                     first bounce
 //   tw_hit_kernel     per round, the closest hits of the round's bounce rays (persistent, each lane
-//                     refilled with the next ray between rounds of kHitSteps node visits)
+//                     refilled with the next ray between rounds of node visits)
 //   tw_shade_kernel   per round, one thread per hit: the vertex record, the NEE candidate (its light
 //                     segment queued for vis_kernel) and the next bounce
 //   vis_kernel        the light segments; an occluded one zeroes its candidate's weight
@@ -620,107 +620,25 @@ __global__ void __launch_bounds__(128) tw_start_kernel(const __grid_constant__ I
     }
 }
 
-// closest hits of the rays of one round: the loop of traverse<false> with the vis_kernel's lane
-// refill; hits[i] = (tri, b1, b2, t) of ray i, or kNoHit
-constexpr int kHitSteps = 32;
+// closest hits of the rays of one round (trace_queue); hits[i] = (tri, b1, b2, t) of ray i, or kNoHit
+struct HitQueue {
+    const float4* rays;
+    float4* hits;
+    uint32_t cur;
+    __device__ void load(uint32_t i, float3& o, float3& d, float& tmax) {
+        float4 ra = rays[2 * (size_t)i], rb = rays[2 * (size_t)i + 1];
+        o = f3(ra.x, ra.y, ra.z); d = f3(rb.x, rb.y, rb.z); tmax = ra.w;
+        cur = i;
+    }
+    __device__ void done(const RayState& r) {
+        hits[cur] = r.found ? make_float4(__int_as_float(r.tri), r.b1, r.b2, r.best) : make_float4(__uint_as_float(kNoHit), 0.f, 0.f, 0.f);
+    }
+};
 __global__ void __launch_bounds__(128, 8) tw_hit_kernel(const GeomDev gref, const float4* __restrict__ rays, const uint32_t* counter,
                                                      uint32_t cap, uint32_t* fetch, float4* __restrict__ hits) {
-    GeomDev g;
-    g.nodes = gref.nodes; g.leaf = gref.leaf; g.nt = gref.nt; g.err = gref.err;
-    const uint32_t n = min(*counter, cap);
-    const int lane = threadIdx.x & 31;
-    unsigned fault = 0u;
-    bool has = false, done = false, found = false;
-    float3 o = f3(0.f, 0.f, 0.f), d = o, id = o, ood = o;
-    float tmax = 0.f, best = 0.f, bb1 = 0.f, bb2 = 0.f;
-    int btri = 0;
-    uint32_t cur = 0;
-    int node = 0, sp = 0, budget = 0;
-    int stack[kStack];
-    while (true) {
-        const bool need = !has && !done;
-        const uint32_t want = __ballot_sync(0xFFFFFFFFu, need);
-        if (want) {
-            const int leader = __ffs(want) - 1;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(want));
-            base = __shfl_sync(0xFFFFFFFFu, base, leader);
-            if (need) {
-                const uint32_t i = base + (uint32_t)__popc(want & ((1u << lane) - 1u));
-                if (i < n) {
-                    float4 ra = rays[2 * (size_t)i], rb = rays[2 * (size_t)i + 1];
-                    o = f3(ra.x, ra.y, ra.z); d = f3(rb.x, rb.y, rb.z); tmax = ra.w;
-                    id = f3(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
-                    ood = f3(o.x * id.x, o.y * id.y, o.z * id.z);
-                    cur = i; found = false; best = tmax;
-                    node = 0; sp = 0; budget = g.nt + 64;
-                    has = true;
-                } else {
-                    done = true;
-                }
-            }
-        }
-        if (__all_sync(0xFFFFFFFFu, done)) break;
-        bool fin = false;
-        for (int step = 0; step < kHitSteps && has; ++step) {
-            if (g.nt <= 1) {
-                float t, u, v; int orig;
-                if (g.nt == 1 && tri_test(g.leaf, 0, o, d, best, t, u, v, orig) && t < tmax) {
-                    found = true; best = t; btri = orig; bb1 = u; bb2 = v;
-                }
-                has = false; fin = true;
-                break;
-            }
-            if (--budget < 0) {
-                fault |= kErrVisitBudget;
-                has = false; fin = true;
-                break;
-            }
-            const float4* N = g.nodes + 4 * node;
-            float4 n0 = __ldg(N), n1 = __ldg(N + 1), n2 = __ldg(N + 2), n3 = __ldg(N + 3);
-            float a0 = n0.x * id.x - ood.x, a1 = n0.y * id.x - ood.x;
-            float b0 = n0.z * id.y - ood.y, c1y = n0.w * id.y - ood.y;
-            float c0 = n2.x * id.z - ood.z, c1 = n2.y * id.z - ood.z;
-            float lo0 = fmaxf(fmaxf(fminf(a0, a1), fminf(b0, c1y)), fmaxf(fminf(c0, c1), 0.f));
-            float hi0 = fminf(fminf(fmaxf(a0, a1), fmaxf(b0, c1y)), fminf(fmaxf(c0, c1), best));
-            float d0 = n1.x * id.x - ood.x, d1 = n1.y * id.x - ood.x;
-            float e0 = n1.z * id.y - ood.y, e1 = n1.w * id.y - ood.y;
-            float f0 = n2.z * id.z - ood.z, f1 = n2.w * id.z - ood.z;
-            float lo1 = fmaxf(fmaxf(fminf(d0, d1), fminf(e0, e1)), fmaxf(fminf(f0, f1), 0.f));
-            float hi1 = fminf(fminf(fmaxf(d0, d1), fmaxf(e0, e1)), fminf(fmaxf(f0, f1), best));
-            bool h0 = lo0 <= hi0, h1 = lo1 <= hi1;
-            int ch0 = __float_as_int(n3.x), ch1 = __float_as_int(n3.y);
-            if (h0 && ch0 < 0) {
-                float t, u, v; int orig;
-                if (tri_test(g.leaf, ~ch0, o, d, best, t, u, v, orig) && (found || t < tmax) && closer(found, t, orig, best, btri)) {
-                    best = t; btri = orig; bb1 = u; bb2 = v; found = true;
-                }
-                h0 = false;
-            }
-            if (h1 && ch1 < 0) {
-                float t, u, v; int orig;
-                if (tri_test(g.leaf, ~ch1, o, d, best, t, u, v, orig) && (found || t < tmax) && closer(found, t, orig, best, btri)) {
-                    best = t; btri = orig; bb1 = u; bb2 = v; found = true;
-                }
-                h1 = false;
-            }
-            if (h0 && h1) {
-                int nearc = lo0 <= lo1 ? ch0 : ch1, farc = lo0 <= lo1 ? ch1 : ch0;
-                if (sp < kStack) stack[sp++] = farc;
-                else fault |= kErrStackOverflow;   // the far subtree is skipped: reported after the loop
-                node = nearc;
-            } else if (h0) {
-                node = ch0;
-            } else if (h1) {
-                node = ch1;
-            } else {
-                if (sp == 0) { has = false; fin = true; break; }
-                node = stack[--sp];
-            }
-        }
-        if (fin) hits[cur] = found ? make_float4(__int_as_float(btri), bb1, bb2, best) : make_float4(__uint_as_float(kNoHit), 0.f, 0.f, 0.f);
-    }
-    if (fault && g.err) atomicOr(g.err, fault);
+    HitQueue q;
+    q.rays = rays; q.hits = hits; q.cur = 0;
+    trace_queue<false>(gref, min(*counter, cap), fetch, kAloneRays, q);
 }
 
 // the hits of the round towards vertex d: one thread per ray

@@ -292,114 +292,37 @@ __global__ void __launch_bounds__(128, 8) shift_fwd_kernel(const __grid_constant
 }
 
 // --------------------------------------------------------------------------------------------
-// visibility segments queued by a shift kernel; an occluded segment zeroes the result it guards.
-// Persistent, with dynamic fetch: a lane whose segment is settled takes the next queued one
-// between rounds of at most kVisSteps node visits, so lanes do not idle while the warp's longest
-// traversal (grazing segments over a heightfield visit many nodes) runs to its end.  Each
-// segment's node visits are those of traverse<true> in the same order, so the answer is the same.
+// visibility segments queued by a shift kernel (trace_queue); an occluded segment zeroes the result it
+// guards.  Each segment's node visits are those of traverse<true>, so the answer is the same.
 // stat >= 0: the stats counter that counted the guarded shifts as successes (one decrement per
 // shift, however many of its segments are occluded); ray_stat >= 0: the counter of segments.
 // --------------------------------------------------------------------------------------------
-constexpr int kVisSteps = 32;   // 8: 4.63, 16: 4.52, 32: 4.49-4.51, 64 / 128: 4.50 ms per 512 x 512 frame
+struct SegQueue {
+    const float4* rays;
+    float* target;
+    uint32_t tgt;
+    unsigned int lost;
+    __device__ void load(uint32_t i, float3& o, float3& d, float& tmax) {
+        float4 a = rays[2 * (size_t)i], b = rays[2 * (size_t)i + 1];
+        o = f3(a.x, a.y, a.z); d = f3(b.x, b.y, b.z); tmax = a.w; tgt = __float_as_uint(b.w);
+    }
+    __device__ void done(const RayState& r) {
+        if (!r.found) return;
+        float old = atomicExch(&target[tgt], 0.f);
+        if (old != 0.f) ++lost;
+    }
+};
 
 __device__ __forceinline__ void vis_body(const GeomDev& gref, const float4* __restrict__ rays, const uint32_t* counter,
-                                         uint32_t cap, uint32_t* fetch, float* target, StatsDev* stats, int stat, int ray_stat) {
-    // the hierarchy in registers (a batched launch passes the instance's GeomDev in shared memory)
-    GeomDev g;
-    g.nodes = gref.nodes; g.leaf = gref.leaf; g.nt = gref.nt; g.err = gref.err;
+                                         uint32_t cap, uint32_t* fetch, float* target, StatsDev* stats, int stat, int ray_stat,
+                                         uint32_t min_rays) {
     const uint32_t n = min(*counter, cap);
     if (stats && ray_stat >= 0 && blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&stats->v[ray_stat], (unsigned long long)n);
     const int lane = threadIdx.x & 31;
-    unsigned long long lost = 0;
-    unsigned fault = 0u;         // traversal overflows of this lane, published after the loop
-    bool has = false, done = false;
-    float3 o = f3(0.f, 0.f, 0.f), d = o, id = o, ood = o;
-    float tmax = 0.f;
-    uint32_t tgt = 0;
-    int node = 0, sp = 0, budget = 0;
-    int stack[kStack];
-    while (true) {
-        // refill: every lane of the warp takes part (uniform control flow around the ballot)
-        const bool need = !has && !done;
-        const uint32_t want = __ballot_sync(0xFFFFFFFFu, need);
-        if (want) {
-            const int leader = __ffs(want) - 1;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(want));
-            base = __shfl_sync(0xFFFFFFFFu, base, leader);
-            if (need) {
-                const uint32_t i = base + (uint32_t)__popc(want & ((1u << lane) - 1u));
-                if (i < n) {
-                    float4 a = rays[2 * (size_t)i], b = rays[2 * (size_t)i + 1];
-                    o = f3(a.x, a.y, a.z); d = f3(b.x, b.y, b.z); tmax = a.w; tgt = __float_as_uint(b.w);
-                    id = f3(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
-                    ood = f3(o.x * id.x, o.y * id.y, o.z * id.z);
-                    node = 0; sp = 0; budget = g.nt + 64;
-                    has = true;
-                } else {
-                    done = true;
-                }
-            }
-        }
-        if (__all_sync(0xFFFFFFFFu, done)) break;
-        bool hit = false;
-        for (int step = 0; step < kVisSteps && has; ++step) {
-            if (g.nt <= 0) { has = false; break; }
-            if (g.nt == 1) {
-                float t, u, w; int orig;
-                hit = tri_test(g.leaf, 0, o, d, tmax, t, u, w, orig) && t < tmax;
-                has = false;
-                break;
-            }
-            if (--budget < 0) {
-                fault |= kErrVisitBudget;
-                has = false;
-                break;
-            }
-            const float4* N = g.nodes + 4 * node;
-            float4 n0 = __ldg(N), n1 = __ldg(N + 1), n2 = __ldg(N + 2), n3 = __ldg(N + 3);
-            float a0 = n0.x * id.x - ood.x, a1 = n0.y * id.x - ood.x;
-            float b0 = n0.z * id.y - ood.y, bb1 = n0.w * id.y - ood.y;
-            float c0 = n2.x * id.z - ood.z, c1 = n2.y * id.z - ood.z;
-            float lo0 = fmaxf(fmaxf(fminf(a0, a1), fminf(b0, bb1)), fmaxf(fminf(c0, c1), 0.f));
-            float hi0 = fminf(fminf(fmaxf(a0, a1), fmaxf(b0, bb1)), fminf(fmaxf(c0, c1), tmax));
-            float d0 = n1.x * id.x - ood.x, d1 = n1.y * id.x - ood.x;
-            float e0 = n1.z * id.y - ood.y, e1 = n1.w * id.y - ood.y;
-            float f0 = n2.z * id.z - ood.z, f1 = n2.w * id.z - ood.z;
-            float lo1 = fmaxf(fmaxf(fminf(d0, d1), fminf(e0, e1)), fmaxf(fminf(f0, f1), 0.f));
-            float hi1 = fminf(fminf(fmaxf(d0, d1), fmaxf(e0, e1)), fminf(fmaxf(f0, f1), tmax));
-            bool h0 = lo0 <= hi0, h1 = lo1 <= hi1;
-            int ch0 = __float_as_int(n3.x), ch1 = __float_as_int(n3.y);
-            if (h0 && ch0 < 0) {
-                float t, u, w; int orig;
-                if (tri_test(g.leaf, ~ch0, o, d, tmax, t, u, w, orig) && t < tmax) { hit = true; has = false; break; }
-                h0 = false;
-            }
-            if (h1 && ch1 < 0) {
-                float t, u, w; int orig;
-                if (tri_test(g.leaf, ~ch1, o, d, tmax, t, u, w, orig) && t < tmax) { hit = true; has = false; break; }
-                h1 = false;
-            }
-            if (h0 && h1) {
-                int nearc = lo0 <= lo1 ? ch0 : ch1, farc = lo0 <= lo1 ? ch1 : ch0;
-                if (sp < kStack) stack[sp++] = farc;
-                else fault |= kErrStackOverflow;   // the far subtree is skipped: reported after the loop
-                node = nearc;
-            } else if (h0) {
-                node = ch0;
-            } else if (h1) {
-                node = ch1;
-            } else {
-                if (sp == 0) { has = false; break; }
-                node = stack[--sp];
-            }
-        }
-        if (hit) {
-            float old = atomicExch(&target[tgt], 0.f);
-            if (old != 0.f) ++lost;
-        }
-    }
-    if (fault && g.err) atomicOr(g.err, fault);
+    SegQueue q;
+    q.rays = rays; q.target = target; q.lost = 0; q.tgt = 0;
+    trace_queue<true>(gref, n, fetch, min_rays, q);
+    const unsigned long long lost = q.lost;
     if (stats && stat >= 0) {
         unsigned long long x = lost;
         for (int o2 = 16; o2 > 0; o2 >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o2);
@@ -409,7 +332,7 @@ __device__ __forceinline__ void vis_body(const GeomDev& gref, const float4* __re
 __global__ void __launch_bounds__(128, 8) vis_kernel(const GeomDev g, const float4* __restrict__ rays, const uint32_t* counter,
                                                   uint32_t cap, uint32_t* fetch, float* target, StatsDev* stats, int stat,
                                                   int ray_stat) {
-    vis_body(g, rays, counter, cap, fetch, target, stats, stat, ray_stat);
+    vis_body(g, rays, counter, cap, fetch, target, stats, stat, ray_stat, kAloneRays);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -706,13 +629,13 @@ __global__ void __launch_bounds__(128, 8) reuse_persist_batch_kernel(const Reuse
         const WaveDev& w = s.w;
         if constexpr (kStage == 0) shift_fwd_body<false>(a, w);
         else if constexpr (kStage == 1)
-            vis_body(a.cur.g, w.rays, &w.counters[4], w.ray_cap, &w.counters[6], w.py, a.stats, 4, a.temporal ? -1 : 8);
+            vis_body(a.cur.g, w.rays, &w.counters[4], w.ray_cap, &w.counters[6], w.py, a.stats, 4, a.temporal ? -1 : 8, 32u);
         else if constexpr (kStage == 2) emit_inv_body(a, w);
         else if constexpr (kStage == 3)
             shift_inv_body<false>(a, w, 0u, min(w.counters[2], inv_task_cap(w)), w.rays, &w.counters[5], w.ray_cap);
         else if constexpr (kStage == 4)
             vis_body(a.temporal ? a.prev.g : a.cur.g, w.rays, &w.counters[5], w.ray_cap, &w.counters[7], w.terms, a.stats, -1,
-                     a.temporal ? -1 : 9);
+                     a.temporal ? -1 : 9, 32u);
         else reuse_merge_body(a, w);
     }
 }
