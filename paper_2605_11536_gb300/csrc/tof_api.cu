@@ -29,9 +29,9 @@ cudaError_t launch_initial_ell_tree_wave(const InitArgs& a, const TreeWaveDev& t
                                          int place_blocks, int vis_blocks, cudaStream_t s);
 cudaError_t ell_place_blocks(int* out);
 cudaError_t launch_initial_shrink(const InitArgs& a, int tile_h, cudaStream_t s);
-cudaError_t launch_reuse_wave(const ReuseArgs& a, const WaveDev& w, int p0, int p1, int persist_blocks, int vis_blocks,
-                              cudaEvent_t* ev, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join);
-cudaError_t reuse_persist_blocks(int* out, int* vis_out);
+cudaError_t launch_reuse_wave(const ReuseArgs& a, const WaveDev& w, int p0, int p1, int persist_blocks, int shift_blocks,
+                              int vis_blocks, cudaEvent_t* ev, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join);
+cudaError_t reuse_persist_blocks(int* merge_out, int* shift_out, int* vis_out);
 cudaError_t launch_splat(const SplatArgs& a, cudaStream_t s);
 cudaError_t launch_pt(const PtArgs& a, cudaStream_t s);
 cudaError_t launch_laser(const GeomDev& g, float3 o, float3 d, float power, LightDev* out, cudaStream_t s);
@@ -153,7 +153,8 @@ struct tof_ctx {
     unsigned* d_err = nullptr;   // device error word (kErr* bits), set by kernels
     unsigned* h_err = nullptr;   // pinned host mirror of it, copied after every render on its stream
     float* d_scratch = nullptr;  // laser spot of plain PT renders
-    int persist_blocks = 0;      // resident blocks of the persistent reuse kernels (all SMs)
+    int persist_blocks = 0;      // resident blocks of the merge and the batched reuse stages (all SMs)
+    int shift_blocks = 0;        // resident blocks of the shift kernels (all SMs)
     int ell_blocks = 0;          // resident blocks of the ellipsoidal placement kernel (all SMs)
     int hit_blocks = 0;          // resident blocks of the wavefront closest-hit kernel (all SMs)
     int vis_blocks = 0;          // resident blocks of the visibility kernel (all SMs)
@@ -668,7 +669,7 @@ constexpr int kReuseEvents = 7;   // events around the kernels of one reuse laun
 // resident-block counts of the persistent reuse kernels, once per context
 static tof_status persist_init(tof_ctx* c) {
     if (c->persist_blocks) return TOF_OK;
-    CK(reuse_persist_blocks(&c->persist_blocks, &c->vis_blocks));
+    CK(reuse_persist_blocks(&c->persist_blocks, &c->shift_blocks, &c->vis_blocks));
     CK(ell_place_blocks(&c->ell_blocks));
     CK(tree_hit_blocks(&c->hit_blocks));
     CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
@@ -852,12 +853,13 @@ static tof_status reuse_pass(tof_ctx* c, ViewH& V, const ReuseArgs& ra, const Wa
             g_rec->pass[g_rec->q].push_back(J);
             continue;
         }
-        int pb = c->persist_blocks, vb = c->vis_blocks;
+        int pb = c->persist_blocks, sb = c->shift_blocks, vb = c->vis_blocks;
         if (V.tune.packet > 0) {
             pb = std::min(pb, c->sms * V.tune.packet);
+            sb = std::min(sb, c->sms * V.tune.packet);
             vb = std::min(vb, c->sms * V.tune.packet);
         }
-        CK(launch_reuse_wave(ra, w, (int)p0, (int)p1, pb, vb, ev, s, beside ? V.side : nullptr, V.side_fork, V.side_join));
+        CK(launch_reuse_wave(ra, w, (int)p0, (int)p1, pb, sb, vb, ev, s, beside ? V.side : nullptr, V.side_fork, V.side_join));
     }
     if (g_rec) ++g_rec->q;
     return TOF_OK;

@@ -879,6 +879,152 @@ static __device__ __noinline__ void build_rec(const Domain& D, const TreeVerts& 
 }
 
 // ============================================================================================
+// Fixed rounding.  The shift's functions with every multiplication and addition rounded in one given way (a
+// dot product as fma(z, z', fma(x, x', y y')), a difference of products as fma(a, b, -(c d))).  Left to the
+// compiler, which products it fuses depends on how often each is used nearby, so the same expression
+// rounds differently in code that is cut in another way; here a shift's bits do not depend on which kernel
+// runs it, and these are the roundings that the one-kernel form had.
+// ============================================================================================
+static __device__ __forceinline__ float dot3c(float3 a, float3 b) {
+    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+static __device__ __forceinline__ float len3c(float3 a) { return sqrtf(dot3c(a, a)); }
+static __device__ __forceinline__ float3 scale3c(float3 a, float s) { return f3(__fmul_rn(a.x, s), __fmul_rn(a.y, s), __fmul_rn(a.z, s)); }
+static __device__ __forceinline__ float3 sum3c(float3 a, float3 b) { return f3(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z)); }
+// a b - c d
+static __device__ __forceinline__ float det2c(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+// a / b correctly rounded, from rb = 1 / b correctly rounded: q = a rb is within one unit of the quotient,
+// and q + (a - b q) rb then rounds to it (Markstein, IBM J. Res. Dev. 34(1), 1990).  Three operations where
+// several numerators share b, against a full division with its branch for extreme operands each; b and
+// the quotient have to be far from the ends of the exponent range.
+static __device__ __forceinline__ float div_by(float a, float b, float rb) {
+    const float q = __fmul_rn(a, rb);
+    return __fmaf_rn(__fmaf_rn(-b, q, a), rb, q);
+}
+static __device__ __forceinline__ float3 norm3c(float3 a) {
+    const float l = len3c(a);
+    return scale3c(a, l > 0.f ? 1.0f / l : 0.f);
+}
+static __device__ __forceinline__ float3 dir_toc(float3 from, float3 to) { return norm3c(to - from); }
+static __device__ __forceinline__ float Gtermc(float3 ap, float3 an, float3 bp, float3 bn) {
+    const float3 d = bp - ap;
+    const float d2 = dot3c(d, d);
+    if (!(d2 > 0.f)) return 0.f;
+    const float3 w = scale3c(d, 1.0f / sqrtf(d2));
+    return fabsf(dot3c(an, w)) * fabsf(dot3c(bn, w)) / d2;
+}
+static __device__ __forceinline__ float ggx_Dc(float nh, float a) {
+    const float a2 = __fmul_rn(a, a), t = __fmaf_rn(__fmul_rn(nh, nh), __fadd_rn(a2, -1.0f), 1.0f);
+    return a2 / __fmul_rn(__fmul_rn(kPi, t), t);
+}
+static __device__ __forceinline__ float ggx_G1c(float nv, float a) {
+    const float a2 = __fmul_rn(a, a);
+    return __fmul_rn(2.0f, nv) / __fadd_rn(nv, sqrtf(__fmaf_rn(__fmul_rn(__fadd_rn(1.0f, -a2), nv), nv, a2)));
+}
+// kReplay: the length of the half vector summed from the other end, as the replayed vertices of the one-kernel
+// form had it
+template <bool kReplay = false>
+static __device__ __forceinline__ float bsdf_fc(const Mat& m, float3 n, float3 wi, float3 wo) {
+    float ci = dot3c(n, wi), co = dot3c(n, wo);
+    if (ci * co <= 0.f) return 0.f;
+    if (ci < 0.f) { ci = -ci; co = -co; n = n * -1.0f; }
+    if (m.type == M_LAMBERT) return m.albedo / kPi;
+    if (m.type == M_GGX) {
+        const float3 hs = sum3c(wi, wo);
+        const float hl = kReplay ? sqrtf(__fmaf_rn(hs.z, hs.z, __fmaf_rn(hs.y, hs.y, __fmul_rn(hs.x, hs.x)))) : len3c(hs);
+        const float3 h = scale3c(hs, hl > 0.f ? 1.0f / hl : 0.f);
+        const float nh = dot3c(n, h);
+        if (nh <= 0.f) return 0.f;
+        return m.albedo * ggx_Dc(nh, m.alpha) * ggx_G1c(ci, m.alpha) * ggx_G1c(co, m.alpha) / (4.0f * ci * co);
+    }
+    return 0.f;
+}
+static __device__ __forceinline__ float3 cross3c(float3 a, float3 b) {
+    return f3(__fmaf_rn(a.y, b.z, -__fmul_rn(a.z, b.y)), __fmaf_rn(a.z, b.x, -__fmul_rn(a.x, b.z)), __fmaf_rn(a.x, b.y, -__fmul_rn(a.y, b.x)));
+}
+// t u + b v + n w
+static __device__ __forceinline__ float3 combine3c(float3 t, float u, float3 b, float v, float3 n, float w) {
+    return f3(__fmaf_rn(n.x, w, __fmaf_rn(t.x, u, __fmul_rn(b.x, v))), __fmaf_rn(n.y, w, __fmaf_rn(t.y, u, __fmul_rn(b.y, v))),
+              __fmaf_rn(n.z, w, __fmaf_rn(t.z, u, __fmul_rn(b.z, v))));
+}
+// h k - w
+static __device__ __forceinline__ float3 reflect3c(float3 h, float k, float3 w) {
+    return f3(__fmaf_rn(h.x, k, -w.x), __fmaf_rn(h.y, k, -w.y), __fmaf_rn(h.z, k, -w.z));
+}
+static __device__ __forceinline__ float bsdf_pdfc(const Mat& m, float3 n, float3 wi, float3 wo) {
+    float ci = dot3c(n, wi), co = dot3c(n, wo);
+    if (ci * co <= 0.f) return 0.f;
+    if (ci < 0.f) { co = -co; n = n * -1.0f; }
+    if (m.type == M_LAMBERT) return co / kPi;
+    if (m.type == M_GGX) {
+        const float3 h = norm3c(sum3c(wi, wo));
+        const float nh = dot3c(n, h), oh = dot3c(wo, h);
+        if (nh <= 0.f || oh <= 0.f) return 0.f;
+        return ggx_Dc(nh, m.alpha) * nh / (4.0f * oh);
+    }
+    return 0.f;
+}
+static __device__ __forceinline__ bool bsdf_samplec(const Mat& m, float3 n, float3 wi, float u0, float u1, float3& wo, float& pdf, float& thr,
+                                                    bool& delta) {
+    if (dot3c(n, wi) < 0.f) n = n * -1.0f;
+    delta = false;
+    if (m.type == M_MIRROR) {
+        wo = reflect3c(n, 2.0f * dot3c(wi, n), wi);
+        pdf = 1.0f; thr = m.albedo; delta = true;
+        return true;
+    }
+    const float3 a1 = f3(0.4140355211239282f, 0.731736150464251f, 0.5414210869105452f);
+    const float3 a2 = f3(0.0f, 0.5947978113475719f, -0.8038753408434284f);
+    const float3 t = norm3c(cross3c(fabsf(dot3c(n, a1)) < 0.6f ? a1 : a2, n)), b = cross3c(n, t);
+    if (m.type == M_LAMBERT) {
+        float r = sqrtf(u0), ph = 2.0f * kPi * u1;
+        float lz = sqrtf(fmaxf(0.f, 1.0f - u0));
+        float s, c;
+        sincosf(ph, &s, &c);
+        wo = combine3c(t, __fmul_rn(r, c), b, __fmul_rn(r, s), n, lz);
+    } else {
+        float a = m.alpha;
+        float tan2 = __fmul_rn(__fmul_rn(a, a), u0) / (1.0f - u0);
+        float ct = 1.0f / sqrtf(__fadd_rn(1.0f, tan2)), st = sqrtf(fmaxf(0.f, __fmaf_rn(-ct, ct, 1.0f))), ph = 2.0f * kPi * u1;
+        float s, c;
+        sincosf(ph, &s, &c);
+        float3 h = combine3c(t, __fmul_rn(st, c), b, __fmul_rn(st, s), n, ct);
+        wo = reflect3c(h, 2.0f * dot3c(wi, h), wi);
+    }
+    float co = dot3c(n, wo);
+    if (co <= 0.f) return false;
+    pdf = bsdf_pdfc(m, n, wi, wo);
+    float f = bsdf_fc(m, n, wi, wo);
+    if (!(pdf > 0.f) || !(f > 0.f)) return false;
+    thr = f * co / pdf;
+    return true;
+}
+static __device__ __forceinline__ Surf surf_atc(const GeomDev& g, int tri, float b1, float b2) {
+    const float4 a = __ldg(&g.tri[3 * tri]), e1 = __ldg(&g.tri[3 * tri + 1]), e2 = __ldg(&g.tri[3 * tri + 2]);
+    Surf s;
+    s.tri = tri; s.b1 = b1; s.b2 = b2;
+    s.p = xyz(a) + f3(__fmaf_rn(e1.x, b1, __fmul_rn(e2.x, b2)), __fmaf_rn(e1.y, b1, __fmul_rn(e2.y, b2)), __fmaf_rn(e1.z, b1, __fmul_rn(e2.z, b2)));
+    s.n = norm3c(cross3c(xyz(e1), xyz(e2)));
+    s.mat = __float_as_int(a.w);
+    return s;
+}
+static __device__ __forceinline__ float light_termc(const Domain& D, float3 xp, float3 xn, float3& wl, float& seg) {
+    const LightDev& L = D.light;
+    float I = 0.f;
+    if (L.kind == 1) I = L.I;
+    else if (L.kind == 2) {
+        const float3 w = dir_toc(L.pos, xp);
+        I = L.I * bsdf_fc(load_mat(D.F->g, D.spot_mat), D.spot_n, L.to_origin, w) * fabsf(dot3c(D.spot_n, w));
+    }
+    const float3 dd = L.pos - xp;
+    const float dist = len3c(dd);
+    if (!(dist > 0.f) || !(I > 0.f)) return 0.f;
+    wl = scale3c(dd, 1.0f / dist);
+    seg = dist + (L.kind == 2 ? L.emit_len : 0.f);
+    return I * fabsf(dot3c(xn, wl)) / __fmul_rn(dist, dist);
+}
+
+// ============================================================================================
 // path-length derivatives (Sec. 4.3 "Gradient and Hessian Evaluation"):
 //   L(p) = |p1 - p| + |p2 - p|, grad_p L = -(d1 + d2), hess_p L = A = sum (I - d d^T)/|p_i - p|,
 //   grad_xi L = J^T grad_p L, hess_xi L = J^T A J (Q = 0 on flat triangles)
@@ -888,27 +1034,31 @@ static __device__ __forceinline__ Frame2 tri_frame(const GeomDev& g, int tri) {
     float4 a = __ldg(&g.tri[3 * tri]), e1 = __ldg(&g.tri[3 * tri + 1]), e2 = __ldg(&g.tri[3 * tri + 2]);
     Frame2 f;
     f.o = xyz(a);
-    f.t = norm3(xyz(e1));
-    float3 n = norm3(cross3(xyz(e1), xyz(e2)));
-    f.b = cross3(n, f.t);
+    f.t = norm3c(xyz(e1));
+    float3 n = norm3c(cross3c(xyz(e1), xyz(e2)));
+    f.b = cross3c(n, f.t);
     return f;
 }
-static __device__ __forceinline__ float3 frame_point(const Frame2& f, float x0, float x1) { return f.o + (f.t * x0 + f.b * x1); }
+static __device__ __forceinline__ float3 frame_point(const Frame2& f, float x0, float x1) {
+    return f.o + f3(__fmaf_rn(f.t.x, x0, __fmul_rn(f.b.x, x1)), __fmaf_rn(f.t.y, x0, __fmul_rn(f.b.y, x1)),
+                    __fmaf_rn(f.t.z, x0, __fmul_rn(f.b.z, x1)));
+}
 
 static __device__ __forceinline__ void length_derivs(float3 p1, float3 p2, const Frame2& f, float x0, float x1, float& L,
                                               float g[2], float h[3]) {
     float3 p = frame_point(f, x0, x1);
     float3 a1 = p1 - p, a2 = p2 - p;
-    float l1 = len3(a1), l2 = len3(a2);
-    float3 d1 = a1 * (1.0f / l1), d2 = a2 * (1.0f / l2);
-    float3 s = d1 + d2;
+    float l1 = len3c(a1), l2 = len3c(a2);
+    const float i1 = 1.0f / l1, i2 = 1.0f / l2;
+    float3 d1 = scale3c(a1, i1), d2 = scale3c(a2, i2);
+    float3 s = sum3c(d1, d2);
     L = l1 + l2;
-    g[0] = -dot3(f.t, s);
-    g[1] = -dot3(f.b, s);
-    float d1t = dot3(d1, f.t), d1b = dot3(d1, f.b), d2t = dot3(d2, f.t), d2b = dot3(d2, f.b);
-    h[0] = (1.0f - d1t * d1t) / l1 + (1.0f - d2t * d2t) / l2;
-    h[1] = (-d1t * d1b) / l1 + (-d2t * d2b) / l2;
-    h[2] = (1.0f - d1b * d1b) / l1 + (1.0f - d2b * d2b) / l2;
+    g[0] = -dot3c(f.t, s);
+    g[1] = -dot3c(f.b, s);
+    float d1t = dot3c(d1, f.t), d1b = dot3c(d1, f.b), d2t = dot3c(d2, f.t), d2b = dot3c(d2, f.b);
+    h[0] = __fadd_rn(div_by(__fmaf_rn(-d1t, d1t, 1.0f), l1, i1), div_by(__fmaf_rn(-d2t, d2t, 1.0f), l2, i2));
+    h[1] = __fadd_rn(div_by(__fmul_rn(-d1t, d1b), l1, i1), div_by(__fmul_rn(-d2t, d2b), l2, i2));
+    h[2] = __fadd_rn(div_by(__fmaf_rn(-d1b, d1b, 1.0f), l1, i1), div_by(__fmaf_rn(-d2b, d2b, 1.0f), l2, i2));
 }
 
 // gauge of the Newton system: the paper's average gradient, or a comparison gauge of Sec. 4.3
@@ -921,21 +1071,15 @@ struct NewtonGeo { float3 p1x, p2x; Frame2 fx; float3 p1y, p2y; Frame2 fy; int g
 
 // F(xi, xi') = [L_y(xi') - L_x(xi) - delta ; (R m)^T (xi' - xi)], m = (grad L_x(xi) + grad L_y(xi'))/2,
 // R = 90-degree rotation; each gradient on its own path (Sec. 4.3, average-gradient gauge)
-static __device__ __forceinline__ void newton_F_f(const NewtonGeo& N, const Frame2& fy, const float xi[2], float Lx, const float gx[2],
-                                           float delta, const float xp[2], float F[2], float gy[2], float hy[3], float m[2]) {
-    float Ly;
-    length_derivs(N.p1y, N.p2y, fy, xp[0], xp[1], Ly, gy, hy);
-    m[0] = 0.5f * (gx[0] + gy[0]);
-    m[1] = 0.5f * (gx[1] + gy[1]);
+static __device__ __forceinline__ void newton_F(int gauge, const float xi[2], float Lx, const float gx[2], float delta, const float xp[2],
+                                                float Ly, const float gy[2], float F[2], float m[2]) {
+    m[0] = __fmul_rn(0.5f, __fadd_rn(gx[0], gy[0]));
+    m[1] = __fmul_rn(0.5f, __fadd_rn(gx[1], gy[1]));
     F[0] = Ly - Lx - delta;
-    if (N.gauge == G_AVERAGE) F[1] = -m[1] * (xp[0] - xi[0]) + m[0] * (xp[1] - xi[1]);
-    else if (N.gauge == G_AXIS_T) F[1] = xp[1] - xi[1];
-    else if (N.gauge == G_AXIS_B) F[1] = xp[0] - xi[0];
-    else F[1] = -gx[1] * (xp[0] - xi[0]) + gx[0] * (xp[1] - xi[1]);
-}
-static __device__ __forceinline__ void newton_F(const NewtonGeo& N, const float xi[2], float Lx, const float gx[2], float delta,
-                                         const float xp[2], float F[2], float gy[2], float hy[3], float m[2]) {
-    newton_F_f(N, N.fy, xi, Lx, gx, delta, xp, F, gy, hy, m);
+    if (gauge == G_AVERAGE) F[1] = det2c(m[0], xp[1] - xi[1], m[1], xp[0] - xi[0]);
+    else if (gauge == G_AXIS_T) F[1] = xp[1] - xi[1];
+    else if (gauge == G_AXIS_B) F[1] = xp[0] - xi[0];
+    else F[1] = __fmaf_rn(-gx[1], xp[0] - xi[0], __fmul_rn(gx[0], xp[1] - xi[1]));
 }
 // dF/dxi' rows: (grad L_y(xi'), R m - 0.5 H_y R (xi' - xi)); dF/dxi rows: (-grad L_x(xi), -(R m + 0.5 H_x R (xi' - xi)))
 // comparison gauges: fixed axis rows (0, 1) / (1, 0); start gradient dF2/dxi' = R g_x,
@@ -944,14 +1088,14 @@ static __device__ __forceinline__ void newton_J(int gauge, const float xi[2], co
                                          const float gy[2], const float hy[3], const float m[2], float A[4], float Bm[4]) {
     float Rm0 = -m[1], Rm1 = m[0];
     float dd0 = xp[0] - xi[0], dd1 = xp[1] - xi[1];
-    float Rd0 = -dd1, Rd1 = dd0;
-    float HyRd0 = hy[0] * Rd0 + hy[1] * Rd1, HyRd1 = hy[1] * Rd0 + hy[2] * Rd1;
-    float HxRd0 = hx[0] * Rd0 + hx[1] * Rd1, HxRd1 = hx[1] * Rd0 + hx[2] * Rd1;
+    // H R (xi' - xi), R (xi' - xi) = (-dd1, dd0)
+    float HyRd0 = det2c(hy[1], dd0, hy[0], dd1), HyRd1 = det2c(hy[2], dd0, hy[1], dd1);
+    float HxRd0 = det2c(hx[1], dd0, hx[0], dd1), HxRd1 = det2c(hx[2], dd0, hx[1], dd1);
     A[0] = gy[0]; A[1] = gy[1];
     Bm[0] = -gx[0]; Bm[1] = -gx[1];
     if (gauge == G_AVERAGE) {
-        A[2] = Rm0 - 0.5f * HyRd0; A[3] = Rm1 - 0.5f * HyRd1;
-        Bm[2] = -(Rm0 + 0.5f * HxRd0); Bm[3] = -(Rm1 + 0.5f * HxRd1);
+        A[2] = __fmaf_rn(-0.5f, HyRd0, Rm0); A[3] = __fmaf_rn(-0.5f, HyRd1, Rm1);
+        Bm[2] = -__fmaf_rn(0.5f, HxRd0, Rm0); Bm[3] = -__fmaf_rn(0.5f, HxRd1, Rm1);
     } else if (gauge == G_AXIS_T) {
         A[2] = 0.f; A[3] = 1.f; Bm[2] = 0.f; Bm[3] = -1.f;
     } else if (gauge == G_AXIS_B) {
@@ -962,29 +1106,58 @@ static __device__ __forceinline__ void newton_J(int gauge, const float xi[2], co
     }
 }
 
-// Newton iteration with backtracking (Sec. 4.3); returns success, xi', |det(dxi'/dxi)| and the
-// iteration count.  Stops at |F|_inf <= tol_stop (after one polishing step there) or after
-// max_iter (up to 2 max_iter while |F|_inf <= tol_succ, the paper's 1 %-of-the-gate band);
-// success if converged, |F|_inf <= tol_stop.
-static __device__ bool newton_solve(const NewtonGeo& N, const float xi[2], float delta, int max_iter, float tol_stop,
-                             float tol_succ, float xp[2], float& jdet, int& iters) {
-    float Lx, gx[2], hx[3];
-    length_derivs(N.p1x, N.p2x, N.fx, xi[0], xi[1], Lx, gx, hx);
-    xp[0] = xi[0]; xp[1] = xi[1];
-    float F[2], gy[2], hy[3], m[2];
-    newton_F(N, xi, Lx, gx, delta, xp, F, gy, hy, m);
-    int it = 0;
-    bool polished = false;
-    // loops kept rolled: the unrolled copies of the line search cost more in instruction-cache misses
-    // than they save (4.9 against 5.1 ms per 512 x 512 frame)
-    // the paper's budget is max_iter iterations; a solve that spends it inside the success band
-    // (|F| <= tol_succ) short of convergence continues toward the root, at most max_iter more, so
-    // that an accepted shift is the root F = 0 and not a point of the band that depends on rounding
+// Newton iteration with backtracking (Sec. 4.3) from xp on the plane of frame fy; leaves the last accepted
+// point in xp, |F|_inf there in nF, and the determinants of dF/dxi' and dF/dxi there.  Stops at
+// |F|_inf <= tol_stop (after one polishing step there) or after max_iter (up to 2 max_iter while
+// |F|_inf <= tol_succ, the paper's 1 %-of-the-gate band).
+// One flat loop over evaluations of the path length's derivatives -- the base path's (has_base: taken
+// already), the starting point's, then each candidate's, a backtracked one among them -- so that they share
+// one copy of that code (the kernels wait on instruction fetch more than on anything else), a warp's lanes
+// meet in it whatever step they are at, and only the point, the step and two determinants live across it.
+struct NewtonBase { float L, g[2], h[3]; };
+static __device__ __forceinline__ int newton_core(const NewtonGeo& N, const Frame2& fy, const float xi[2], NewtonBase& B, bool has_base,
+                                                  float delta, int max_iter, float tol_stop, float tol_succ, float xp[2], float& nF,
+                                                  float& dA, float& dB) {
+    int it = 0, ls = 0;
+    int phase = has_base ? 1 : 0;   // 0 the base path, 1 the starting point, 2 a candidate
+    bool polish = false, polished = false;
+    float c0 = has_base ? xp[0] : xi[0], c1 = has_base ? xp[1] : xi[1];
+    float s0 = 0.f, s1 = 0.f, lam = 1.0f;
+    nF = 0.f; dA = 0.f; dB = 0.f;
 #pragma unroll 1
-    while (it < 2 * max_iter) {
-        float nF = fmaxf(fabsf(F[0]), fabsf(F[1]));
-        if (it >= max_iter && !(nF <= tol_succ)) break;
-        bool polish = false;
+    while (true) {
+        const bool base = phase == 0;
+        float L, g[2], h[3];
+        length_derivs(base ? N.p1x : N.p1y, base ? N.p2x : N.p2y, base ? N.fx : fy, c0, c1, L, g, h);
+        if (base) {
+            B.L = L; B.g[0] = g[0]; B.g[1] = g[1]; B.h[0] = h[0]; B.h[1] = h[1]; B.h[2] = h[2];
+            c0 = xp[0]; c1 = xp[1];
+            phase = 1;
+            continue;
+        }
+        const float c[2] = {c0, c1};
+        float F[2], m[2];
+        newton_F(N.gauge, xi, B.L, B.g, delta, c, L, g, F, m);
+        const float n = fmaxf(fabsf(F[0]), fabsf(F[1]));
+        if (phase == 2 && !(polish ? n <= nF : n < nF)) {
+            if (polish || ++ls == 5) break;
+            lam *= 0.5f;
+            c0 = __fmaf_rn(lam, s0, xp[0]); c1 = __fmaf_rn(lam, s1, xp[1]);
+            continue;
+        }
+        if (phase == 2 && !polish) ++it;
+        phase = 2;
+        xp[0] = c0; xp[1] = c1;
+        nF = n;
+        float A[4], Bm[4];
+        newton_J(N.gauge, xi, xp, B.g, B.h, g, h, m, A, Bm);
+        dA = det2c(A[0], A[3], A[1], A[2]);
+        dB = det2c(Bm[0], Bm[3], Bm[1], Bm[2]);
+        // the paper's budget is max_iter iterations; a solve that spends it inside the success band
+        // (|F| <= tol_succ) short of convergence continues toward the root, at most max_iter more, so
+        // that an accepted shift is the root F = 0 and not a point of the band that depends on rounding
+        if (it >= 2 * max_iter || (it >= max_iter && !(nF <= tol_succ))) break;
+        polish = false;
         if (nF <= tol_stop) {
             // converged: one more full Newton step at the root, kept if |F| does not grow, so that the
             // result is the root itself (to FP32 rounding) and not the first iterate under the
@@ -992,42 +1165,33 @@ static __device__ bool newton_solve(const NewtonGeo& N, const float xi[2], float
             if (polished || !(nF > 0.f)) break;
             polish = polished = true;
         }
-        float A[4], Bm[4];
-        newton_J(N.gauge, xi, xp, gx, hx, gy, hy, m, A, Bm);
-        float det = A[0] * A[3] - A[1] * A[2];
-        if (!(fabsf(det) > 1e-30f)) break;
-        float s0 = -(A[3] * F[0] - A[1] * F[1]) / det, s1 = -(-A[2] * F[0] + A[0] * F[1]) / det;
-        float lam = 1.0f;
-        bool accepted = false;
-#pragma unroll 1
-        for (int ls = 0; ls < (polish ? 1 : 5); ++ls) {
-            float c[2] = {xp[0] + lam * s0, xp[1] + lam * s1};
-            float Fc[2], gyc[2], hyc[3], mc[2];
-            newton_F(N, xi, Lx, gx, delta, c, Fc, gyc, hyc, mc);
-            if (polish ? fmaxf(fabsf(Fc[0]), fabsf(Fc[1])) <= nF : fmaxf(fabsf(Fc[0]), fabsf(Fc[1])) < nF) {
-                xp[0] = c[0]; xp[1] = c[1];
-                F[0] = Fc[0]; F[1] = Fc[1];
-                gy[0] = gyc[0]; gy[1] = gyc[1]; hy[0] = hyc[0]; hy[1] = hyc[1]; hy[2] = hyc[2];
-                m[0] = mc[0]; m[1] = mc[1];
-                accepted = true;
-                break;
-            }
-            lam *= 0.5f;
-        }
-        if (!accepted) break;
-        if (!polish) ++it;
+        if (!(fabsf(dA) > 1e-30f)) break;
+        const float rd = 1.0f / dA;
+        s0 = div_by(-det2c(A[3], F[0], A[1], F[1]), dA, rd);
+        s1 = div_by(-det2c(A[0], F[1], A[2], F[0]), dA, rd);
+        lam = 1.0f;
+        ls = 0;
+        c0 = __fmaf_rn(lam, s0, xp[0]); c1 = __fmaf_rn(lam, s1, xp[1]);
     }
-    iters = it;
-    // success: converged (|F| <= tol_stop), so that the shift satisfies its constraint and stays
-    // invertible; a solve stalled inside the band (ill-conditioned: L nearly stationary at the
-    // vertex) is rejected, in FP32 as in FP64, instead of ending at a rounding-dependent point
-    if (!(fmaxf(fabsf(F[0]), fabsf(F[1])) <= tol_stop)) return false;
-    float A[4], Bm[4];
-    newton_J(N.gauge, xi, xp, gx, hx, gy, hy, m, A, Bm);
-    float dA = A[0] * A[3] - A[1] * A[2], dB = Bm[0] * Bm[3] - Bm[1] * Bm[2];
-    if (!(fabsf(dA) > 0.f)) return false;
+    return it;
+}
+
+// xi', |det(dxi'/dxi)| and the iteration count; success: converged (|F| <= tol_stop), so that the shift
+// satisfies its constraint and stays invertible; a solve stalled inside the band (ill-conditioned: L
+// nearly stationary at the vertex) is rejected, in FP32 as in FP64, instead of ending at a
+// rounding-dependent point
+static __device__ __forceinline__ bool newton_end(float nF, float tol_stop, float dA, float dB, float& jdet) {
+    if (!(nF <= tol_stop) || !(fabsf(dA) > 0.f)) return false;
     jdet = fabsf(dB / dA);
     return isfinite(jdet);
+}
+static __device__ __forceinline__ bool newton_solve(const NewtonGeo& N, const float xi[2], float delta, int max_iter, float tol_stop,
+                                                    float tol_succ, float xp[2], float& jdet, int& iters) {
+    NewtonBase B;
+    float nF, dA, dB;
+    xp[0] = xi[0]; xp[1] = xi[1];
+    iters = newton_core(N, N.fy, xi, B, false, delta, max_iter, tol_stop, tol_succ, xp, nF, dA, dB);
+    return newton_end(nF, tol_stop, dA, dB, jdet);
 }
 
 // ============================================================================================
@@ -1128,63 +1292,20 @@ static __device__ bool walk_locate(const GeomDev& g, Walk& W, const float from_i
 // cost what they cost without the walk.
 static __device__ bool newton_solve_walk(const GeomDev& gi, const NewtonGeo& N, Walk& W, const float xi[2], float delta,
                                          int max_iter, float tol_stop, float tol_succ, float xp[2], float& jdet, int& iters) {
-    float Lx, gx[2], hx[3];
-    length_derivs(N.p1x, N.p2x, N.fx, xi[0], xi[1], Lx, gx, hx);
+    NewtonBase B;
     xp[0] = xi[0]; xp[1] = xi[1];
     float start[2] = {xi[0], xi[1]};
-    float F[2], gy[2], hy[3], m[2];
     int total = 0;
 #pragma unroll 1
     for (int cross = 0;; ++cross) {
-        newton_F_f(N, W.f, xi, Lx, gx, delta, xp, F, gy, hy, m);
-        int it = 0;
-        bool polished = false;
-#pragma unroll 1
-        while (it < 2 * max_iter) {   // budget as in newton_solve
-            float nF = fmaxf(fabsf(F[0]), fabsf(F[1]));
-            if (it >= max_iter && !(nF <= tol_succ)) break;
-            bool polish = false;
-            if (nF <= tol_stop) {   // converged: one polishing step, as in newton_solve
-                if (polished || !(nF > 0.f)) break;
-                polish = polished = true;
-            }
-            float A[4], Bm[4];
-            newton_J(N.gauge, xi, xp, gx, hx, gy, hy, m, A, Bm);
-            float det = A[0] * A[3] - A[1] * A[2];
-            if (!(fabsf(det) > 1e-30f)) break;
-            float s0 = -(A[3] * F[0] - A[1] * F[1]) / det, s1 = -(-A[2] * F[0] + A[0] * F[1]) / det;
-            float lam = 1.0f;
-            bool accepted = false;
-#pragma unroll 1
-            for (int ls = 0; ls < (polish ? 1 : 5); ++ls) {
-                float c[2] = {xp[0] + lam * s0, xp[1] + lam * s1};
-                float Fc[2], gyc[2], hyc[3], mc[2];
-                newton_F_f(N, W.f, xi, Lx, gx, delta, c, Fc, gyc, hyc, mc);
-                if (polish ? fmaxf(fabsf(Fc[0]), fabsf(Fc[1])) <= nF : fmaxf(fabsf(Fc[0]), fabsf(Fc[1])) < nF) {
-                    xp[0] = c[0]; xp[1] = c[1];
-                    F[0] = Fc[0]; F[1] = Fc[1];
-                    gy[0] = gyc[0]; gy[1] = gyc[1]; hy[0] = hyc[0]; hy[1] = hyc[1]; hy[2] = hyc[2];
-                    m[0] = mc[0]; m[1] = mc[1];
-                    accepted = true;
-                    break;
-                }
-                lam *= 0.5f;
-            }
-            if (!accepted) break;
-            if (!polish) ++it;
-        }
-        total += it;
-        if (!(fmaxf(fabsf(F[0]), fabsf(F[1])) <= tol_stop)) break;   // converged, as in newton_solve
+        float nF, dA, dB;
+        total += newton_core(N, W.f, xi, B, cross > 0, delta, max_iter, tol_stop, tol_succ, xp, nF, dA, dB);
+        if (!(nF <= tol_stop)) break;   // converged, as in newton_end
         float lm[3];
         walk_bary(gi, W, xp[0], xp[1], lm);
         if (lm[0] >= -kBaryEps && lm[1] >= -kBaryEps && lm[2] >= -kBaryEps) {
             iters = total;
-            float A[4], Bm[4];
-            newton_J(N.gauge, xi, xp, gx, hx, gy, hy, m, A, Bm);
-            float dA = A[0] * A[3] - A[1] * A[2], dB = Bm[0] * Bm[3] - Bm[1] * Bm[2];
-            if (!(fabsf(dA) > 0.f)) return false;
-            jdet = fabsf(dB / dA);
-            return isfinite(jdet);
+            return newton_end(nF, tol_stop, dA, dB, jdet);
         }
         if (cross == kMaxCross) break;
         // the plane's solution lies outside the triangle: walk there and solve again
@@ -1489,55 +1610,55 @@ static __device__ bool shift_rec(const Rec& x, const Domain& Dj, const Domain& D
     // (1) random replay with the base path's random numbers
     Surf yv[kMaxDepth];
     yv[1] = Di.y1;
-    float plen = len3(Di.x0 - yv[1].p);
+    float plen = len3c(Di.x0 - yv[1].p);
     float fpre = 1.0f, pdfy = 1.0f;
     for (int j = 1; j <= r - 2; ++j) {
         uint4 u = philox(x.key_px, x.key_frame, ((uint32_t)tree << 8) | (uint32_t)j, P_BSDF, P.seed);
-        float3 wi = dir_to(yv[j].p, j == 1 ? Di.x0 : yv[j - 1].p);
+        float3 wi = dir_toc(yv[j].p, j == 1 ? Di.x0 : yv[j - 1].p);
         Mat m = load_mat(gi, yv[j].mat);
         if (mat_class(m) != rec_cls(x, j)) return false;
         float3 wo; float pdf, thr; bool delta;
-        if (!bsdf_sample(m, yv[j].n, wi, u01(u.x), u01(u.y), wo, pdf, thr, delta)) return false;
+        if (!bsdf_samplec(m, yv[j].n, wi, u01(u.x), u01(u.y), wo, pdf, thr, delta)) return false;
         if (!trace_from(gi, yv[j], wo, eps, yv[j + 1])) return false;
-        float seg = len3(yv[j + 1].p - yv[j].p);
+        float seg = len3c(yv[j + 1].p - yv[j].p);
         plen += seg;
         if (delta) fpre *= m.albedo;
         else {
-            fpre *= bsdf_f(m, yv[j].n, wi, wo) * Gterm(yv[j], yv[j + 1]);
-            pdfy *= pdf * fabsf(dot3(yv[j + 1].n, wo)) / (seg * seg);
+            fpre *= bsdf_fc<true>(m, yv[j].n, wi, wo) * Gtermc(yv[j].p, yv[j].n, yv[j + 1].p, yv[j + 1].n);
+            pdfy *= pdf * fabsf(dot3c(yv[j + 1].n, wo)) / __fmul_rn(seg, seg);
         }
     }
     if (mat_class(load_mat(gi, yv[r - 1].mat)) != rec_cls(x, r - 1)) return false;
 
     // (2) suffix and light in the target domain
     Surf sv[3];
-    for (int q = 0; q < ns; ++q) sv[q] = surf_at(gi, x.s_tri[q], x.s_b1[q], x.s_b2[q]);
+    for (int q = 0; q < ns; ++q) sv[q] = surf_atc(gi, x.s_tri[q], x.s_b1[q], x.s_b2[q]);
     if (Di.light.kind == 0) return false;
     float3 lpos_i = Di.light.pos;
     float emit_i = Di.light.kind == 2 ? Di.light.emit_len : 0.f;
     float slen = 0.f;
-    for (int q = 0; q + 1 < ns; ++q) slen += len3(sv[q].p - sv[q + 1].p);
-    if (ns > 0) slen += len3(sv[ns - 1].p - lpos_i) + emit_i;
+    for (int q = 0; q + 1 < ns; ++q) slen += len3c(sv[q].p - sv[q + 1].p);
+    if (ns > 0) slen += len3c(sv[ns - 1].p - lpos_i) + emit_i;
     else slen += emit_i;
     float3 p2y = ns > 0 ? sv[0].p : lpos_i;
 
     // (3) base-path quantities in the record's own frame
     NewtonGeo N;
     N.fx = tri_frame(gj, x.p_tri);
-    Surf pbase = surf_at(gj, x.p_tri, x.p_b1, x.p_b2);
-    float3 p2x = ns > 0 ? surf_at(gj, x.s_tri[0], x.s_b1[0], x.s_b2[0]).p : Dj.light.pos;
+    Surf pbase = surf_atc(gj, x.p_tri, x.p_b1, x.p_b2);
+    float3 p2x = ns > 0 ? surf_atc(gj, x.s_tri[0], x.s_b1[0], x.s_b2[0]).p : Dj.light.pos;
     float xi[2];
     {
         float3 dd = pbase.p - N.fx.o;
-        xi[0] = dot3(dd, N.fx.t);
-        xi[1] = dot3(dd, N.fx.b);
+        xi[0] = dot3c(dd, N.fx.t);
+        xi[1] = dot3c(dd, N.fx.b);
     }
     N.p1x = x.xprev; N.p2x = p2x; N.gauge = gauge_of(P.flags);
     N.p1y = yv[r - 1].p; N.p2y = p2y; N.fy = tri_frame(gi, x.p_tri);
 
     // (4) Newton solve of L(y') = L(x) + delta (eq. path_length_constraint), delta keeping the
     // sample at the same position inside the target gate
-    float Lx_seg = len3(x.xprev - pbase.p) + len3(p2x - pbase.p);
+    float Lx_seg = len3c(x.xprev - pbase.p) + len3c(p2x - pbase.p);
     float tau_t = 0.f;   // target gated length under a gate map
     float ell;
     if (gm) {
@@ -1574,12 +1695,12 @@ static __device__ bool shift_rec(const Rec& x, const Domain& Dj, const Domain& D
         float4 a = __ldg(&gi.tri[3 * x.p_tri]), e1v = __ldg(&gi.tri[3 * x.p_tri + 1]), e2v = __ldg(&gi.tri[3 * x.p_tri + 2]);
         (void)a;
         float3 e1 = xyz(e1v), e2 = xyz(e2v);
-        float e1t = dot3(e1, N.fy.t), e2t = dot3(e2, N.fy.t), e2b = dot3(e2, N.fy.b);
+        float e1t = dot3c(e1, N.fy.t), e2t = dot3c(e2, N.fy.t), e2b = dot3c(e2, N.fy.b);
         nb2 = xp[1] / e2b;
-        nb1 = (xp[0] - nb2 * e2t) / e1t;
+        nb1 = __fmaf_rn(-nb2, e2t, xp[0]) / e1t;
     }
     if (!(nb1 >= -kBaryEps && nb2 >= -kBaryEps && nb1 + nb2 <= 1.0f + kBaryEps)) return false;
-    Surf pp = surf_at(gi, ptri, nb1, nb2);
+    Surf pp = surf_atc(gi, ptri, nb1, nb2);
 
     // (5) the offset path must reconnect at the same index
     {
@@ -1593,23 +1714,23 @@ static __device__ bool shift_rec(const Rec& x, const Domain& Dj, const Domain& D
 
     // (6) target function in Di without the suffix radiance, the gate and the Jacobian: cheap
     // rejections, taken before any ray is traced (the result is the same in either order)
-    float3 wprev = dir_to(yv[r - 1].p, r - 1 == 1 ? Di.x0 : yv[r - 2].p);
+    float3 wprev = dir_toc(yv[r - 1].p, r - 1 == 1 ? Di.x0 : yv[r - 2].p);
     float f = fpre;
-    f *= bsdf_f(load_mat(gi, yv[r - 1].mat), yv[r - 1].n, wprev, dir_to(yv[r - 1].p, pp.p));
-    f *= Gterm(yv[r - 1], pp);
+    f *= bsdf_fc(load_mat(gi, yv[r - 1].mat), yv[r - 1].n, wprev, dir_toc(yv[r - 1].p, pp.p));
+    f *= Gtermc(yv[r - 1].p, yv[r - 1].n, pp.p, pp.n);
     Mat mp = load_mat(gi, pp.mat);
     if (ns == 0) {
         float3 wl; float seg;
-        float lt = light_term(Di, pp, wl, seg);
-        f *= bsdf_f(mp, pp.n, dir_to(pp.p, yv[r - 1].p), wl) * lt;
+        float lt = light_termc(Di, pp.p, pp.n, wl, seg);
+        f *= bsdf_fc(mp, pp.n, dir_toc(pp.p, yv[r - 1].p), wl) * lt;
     } else {
-        f *= bsdf_f(mp, pp.n, dir_to(pp.p, yv[r - 1].p), dir_to(pp.p, sv[0].p));
-        f *= Gterm(pp, sv[0]);
-        float3 wnext = ns > 1 ? dir_to(sv[0].p, sv[1].p) : dir_to(sv[0].p, lpos_i);
-        f *= bsdf_f(load_mat(gi, sv[0].mat), sv[0].n, dir_to(sv[0].p, pp.p), wnext);
+        f *= bsdf_fc(mp, pp.n, dir_toc(pp.p, yv[r - 1].p), dir_toc(pp.p, sv[0].p));
+        f *= Gtermc(pp.p, pp.n, sv[0].p, sv[0].n);
+        float3 wnext = ns > 1 ? dir_toc(sv[0].p, sv[1].p) : dir_toc(sv[0].p, lpos_i);
+        f *= bsdf_fc(load_mat(gi, sv[0].mat), sv[0].n, dir_toc(sv[0].p, pp.p), wnext);
     }
     if (!(f > 0.f) || !isfinite(f)) return false;
-    float Lnew = plen + len3(yv[r - 1].p - pp.p) + len3(pp.p - p2y) + slen;
+    float Lnew = plen + len3c(yv[r - 1].p - pp.p) + len3c(pp.p - p2y) + slen;
     float tau = Lnew - Di.o;
     if (gm) {
         if (!(tau >= gm->lo && tau < gm->hi)) return false;
@@ -1629,17 +1750,17 @@ static __device__ bool shift_rec(const Rec& x, const Domain& Dj, const Domain& D
             float Ls = 1.0f;
             for (int q = 1; q < ns; ++q) {
                 Mat mq = load_mat(gi, sv[q].mat);
-                float gg = mat_class(load_mat(gi, sv[q - 1].mat)) == C_DELTA ? 1.0f : Gterm(sv[q - 1], sv[q]);
+                float gg = mat_class(load_mat(gi, sv[q - 1].mat)) == C_DELTA ? 1.0f : Gtermc(sv[q - 1].p, sv[q - 1].n, sv[q].p, sv[q].n);
                 if (mat_class(mq) == C_DELTA) {
                     if (!geom_static) return false;
                     Ls *= gg * mq.albedo;
                 } else {
-                    float3 wn = q + 1 < ns ? dir_to(sv[q].p, sv[q + 1].p) : dir_to(sv[q].p, lpos_i);
-                    Ls *= gg * bsdf_f(mq, sv[q].n, dir_to(sv[q].p, sv[q - 1].p), wn);
+                    float3 wn = q + 1 < ns ? dir_toc(sv[q].p, sv[q + 1].p) : dir_toc(sv[q].p, lpos_i);
+                    Ls *= gg * bsdf_fc(mq, sv[q].n, dir_toc(sv[q].p, sv[q - 1].p), wn);
                 }
             }
             float3 wl; float seg;
-            Ls *= light_term(Di, sv[ns - 1], wl, seg);
+            Ls *= light_termc(Di, sv[ns - 1].p, sv[ns - 1].n, wl, seg);
             Lsuf_i = Ls;
         }
         f *= Lsuf_i;
@@ -1662,6 +1783,195 @@ static __device__ bool shift_rec(const Rec& x, const Domain& Dj, const Domain& D
         y.tau = tau;
         y.xprev = yv[r - 1].p;
         y.pdf_pre = pdfy;
+        y.p_tri = ptri; y.p_b1 = nb1; y.p_b2 = nb2;
+        y.Lsuf = Lsuf_i;
+        y.phat = f;
+    }
+    phat_out = f;
+    jac_out = jac;
+    if (st) st->shift_ok++;
+    return true;
+}
+
+
+// The shift of a record that reconnects at its second vertex (r = 2: 99 % of the tasks of the dynamic and
+// confocal workloads), for the persistent shift kernels: shift_rec's steps, expressions and order
+// with nothing to replay, so no arrays of vertices (local memory) and less code.  Fj / Fi: the frames of
+// the record's domain and of the target domain, gbj / gbi their primary hits, L0j / L0i their gates; kSame:
+// both frames are one (spatial reuse), so that the triangle's frame is built once.  The caller has tested
+// r = 2.  (Queueing both segments at once, with no in-place tracing here, and resolving the target's light
+// only after the solve was slower: 3.04 against 2.80 ms a 512 x 512 frame, for the code it added.)
+template <bool kOut, bool kWalk, bool kSame>
+static __device__ __forceinline__ bool shift_r2(const Rec& x, const FrameDev* Fj, float4 gbj, float L0j, const FrameDev* Fi, float4 gbi,
+                                                float L0i, const ParamsDev& P, bool geom_static, Rec& y, float& phat_out,
+                                                float& jac_out, ShiftStats* st, const VisQ* vq) {
+    const GeomDev& gi = Fi->g;
+    const GeomDev& gj = Fj->g;
+    const int ns = rec_ns(x);
+    const float eps = P.ray_eps;
+    if (__float_as_uint(gbi.x) == kNoHit || __float_as_uint(gbj.x) == kNoHit) return false;
+    if (st) st->shift_calls++;
+    const Domain Di = make_domain_hit(Fi, true, __float_as_int(gbi.x), gbi.y, gbi.z, gbi.w, L0i, Fi->dL);
+    const float plen = len3c(Di.x0 - Di.y1.p);
+    if (mat_class(load_mat(gi, Di.y1.mat)) != rec_cls(x, 1)) return false;
+    if (Di.light.kind == 0) return false;
+    const float3 lpos_i = Di.light.pos;
+
+    // suffix: the vertex after p, and the lengths behind it
+    float slen = 0.f;
+    Surf sv;
+    sv.tri = 0; sv.b1 = sv.b2 = 0.f; sv.p = sv.n = f3(0.f, 0.f, 0.f); sv.mat = 0;
+    if (ns > 0) {
+        sv = surf_atc(gi, x.s_tri[0], x.s_b1[0], x.s_b2[0]);
+        float3 last = sv.p;
+        if (ns > 1) {
+            float3 b = surf_atc(gi, x.s_tri[1], x.s_b1[1], x.s_b2[1]).p;
+            slen += len3c(last - b);
+            last = b;
+            if (ns > 2) {
+                b = surf_atc(gi, x.s_tri[2], x.s_b1[2], x.s_b2[2]).p;
+                slen += len3c(last - b);
+                last = b;
+            }
+        }
+        slen += len3c(last - lpos_i) + (Di.light.kind == 2 ? Di.light.emit_len : 0.f);
+    } else {
+        slen += Di.light.kind == 2 ? Di.light.emit_len : 0.f;
+    }
+    const float3 p2y = ns > 0 ? sv.p : lpos_i;
+
+    // base path
+    NewtonGeo N;
+    bool cache_ok = true;
+    {
+        const Domain Dj = make_domain_hit(Fj, true, __float_as_int(gbj.x), gbj.y, gbj.z, gbj.w, L0j, Fj->dL);
+        cache_ok = geom_static && light_same(Dj.light, Di.light);
+        N.p2x = ns > 0 ? (kSame ? sv.p : surf_atc(gj, x.s_tri[0], x.s_b1[0], x.s_b2[0]).p) : Dj.light.pos;
+    }
+    N.fx = tri_frame(gj, x.p_tri);
+    const float3 pbase = surf_atc(gj, x.p_tri, x.p_b1, x.p_b2).p;
+    float xi[2];
+    {
+        float3 dd = pbase - N.fx.o;
+        xi[0] = dot3c(dd, N.fx.t);
+        xi[1] = dot3c(dd, N.fx.b);
+    }
+    N.p1x = x.xprev; N.gauge = gauge_of(P.flags);
+    N.p1y = Di.y1.p; N.p2y = p2y;
+    if (kSame) N.fy = N.fx;
+    else N.fy = tri_frame(gi, x.p_tri);
+
+    float Lx_seg = len3c(x.xprev - pbase) + len3c(N.p2x - pbase);
+    float ell = x.tau - L0j + L0i + Di.o - plen - slen;
+    float delta = ell - Lx_seg;
+    float xp[2];
+    float jn = 1.0f;
+    const bool walk = kWalk && !(P.flags & 2u);
+    Walk W;
+    if (walk) walk_init(gi, x.p_tri, W);
+    if (P.flags & 2u) {
+        xp[0] = xi[0]; xp[1] = xi[1];
+    } else {
+        int iters = 0;
+        float tol_stop = 1e-6f * fabsf(x.tau + Di.o + L0i - L0j);
+        float tol_succ = P.newton_tol_frac * Fi->dL;
+        bool ok = walk ? newton_solve_walk(gi, N, W, xi, delta, P.newton_max_iter, tol_stop, tol_succ, xp, jn, iters)
+                       : newton_solve(N, xi, delta, P.newton_max_iter, tol_stop, tol_succ, xp, jn, iters);
+        if (st) { st->newton_calls++; st->newton_iters += iters; if (ok) st->newton_ok++; }
+        if (!ok) return false;
+        if (!(jn >= 1.0f / P.jac_max && jn <= P.jac_max)) return false;
+    }
+    float nb1, nb2;
+    int ptri = x.p_tri;
+    if (walk) {
+        float lam[3];
+        walk_bary(gi, W, xp[0], xp[1], lam);
+        ptri = W.tri; nb1 = lam[1]; nb2 = lam[2];
+    } else {
+        float3 e1 = xyz(__ldg(&gi.tri[3 * x.p_tri + 1])), e2 = xyz(__ldg(&gi.tri[3 * x.p_tri + 2]));
+        float e1t = dot3c(e1, N.fy.t), e2t = dot3c(e2, N.fy.t), e2b = dot3c(e2, N.fy.b);
+        nb2 = xp[1] / e2b;
+        nb1 = __fmaf_rn(-nb2, e2t, xp[0]) / e1t;
+    }
+    if (!(nb1 >= -kBaryEps && nb2 >= -kBaryEps && nb1 + nb2 <= 1.0f + kBaryEps)) return false;
+    const Surf pp = surf_atc(gi, ptri, nb1, nb2);
+    const Mat mp = load_mat(gi, pp.mat), m1 = load_mat(gi, Di.y1.mat);
+
+    // the offset path must reconnect at its second vertex too
+    if (mat_class(m1) != C_ROUGH || mat_class(mp) != C_ROUGH) return false;
+    if (len3c(Di.y1.p - pp.p) <= P.d_min) return false;
+    const Mat ms = load_mat(gi, sv.mat);
+    if (ns > 0) {
+        if (mat_class(ms) != C_ROUGH) return false;
+        if (len3c(pp.p - sv.p) <= P.d_min) return false;
+    }
+
+    float f = 1.0f;
+    f *= bsdf_fc(m1, Di.y1.n, dir_toc(Di.y1.p, Di.x0), dir_toc(Di.y1.p, pp.p));
+    f *= Gtermc(Di.y1.p, Di.y1.n, pp.p, pp.n);
+    // the two BSDF values behind p: at p and, with a suffix, at the vertex after it
+    if (ns == 0) {
+        float3 wl; float seg;
+        float lt = light_termc(Di, pp.p, pp.n, wl, seg);
+        f *= bsdf_fc(mp, pp.n, dir_toc(pp.p, Di.y1.p), wl) * lt;
+    } else {
+        f *= bsdf_fc(mp, pp.n, dir_toc(pp.p, Di.y1.p), dir_toc(pp.p, sv.p));
+        f *= Gtermc(pp.p, pp.n, sv.p, sv.n);
+        float3 wnext = ns > 1 ? dir_toc(sv.p, surf_atc(gi, x.s_tri[1], x.s_b1[1], x.s_b2[1]).p) : dir_toc(sv.p, lpos_i);
+        f *= bsdf_fc(ms, sv.n, dir_toc(sv.p, pp.p), wnext);
+    }
+    if (!(f > 0.f) || !isfinite(f)) return false;
+    float Lnew = plen + len3c(Di.y1.p - pp.p) + len3c(pp.p - p2y) + slen;
+    float tau = Lnew - Di.o;
+    if (!(tau >= L0i && tau < L0i + Fi->dL)) return false;
+    float jac = (x.pdf_pre / 1.0f) * jn;
+    if (!(jac > 0.f) || !isfinite(jac)) return false;
+
+    float Lsuf_i = x.Lsuf;
+    const bool suffix_eval = ns > 0 && !cache_ok;
+    if (ns > 0) {
+        if (suffix_eval) {
+            float Ls = 1.0f;
+            Surf a = sv;
+            for (int q = 1; q < ns; ++q) {
+                Surf b = q == 1 ? surf_atc(gi, x.s_tri[1], x.s_b1[1], x.s_b2[1]) : surf_atc(gi, x.s_tri[2], x.s_b1[2], x.s_b2[2]);
+                Mat mq = load_mat(gi, b.mat);
+                float gg = mat_class(load_mat(gi, a.mat)) == C_DELTA ? 1.0f : Gtermc(a.p, a.n, b.p, b.n);
+                if (mat_class(mq) == C_DELTA) {
+                    if (!geom_static) return false;
+                    Ls *= gg * mq.albedo;
+                } else {
+                    float3 wn = q + 1 < ns ? dir_toc(b.p, surf_atc(gi, x.s_tri[2], x.s_b1[2], x.s_b2[2]).p) : dir_toc(b.p, lpos_i);
+                    Ls *= gg * bsdf_fc(mq, b.n, dir_toc(b.p, a.p), wn);
+                }
+                a = b;
+            }
+            float3 wl; float seg;
+            Ls *= light_termc(Di, a.p, a.n, wl, seg);
+            Lsuf_i = Ls;
+        }
+        f *= Lsuf_i;
+    }
+    if (!(f > 0.f) || !isfinite(f)) return false;
+
+    if (!visible_q(vq, gi, Di.y1.p, Di.y1.n, pp.p, &pp.n, eps)) return false;
+    if (ns > 0) { if (!visible_q(vq, gi, pp.p, pp.n, sv.p, &sv.n, eps)) return false; }
+    else if (!light_visible(Di, gi, pp, eps, vq)) return false;
+    if (suffix_eval) {
+        Surf a = sv;
+        for (int q = 1; q < ns; ++q) {
+            Surf b = q == 1 ? surf_atc(gi, x.s_tri[1], x.s_b1[1], x.s_b2[1]) : surf_atc(gi, x.s_tri[2], x.s_b1[2], x.s_b2[2]);
+            if (!visible_q(vq, gi, a.p, a.n, b.p, &b.n, eps)) return false;
+            a = b;
+        }
+        if (!light_visible(Di, gi, a, eps, vq)) return false;
+    }
+
+    if (kOut) {
+        y = x;
+        y.tau = tau;
+        y.xprev = Di.y1.p;
+        y.pdf_pre = 1.0f;
         y.p_tri = ptri; y.p_b1 = nb1; y.p_b2 = nb2;
         y.Lsuf = Lsuf_i;
         y.phat = f;

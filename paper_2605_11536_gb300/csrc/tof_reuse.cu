@@ -240,39 +240,114 @@ __global__ void __launch_bounds__(128) reuse_units_kernel(const __grid_constant_
 // --------------------------------------------------------------------------------------------
 // forward shifts: slot s's sample into the unit's domain
 // --------------------------------------------------------------------------------------------
+// The shift kernels are bound by instruction fetch and the latency of scattered loads, not by occupancy:
+// they run the shift of records with r = 2 (shift_r2) in their loop and put the few others off, and 4
+// resident blocks an SM with all the registers they ask for are faster than 8 with a kilobyte of spills
+// (walking kernels of a 512 x 512 frame with flags 324: 5.12 -> 4.92 ms; transient 128 x 128 x 1024 4.67 ->
+// 4.52; the plain 512 x 512 frame 2.75 -> 2.73; 3, 5 and 6 blocks: 2.80, 2.85, 2.82).  Together with the
+// flat solve (newton_core): 512 x 512 frame 2.99 -> 2.73 ms, 1024 x 1024 12.1 -> 11.2, batch of 32 views
+// 16.3 -> 15.5.
+constexpr int kShiftBlocks = 4;
+
+// one forward task by the general shift; returns (shift_ok, newton called, newton ok, iterations << 3).
+// Out of line: few tasks need it, and its replay and local arrays stay out of the persistent loop.
 template <bool kWalk>
+__device__ __noinline__ uint32_t shift_fwd_general(const ReuseArgs& a, const WaveDev& w, uint32_t task) {
+    const int S = w.slots;
+    const uint32_t u = task >> 4;
+    const int s = (int)(task & 15u);
+    const int2 ub = w.units[u];
+    const int pix = ub.x, b = ub.y;
+    const int q = w.slot_pix[(size_t)pix * S + s];
+    const FrameDev* Fs = slot_frame(a, s);
+    const int sb = slot_bin(a, s, b);
+    Rec x, y;
+    rec_load(*slot_res(a, s), (size_t)q * (Fs->B > 0 ? Fs->B : 1) + sb, x);
+    const Domain Ds = pix_domain(Fs, q, sb), D0 = pix_domain(&a.cur, pix, b);
+    float py = 0.f, J = 1.f;
+    const bool geom_static = (a.temporal && s == 1) ? a.geom_static != 0 : true;
+    const size_t ui = (size_t)u * S + s;
+    VisQ vq;
+    vq.rays = w.rays; vq.counter = &w.counters[4]; vq.cap = w.ray_cap; vq.target = (uint32_t)ui;
+    ShiftStats st = {0, 0, 0, 0, 0};
+    const bool ok = shift_rec<true, kWalk>(x, Ds, D0, a.P, geom_static, y, py, J, &st, &vq);
+    w.py[ui] = ok ? py : 0.f;
+    w.jac[ui] = ok ? J : 1.f;
+    if (ok) store_rec(w.yrec, (size_t)w.cap_units * (S - 1), (size_t)u * (S - 1) + (s - 1), y);
+    return (st.shift_ok ? 1u : 0u) | (st.newton_calls ? 2u : 0u) | (st.newton_ok ? 4u : 0u) | (st.newton_iters << 3) |
+           (st.shift_calls ? 0x80000000u : 0u);
+}
+
+// tasks whose record reconnects beyond its second vertex, put off to the end of the warp's loop (or
+// until 32 of them wait), so that the others run without them
+struct Later {
+    uint32_t* list;   // the warp's 64 entries in shared memory
+    int n;
+    __device__ __forceinline__ void add(bool mine, uint32_t task) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, mine);
+        if (mine) list[n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = task;
+        n += __popc(m);
+        __syncwarp();
+    }
+};
+
+template <bool kWalk, bool kSame>
 __device__ __forceinline__ void shift_fwd_body(const ReuseArgs& a, const WaveDev& w) {
+    __shared__ uint32_t later_list[4][64];
     ShiftStats st = {0, 0, 0, 0, 0};
     const uint32_t ntask = min(w.counters[1], (uint32_t)w.cap_units * (uint32_t)(w.slots - 1));
     const int S = w.slots;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < ntask; t += gridDim.x * blockDim.x) {
-        uint32_t task = w.fwd[t];
-        uint32_t u = task >> 4;
-        int s = (int)(task & 15u);
-        int2 ub = w.units[u];
-        int pix = ub.x, b = ub.y;
-        int q = w.slot_pix[(size_t)pix * S + s];
-        const FrameDev* Fs = slot_frame(a, s);
-        const ResDev* Rs = slot_res(a, s);
-        int Bs = Fs->B > 0 ? Fs->B : 1;
-        Rec x;
-        const int sb = slot_bin(a, s, b);
-        rec_load(*Rs, (size_t)q * Bs + sb, x);
-        Domain Ds = pix_domain(Fs, q, sb);
-        Domain D0 = pix_domain(&a.cur, pix, b);
-        Rec y;
-        float py = 0.f, J = 1.f;
-        bool geom_static = (a.temporal && s == 1) ? a.geom_static != 0 : true;
-        size_t ui = (size_t)u * S + s;
-        VisQ vq;
-        vq.rays = w.rays; vq.counter = &w.counters[4]; vq.cap = w.ray_cap; vq.target = (uint32_t)ui;
-        bool ok = shift_rec<true, kWalk>(x, Ds, D0, a.P, geom_static, y, py, J, &st, &vq);
-        // visibility is settled by vis_kernel, which zeroes py of an occluded shift
-        w.py[ui] = ok ? py : 0.f;
-        w.jac[ui] = ok ? J : 1.f;
-        if (ok) {
-            store_rec(w.yrec, (size_t)w.cap_units * (S - 1), (size_t)u * (S - 1) + (s - 1), y);
+    const int lane = threadIdx.x & 31;
+    Later later;
+    later.list = later_list[threadIdx.x >> 5];
+    later.n = 0;
+    for (uint32_t t0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);; t0 += gridDim.x * blockDim.x) {
+        const bool more = t0 < ntask;
+        if (!more || later.n >= 32) {
+            if (lane < min(later.n, 32)) {
+                const uint32_t r = shift_fwd_general<kWalk>(a, w, later.list[later.n - 1 - lane]);
+                st.shift_ok += r & 1u; st.newton_calls += (r >> 1) & 1u; st.newton_ok += (r >> 2) & 1u;
+                st.newton_iters += (r & 0x7FFFFFFFu) >> 3; st.shift_calls += r >> 31;
+            }
+            __syncwarp();
+            later.n -= min(later.n, 32);
         }
+        if (!more) {
+            if (later.n > 0) { continue; }
+            break;
+        }
+        const uint32_t t = t0 + lane;
+        bool put_off = false;
+        uint32_t task = 0u;
+        if (t < ntask) {
+            task = w.fwd[t];
+            const uint32_t u = task >> 4;
+            const int s = (int)(task & 15u);
+            const int2 ub = w.units[u];
+            const int pix = ub.x, b = ub.y;
+            const int q = w.slot_pix[(size_t)pix * S + s];
+            const FrameDev* Fs = kSame ? &a.cur : slot_frame(a, s);
+            const int sb = slot_bin(a, s, b);
+            Rec x;
+            rec_load(kSame ? a.src : *slot_res(a, s), (size_t)q * (Fs->B > 0 ? Fs->B : 1) + sb, x);
+            const size_t ui = (size_t)u * S + s;
+            put_off = rec_r(x) > 2;
+            if (!put_off) {
+                Rec y;
+                float py = 0.f, J = 1.f;
+                const bool geom_static = kSame || (s == 1 ? a.geom_static != 0 : true);
+                VisQ vq;
+                vq.rays = w.rays; vq.counter = &w.counters[4]; vq.cap = w.ray_cap; vq.target = (uint32_t)ui;
+                const bool ok = rec_r(x) == 2 &&
+                    shift_r2<true, kWalk, kSame>(x, Fs, __ldg(&Fs->gb[q]), gate_L0r(*Fs, sb), &a.cur, __ldg(&a.cur.gb[pix]),
+                                                 gate_L0r(a.cur, b), a.P, geom_static, y, py, J, &st, &vq);
+                // visibility is settled by vis_kernel, which zeroes py of an occluded shift
+                w.py[ui] = ok ? py : 0.f;
+                w.jac[ui] = ok ? J : 1.f;
+                if (ok) store_rec(w.yrec, (size_t)w.cap_units * (S - 1), (size_t)u * (S - 1) + (s - 1), y);
+            }
+        }
+        later.add(put_off, task);
     }
     // warp-level flush of the shift statistics
     if (a.stats) {
@@ -286,9 +361,9 @@ __device__ __forceinline__ void shift_fwd_body(const ReuseArgs& a, const WaveDev
         }
     }
 }
-template <bool kWalk>
-__global__ void __launch_bounds__(128, 8) shift_fwd_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w) {
-    shift_fwd_body<kWalk>(a, w);
+template <bool kWalk, bool kSame>
+__global__ void __launch_bounds__(128, kShiftBlocks) shift_fwd_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w) {
+    shift_fwd_body<kWalk, kSame>(a, w);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -367,41 +442,92 @@ __global__ void __launch_bounds__(128) emit_inv_kernel(const __grid_constant__ R
 // --------------------------------------------------------------------------------------------
 // inverse shifts: candidate s's offset path (in the unit's domain) into domain j
 // --------------------------------------------------------------------------------------------
-// tasks [t0, t1) of the list; their visibility segments go to `rays` (counter rcount, capacity rcap)
+__device__ __forceinline__ void inv_record(const ReuseArgs& a, const WaveDev& w, uint32_t u, int s, int pix, int b, Rec& y) {
+    const int S = w.slots;
+    if (s == 0) {
+        rec_load(a.src, (size_t)pix * (a.cur.B > 0 ? a.cur.B : 1) + b, y);
+    } else {
+        ResDev R;
+        R.planes = w.yrec; R.stride = (size_t)w.cap_units * (S - 1); R.estride = 1;
+        rec_load(R, (size_t)u * (S - 1) + (s - 1), y);
+    }
+}
+// one inverse task by the general shift (see shift_fwd_general)
 template <bool kWalk>
+__device__ __noinline__ void shift_inv_general(const ReuseArgs& a, const WaveDev& w, uint32_t task, float4* rays, uint32_t* rcount,
+                                               uint32_t rcap) {
+    const int S = w.slots;
+    const uint32_t u = task >> 8;
+    const int s = (int)((task >> 4) & 15u), j = (int)(task & 15u);
+    const int2 ub = w.units[u];
+    const int pix = ub.x, b = ub.y;
+    Rec y, tmp;
+    inv_record(a, w, u, s, pix, b, y);
+    const int q = w.slot_pix[(size_t)pix * S + j];
+    const Domain D0 = pix_domain(&a.cur, pix, b), Dj = pix_domain(slot_frame(a, j), q, slot_bin(a, j, b));
+    const bool geom_static = (a.temporal && j == 1) ? a.geom_static != 0 : true;
+    float pj = 0.f, Jj = 1.f, term = 0.f;
+    const size_t ti = ((size_t)u * S + s) * S + j;
+    VisQ vq;
+    vq.rays = rays; vq.counter = rcount; vq.cap = rcap; vq.target = (uint32_t)ti;
+    if (slot_present(a, j, b) && shift_rec<false, kWalk>(y, D0, Dj, a.P, geom_static, tmp, pj, Jj, nullptr, &vq))
+        term = w.slot_M[(size_t)pix * S + j] * pj * Jj;
+    w.terms[ti] = term;
+}
+
+// tasks [t0, t1) of the list; their visibility segments go to `rays` (counter rcount, capacity rcap)
+template <bool kWalk, bool kSame>
 __device__ __forceinline__ void shift_inv_body(const ReuseArgs& a, const WaveDev& w, uint32_t t0, uint32_t t1, float4* rays,
                                                uint32_t* rcount, uint32_t rcap) {
+    __shared__ uint32_t later_list[4][64];
     const int S = w.slots;
-    const int Bn = a.cur.B > 0 ? a.cur.B : 1;
+    const int lane = threadIdx.x & 31;
     unsigned long long ninv = 0;
-    for (uint32_t t = t0 + blockIdx.x * blockDim.x + threadIdx.x; t < t1; t += gridDim.x * blockDim.x) {
-        ++ninv;
-        uint32_t task = w.inv[t];
-        uint32_t u = task >> 8;
-        int s = (int)((task >> 4) & 15u), j = (int)(task & 15u);
-        int2 ub = w.units[u];
-        int pix = ub.x, b = ub.y;
-        Rec y;
-        if (s == 0) {
-            rec_load(a.src, (size_t)pix * Bn + b, y);
-        } else {
-            ResDev R;
-            R.planes = w.yrec; R.stride = (size_t)w.cap_units * (S - 1); R.estride = 1;
-            rec_load(R, (size_t)u * (S - 1) + (s - 1), y);
+    Later later;
+    later.list = later_list[threadIdx.x >> 5];
+    later.n = 0;
+    for (uint32_t tw = t0 + blockIdx.x * blockDim.x + (threadIdx.x & ~31u);; tw += gridDim.x * blockDim.x) {
+        const bool more = tw < t1;
+        if (!more || later.n >= 32) {
+            if (lane < min(later.n, 32)) shift_inv_general<kWalk>(a, w, later.list[later.n - 1 - lane], rays, rcount, rcap);
+            __syncwarp();
+            later.n -= min(later.n, 32);
         }
-        int q = w.slot_pix[(size_t)pix * S + j];
-        Domain D0 = pix_domain(&a.cur, pix, b);
-        Domain Dj = pix_domain(slot_frame(a, j), q, slot_bin(a, j, b));
-        bool geom_static = (a.temporal && j == 1) ? a.geom_static != 0 : true;
-        Rec tmp;
-        float pj = 0.f, Jj = 1.f;
-        float term = 0.f;
-        const size_t ti = ((size_t)u * S + s) * S + j;
-        VisQ vq;
-        vq.rays = rays; vq.counter = rcount; vq.cap = rcap; vq.target = (uint32_t)ti;
-        if (slot_present(a, j, b) && shift_rec<false, kWalk>(y, D0, Dj, a.P, geom_static, tmp, pj, Jj, nullptr, &vq))
-            term = w.slot_M[(size_t)pix * S + j] * pj * Jj;
-        w.terms[ti] = term;
+        if (!more) {
+            if (later.n > 0) continue;
+            break;
+        }
+        const uint32_t t = tw + lane;
+        bool put_off = false;
+        uint32_t task = 0u;
+        if (t < t1) {
+            ++ninv;
+            task = w.inv[t];
+            const uint32_t u = task >> 8;
+            const int s = (int)((task >> 4) & 15u), j = (int)(task & 15u);
+            const int2 ub = w.units[u];
+            const int pix = ub.x, b = ub.y;
+            Rec y;
+            inv_record(a, w, u, s, pix, b, y);
+            put_off = rec_r(y) > 2;
+            if (!put_off) {
+                const int q = w.slot_pix[(size_t)pix * S + j];
+                const FrameDev* Fj = kSame ? &a.cur : slot_frame(a, j);
+                const int jb = slot_bin(a, j, b);
+                const bool geom_static = kSame || (j == 1 ? a.geom_static != 0 : true);
+                Rec tmp;
+                float pj = 0.f, Jj = 1.f, term = 0.f;
+                const size_t ti = ((size_t)u * S + s) * S + j;
+                VisQ vq;
+                vq.rays = rays; vq.counter = rcount; vq.cap = rcap; vq.target = (uint32_t)ti;
+                if (slot_present(a, j, b) && rec_r(y) == 2 &&
+                    shift_r2<false, kWalk, kSame>(y, &a.cur, __ldg(&a.cur.gb[pix]), gate_L0r(a.cur, b), Fj, __ldg(&Fj->gb[q]),
+                                                  gate_L0r(*Fj, jb), a.P, geom_static, tmp, pj, Jj, nullptr, &vq))
+                    term = w.slot_M[(size_t)pix * S + j] * pj * Jj;
+                w.terms[ti] = term;
+            }
+        }
+        later.add(put_off, task);
     }
     if (a.stats) {
         unsigned long long x = ninv;
@@ -416,12 +542,12 @@ __device__ __forceinline__ uint32_t inv_task_cap(const WaveDev& w) {
     return (uint32_t)w.cap_units * (uint32_t)w.slots * (uint32_t)(w.slots - 1);
 }
 // tasks [*lo, *hi) (lo null: from 0), read when the kernel starts
-template <bool kWalk>
-__global__ void __launch_bounds__(128, 8) shift_inv_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w,
+template <bool kWalk, bool kSame>
+__global__ void __launch_bounds__(128, kShiftBlocks) shift_inv_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w,
                                                           const uint32_t* lo, const uint32_t* hi, float4* rays, uint32_t* rcount,
                                                           uint32_t rcap) {
     const uint32_t cap = inv_task_cap(w);
-    shift_inv_body<kWalk>(a, w, lo ? min(*lo, cap) : 0u, min(*hi, cap), rays, rcount, rcap);
+    shift_inv_body<kWalk, kSame>(a, w, lo ? min(*lo, cap) : 0u, min(*hi, cap), rays, rcount, rcap);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -619,7 +745,7 @@ __global__ void __launch_bounds__(128) reuse_units_batch_kernel(const ReuseJob* 
 // stage k of the persistent part: 0 forward shifts, 1 their visibility, 2 inverse-task emission,
 // 3 inverse shifts, 4 their visibility, 5 merge
 template <int kStage>
-__global__ void __launch_bounds__(128, 8) reuse_persist_batch_kernel(const ReuseJob* __restrict__ J, int n) {
+__global__ void __launch_bounds__(128, kStage == 0 || kStage == 3 ? kShiftBlocks : 8) reuse_persist_batch_kernel(const ReuseJob* __restrict__ J, int n) {
     __shared__ ReuseJob s;
     for (int j = 0; j < n; ++j) {
         __syncthreads();
@@ -627,12 +753,18 @@ __global__ void __launch_bounds__(128, 8) reuse_persist_batch_kernel(const Reuse
         __syncthreads();
         const ReuseArgs& a = s.a;
         const WaveDev& w = s.w;
-        if constexpr (kStage == 0) shift_fwd_body<false>(a, w);
+        if constexpr (kStage == 0) {
+            if (a.temporal) shift_fwd_body<false, false>(a, w);
+            else shift_fwd_body<false, true>(a, w);
+        }
         else if constexpr (kStage == 1)
             vis_body(a.cur.g, w.rays, &w.counters[4], w.ray_cap, &w.counters[6], w.py, a.stats, 4, a.temporal ? -1 : 8, 32u);
         else if constexpr (kStage == 2) emit_inv_body(a, w);
         else if constexpr (kStage == 3)
-            shift_inv_body<false>(a, w, 0u, min(w.counters[2], inv_task_cap(w)), w.rays, &w.counters[5], w.ray_cap);
+            {
+                if (a.temporal) shift_inv_body<false, false>(a, w, 0u, min(w.counters[2], inv_task_cap(w)), w.rays, &w.counters[5], w.ray_cap);
+                else shift_inv_body<false, true>(a, w, 0u, min(w.counters[2], inv_task_cap(w)), w.rays, &w.counters[5], w.ray_cap);
+            }
         else if constexpr (kStage == 4)
             vis_body(a.temporal ? a.prev.g : a.cur.g, w.rays, &w.counters[5], w.ray_cap, &w.counters[7], w.terms, a.stats, -1,
                      a.temporal ? -1 : 9, 32u);
@@ -655,6 +787,15 @@ cudaError_t launch_reuse_batch(const ReuseJob* J, int n, const int* blk_slots, i
     return cudaGetLastError();
 }
 
+static void shift_inv_launch(const ReuseArgs& a, const WaveDev& w, const uint32_t* lo, const uint32_t* hi, float4* rays, uint32_t* rcount,
+                             uint32_t rcap, int blocks, cudaStream_t s) {
+    const bool walk = (a.P.flags & kFlagTriangleWalk) != 0u;
+    if (walk && a.temporal) shift_inv_kernel<true, false><<<blocks, 128, 0, s>>>(a, w, lo, hi, rays, rcount, rcap);
+    else if (walk) shift_inv_kernel<true, true><<<blocks, 128, 0, s>>>(a, w, lo, hi, rays, rcount, rcap);
+    else if (a.temporal) shift_inv_kernel<false, false><<<blocks, 128, 0, s>>>(a, w, lo, hi, rays, rcount, rcap);
+    else shift_inv_kernel<false, true><<<blocks, 128, 0, s>>>(a, w, lo, hi, rays, rcount, rcap);
+}
+
 // ev (optional): 7 events recorded around the stages (setup | forward shifts | their visibility and
 // the inverse-task emission | inverse shifts | their visibility | merge) for per-stage timing
 // One reuse pass.  With a second queue (w.rays2) and a second stream s2, the canonical samples'
@@ -664,8 +805,8 @@ cudaError_t launch_reuse_batch(const ReuseJob* J, int n, const int* blk_slots, i
 // segments are the same ones, so the results are those of the single sequence, which runs without
 // rays2 (spatial passes, batches, the allocation-free form).  Small passes gain: their persistent
 // kernels wait on a few long dependent chains while most of the GPU idles.
-cudaError_t launch_reuse_wave(const ReuseArgs& a, const WaveDev& w, int p0, int p1, int persist_blocks, int vis_blocks,
-                              cudaEvent_t* ev, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join) {
+cudaError_t launch_reuse_wave(const ReuseArgs& a, const WaveDev& w, int p0, int p1, int persist_blocks, int shift_blocks,
+                              int vis_blocks, cudaEvent_t* ev, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join) {
     cudaError_t e = cudaMemsetAsync(w.counters, 0, kWaveCounters * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     int np = p1 - p0;
@@ -690,15 +831,17 @@ cudaError_t launch_reuse_wave(const ReuseArgs& a, const WaveDev& w, int p0, int 
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s2, fork, 0);
         if (e != cudaSuccess) return e;
         note_launch(2);
-        if (walk) shift_inv_kernel<true><<<persist_blocks, 128, 0, s2>>>(a, w, nullptr, &w.counters[8], w.rays2, &w.counters[9], w.ray2_cap);
-        else shift_inv_kernel<false><<<persist_blocks, 128, 0, s2>>>(a, w, nullptr, &w.counters[8], w.rays2, &w.counters[9], w.ray2_cap);
+        shift_inv_launch(a, w, nullptr, &w.counters[8], w.rays2, &w.counters[9], w.ray2_cap, shift_blocks, s2);
         vis_kernel<<<vis_blocks, 128, 0, s2>>>(ginv, w.rays2, &w.counters[9], w.ray2_cap, &w.counters[10], w.terms, a.stats, -1,
                                                a.temporal ? -1 : 9);
         e = cudaEventRecord(join, s2);
         if (e != cudaSuccess) return e;
     }
-    if (walk) { note_launch(); shift_fwd_kernel<true><<<persist_blocks, 128, 0, s>>>(a, w); }
-    else { note_launch(); shift_fwd_kernel<false><<<persist_blocks, 128, 0, s>>>(a, w); }
+    note_launch();
+    if (walk && a.temporal) shift_fwd_kernel<true, false><<<shift_blocks, 128, 0, s>>>(a, w);
+    else if (walk) shift_fwd_kernel<true, true><<<shift_blocks, 128, 0, s>>>(a, w);
+    else if (a.temporal) shift_fwd_kernel<false, false><<<shift_blocks, 128, 0, s>>>(a, w);
+    else shift_fwd_kernel<false, true><<<shift_blocks, 128, 0, s>>>(a, w);
     if (ev) cudaEventRecord(ev[2], s);
     // forward shifts land in the current frame; counter 4 of the stats counted them as successes
     note_launch();
@@ -715,8 +858,8 @@ cudaError_t launch_reuse_wave(const ReuseArgs& a, const WaveDev& w, int p0, int 
     }
     if (emits || !beside) {   // beside with nothing emitted: the second stream did every inverse shift
         const uint32_t* lo = beside ? &w.counters[8] : nullptr;
-        if (walk) { note_launch(); shift_inv_kernel<true><<<persist_blocks, 128, 0, s>>>(a, w, lo, &w.counters[2], w.rays, &w.counters[5], w.ray_cap); }
-        else { note_launch(); shift_inv_kernel<false><<<persist_blocks, 128, 0, s>>>(a, w, lo, &w.counters[2], w.rays, &w.counters[5], w.ray_cap); }
+        note_launch();
+        shift_inv_launch(a, w, lo, &w.counters[2], w.rays, &w.counters[5], w.ray_cap, shift_blocks, s);
     }
     if (ev) cudaEventRecord(ev[4], s);
     if (emits || !beside) {
@@ -739,19 +882,21 @@ cudaError_t launch_vis_queue(const GeomDev& g, const float4* rays, const uint32_
     return cudaGetLastError();
 }
 
-cudaError_t reuse_persist_blocks(int* out, int* vis_out) {
+// blocks resident on every SM at once: of the merge (the emission's and the batched stages' grid too), the
+// shift kernels and the visibility kernel
+cudaError_t reuse_persist_blocks(int* merge_out, int* shift_out, int* vis_out) {
     int dev = 0, sms = 0, b1 = 0, b2 = 0, b3 = 0, b4 = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, shift_fwd_kernel<false>, 128, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, shift_inv_kernel<false>, 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, shift_fwd_kernel<false, true>, 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, shift_inv_kernel<false, true>, 128, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b3, reuse_merge_kernel, 128, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b4, vis_kernel, 128, 0);
-    int b = b1;
-    if (b2 < b) b = b2;
-    if (b3 < b) b = b3;
-    *out = sms * (b > 0 ? b : 1);
+    if (b2 < b1) b1 = b2;
+    if (b3 > 8) b3 = 8;
+    *merge_out = sms * (b3 > 0 ? b3 : 1);
+    *shift_out = sms * (b1 > 0 ? b1 : 1);
     *vis_out = sms * (b4 > 0 ? b4 : 1);
     return cudaGetLastError();
 }
