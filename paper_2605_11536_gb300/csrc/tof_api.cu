@@ -44,6 +44,7 @@ cudaError_t launch_etree(int nt, int P, const float4* tri, float4* node, cudaStr
 cudaError_t launch_refit(int n, const uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, const int* child,
                          const int* parent_int, const int* parent_leaf, uint32_t* counter, cudaStream_t s);
 cudaError_t launch_gbuffer_batch(const GbufArgs* A, const int* blk0, int n, int blocks, cudaStream_t s);
+int initial_lanes_blocks(int W, int H, int n_cand);
 cudaError_t launch_initial_batch(const InitArgs* A, const int* blk0, int n, int blocks, cudaStream_t s);
 cudaError_t launch_reuse_batch(const ReuseJob* J, int n, const int* blk_slots, int nblk_slots, const int* blk_units,
                                int nblk_units, int persist_blocks, int vis_blocks, cudaStream_t s);
@@ -133,6 +134,7 @@ struct ViewH {
     void* ell_ptrs[9] = {nullptr};
     TreeWaveDev tw;              // the gated initial stage's bounce wavefront
     size_t tw_paths = 0;         // pixels x trees it holds
+    size_t tw_denied = 0;        // pixels x trees of a histogram view that there was no room for
     void* tw_ptrs[9] = {nullptr};
     tof_tuning tune = {16, 8, 0, TOF_LAYOUT_SOA};   // launch shapes and reservoir layout (autotuner)
 };
@@ -713,19 +715,27 @@ static tof_status ensure_tree_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
     for (void*& p : V.tw_ptrs) { dfree(c, p); p = nullptr; }
     V.tw_paths = 0;
     TreeWaveDev& w = V.tw;
+    w = TreeWaveDev();
     w.nc = nc; w.depth = depth;
-    TRY(dalloc(c, &w.vtx, sizeof(float4) * slots, "tree wave vertices"));
-    TRY(dalloc(c, &w.acand, sizeof(float2) * slots, "tree wave candidates"));
-    TRY(dalloc(c, &w.ps0, sizeof(float4) * paths, "tree wave path throughputs"));
-    TRY(dalloc(c, &w.ps1, sizeof(float4) * paths, "tree wave path vertices"));
-    TRY(dalloc(c, &w.rays[0], sizeof(float4) * 2 * paths, "tree wave rays"));
-    TRY(dalloc(c, &w.rays[1], sizeof(float4) * 2 * paths, "tree wave rays"));
-    TRY(dalloc(c, &w.hits, sizeof(float4) * paths, "tree wave hits"));
-    w.path_cap = (uint32_t)paths;
-    TRY(dalloc(c, &w.srays, sizeof(float4) * 2 * paths, "tree wave light segments"));
-    w.sray_cap = (uint32_t)paths;   // more segments than paths are traced in place
-    TRY(dalloc(c, &w.counters, sizeof(uint32_t) * kTreeWaveCounters, "tree wave counters"));
+    const tof_status st = [&]() -> tof_status {
+        TRY(dalloc(c, &w.vtx, sizeof(float4) * slots, "tree wave vertices"));
+        TRY(dalloc(c, &w.acand, sizeof(float2) * slots, "tree wave candidates"));
+        TRY(dalloc(c, &w.ps0, sizeof(float4) * paths, "tree wave path throughputs"));
+        TRY(dalloc(c, &w.ps1, sizeof(float4) * paths, "tree wave path vertices"));
+        TRY(dalloc(c, &w.rays[0], sizeof(float4) * 2 * paths, "tree wave rays"));
+        TRY(dalloc(c, &w.rays[1], sizeof(float4) * 2 * paths, "tree wave rays"));
+        TRY(dalloc(c, &w.hits, sizeof(float4) * paths, "tree wave hits"));
+        w.path_cap = (uint32_t)paths;
+        TRY(dalloc(c, &w.srays, sizeof(float4) * 2 * paths, "tree wave light segments"));
+        w.sray_cap = (uint32_t)paths;   // more segments than paths are traced in place
+        TRY(dalloc(c, &w.counters, sizeof(uint32_t) * kTreeWaveCounters, "tree wave counters"));
+        return TOF_OK;
+    }();
     void* ps[9] = {w.vtx, w.acand, w.ps0, w.ps1, w.rays[0], w.rays[1], w.hits, w.srays, w.counters};
+    if (st != TOF_OK) {
+        for (void* p : ps) dfree(c, p);   // nothing is kept of what there was room for
+        return st;
+    }
     for (int k = 0; k < 9; ++k) V.tw_ptrs[k] = ps[k];
     V.tw_paths = paths;
     return TOF_OK;
@@ -737,7 +747,7 @@ static tof_status ensure_tree_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
 // pay for its 2 * depth + 1 launches each).  The rest keep the single kernel, which needs no scratch.
 // Both give the same reservoirs.
 static bool use_tree_wave(const ViewH& V, int B, const tof_params* p, bool fixed) {
-    if (fixed || B > 0 || (p->flags & TOF_FLAG_ELLIPSOID) || p->shrink_k > 1.f) return false;
+    if (fixed || (p->flags & TOF_FLAG_ELLIPSOID) || p->shrink_k > 1.f) return false;
     return (double)V.W * V.H * p->n_cand <= 16.0 * 1024.0 * 1024.0;
 }
 
@@ -753,6 +763,20 @@ static bool batch_tree_wave(const ViewH& V, const tof_job& J) {
 static bool tree_wave_ready(const ViewH& V, const tof_params* p) {
     return (size_t)V.W * V.H >= kBatchWaveMinPix && V.tw_paths >= (size_t)V.W * V.H * (size_t)p->n_cand &&
            V.tw.nc == p->n_cand && V.tw.depth == p->depth;
+}
+
+// a histogram's initial stage runs as the wavefront in direct renders, where its scratch (2 KB a pixel with 8
+// trees of depth 4, against 300 B a bin of the view itself) is to be had; batches and the served form, which
+// account their views' memory beforehand, keep the single kernel
+static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p) {
+    if (c->in_batch || g_rec) return false;
+    const std::string before = c->err;
+    const size_t paths = (size_t)V.W * V.H * (size_t)p->n_cand;
+    if (V.tw_denied && paths >= V.tw_denied) return false;
+    if (ensure_tree_wave(c, V, p->n_cand, p->depth) == TOF_OK) return true;
+    V.tw_denied = paths;   // not tried again at every frame
+    c->err = before;
+    return false;
 }
 
 // the initial stage runs as the ellipsoidal wavefront: gated, ellipsoidal connection, not the
@@ -950,7 +974,7 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
             CK(launch_initial_ell_wave(ia, V.ell, V.tune.tile_h, eb, vb, s));
         }
     } else if (use_tree_wave(V, B, params, fixed_wave != nullptr) &&
-               (!(c->in_batch || g_rec) || tree_wave_ready(V, params))) {
+               (B > 0 ? hist_tree_wave(c, V, params) : !(c->in_batch || g_rec) || tree_wave_ready(V, params))) {
         // a batch uses the wavefront only where prepare_job allocated its scratch (large views)
         TRY(ensure_tree_wave(c, V, params->n_cand, params->depth));
         TRY(persist_init(c));
@@ -1187,24 +1211,29 @@ static size_t al256h(size_t b) { return (b + 255) / 256 * 256; }
 // argument tables of one group of a staged batch, laid out in the slot's staging buffer from `off`
 struct StagedGroup {
     BatchRec rec;
-    std::vector<int> bpix;
+    std::vector<int> bpix, binit;
     std::vector<std::vector<int>> bs, bu;
-    size_t o_g = 0, o_i = 0, o_b = 0;
+    size_t o_g = 0, o_i = 0, o_b = 0, o_bi = 0;
     std::vector<size_t> o_p, o_s, o_u;
 };
 static size_t staged_layout(StagedGroup& G, size_t off) {
     const size_t nj = G.rec.gbuf.size(), np = G.rec.pass.size();
     G.bpix.assign(nj + 1, 0);
+    G.binit.assign(nj + 1, 0);
     for (size_t j = 0; j < nj; ++j) {
         const GbufArgs& g = G.rec.gbuf[j];
         const int tw = g.tile_w, th = 128 / tw;
         G.bpix[j + 1] = G.bpix[j] + ((g.F.W + tw - 1) / tw) * ((g.F.H + th - 1) / th);
+        // an instance that runs the bounce wavefront needs no blocks here
+        G.binit[j + 1] = G.binit[j] + (G.rec.init[j].wave ? 0 : initial_lanes_blocks(g.F.W, g.F.H, g.P.n_cand));
     }
     G.o_g = off;
     off = al256h(off + sizeof(GbufArgs) * nj);
     G.o_i = off;
     off = al256h(off + sizeof(InitArgs) * nj);
     G.o_b = off;
+    off = al256h(off + sizeof(int) * (nj + 1));
+    G.o_bi = off;
     off = al256h(off + sizeof(int) * (nj + 1));
     G.o_p.assign(np, 0); G.o_s.assign(np, 0); G.o_u.assign(np, 0);
     G.bs.assign(np, {}); G.bu.assign(np, {});
@@ -1231,6 +1260,7 @@ static void staged_fill(const StagedGroup& G, unsigned char* h) {
     memcpy(h + G.o_g, G.rec.gbuf.data(), sizeof(GbufArgs) * nj);
     memcpy(h + G.o_i, G.rec.init.data(), sizeof(InitArgs) * nj);
     memcpy(h + G.o_b, G.bpix.data(), sizeof(int) * (nj + 1));
+    memcpy(h + G.o_bi, G.binit.data(), sizeof(int) * (nj + 1));
     for (size_t q = 0; q < G.rec.pass.size(); ++q) {
         memcpy(h + G.o_p[q], G.rec.pass[q].data(), sizeof(ReuseJob) * G.rec.pass[q].size());
         memcpy(h + G.o_s[q], G.bs[q].data(), sizeof(int) * G.bs[q].size());
@@ -1241,7 +1271,8 @@ static cudaError_t staged_launch(tof_ctx* c, const StagedGroup& G, unsigned char
     const int nj = (int)G.rec.gbuf.size();
     if (nj == 0) return cudaSuccess;
     cudaError_t e = launch_gbuffer_batch((const GbufArgs*)(d + G.o_g), (const int*)(d + G.o_b), nj, G.bpix[nj], q);
-    if (e == cudaSuccess) e = launch_initial_batch((const InitArgs*)(d + G.o_i), (const int*)(d + G.o_b), nj, G.bpix[nj], q);
+    if (e == cudaSuccess && G.binit[nj] > 0)
+        e = launch_initial_batch((const InitArgs*)(d + G.o_i), (const int*)(d + G.o_bi), nj, G.binit[nj], q);
     for (size_t k = 0; k < G.rec.wave.size() && e == cudaSuccess; ++k) {
         const WaveRec& w = G.rec.wave[k];
         e = launch_initial_tree_wave(w.a, w.w, w.tile_h, w.hit_blocks, w.vis_blocks, q);

@@ -65,8 +65,9 @@ static __device__ __noinline__ float nee_eval(const Domain& D, const Surf& x, co
 // by the balance heuristic over the two densities of that vertex (Sec. 5: MIS between the direct
 // and the ellipsoidal connection):  c_tree *= p_tree / (p_tree + p_ell),  c_ell = f / (p_tree + p_ell).
 // kEll = 1 places the ellipsoidal vertex in place; kEll = 2 (the wavefront) only records every
-// vertex (sink.vertex) and the ellipsoidal requests (sink.request) for a later pass.
-template <int kEll = 0, class Sink>
+// vertex (sink.vertex) and the ellipsoidal requests (sink.request) for a later pass.  kRecord: every vertex
+// goes to sink.vertex.
+template <int kEll = 0, bool kRecord = false, class Sink>
 __device__ void trace_tree(const Domain& D, const ParamsDev& P, uint32_t px, uint32_t frame, int tree, float glo, float ghi,
                            TreeVerts& T, Sink& sink) {
     const GeomDev& g = D.F->g;
@@ -82,7 +83,7 @@ __device__ void trace_tree(const Domain& D, const ParamsDev& P, uint32_t px, uin
         const Surf& x = T.v[d];
         Mat m = load_mat(g, x.mat);
         float3 wi = dir_to(x.p, d == 1 ? D.x0 : T.v[d - 1].p);
-        if constexpr (kEll == 2) sink.vertex(d, T, beta, len);
+        if constexpr (kEll == 2 || kRecord) sink.vertex(d, T, beta, len);
         if (d >= kmin && mat_class(m) != C_DELTA) {
             float lt, seg;
             const float fs = nee_eval(D, x, m, wi, lt, seg);
@@ -258,12 +259,12 @@ struct GatedSink {
     }
 };
 
-// gated views: the same trees, candidates, order and uniforms as initial_kernel, into GatedSink
-template <bool kEll>
-__device__ __forceinline__ void initial_gated_body(const InitArgs& a, int bx, int by) {
+// gated views with the ellipsoidal connection: the same trees, candidates, order and uniforms as
+// initial_kernel, into GatedSink
+__global__ void __launch_bounds__(128, 4) initial_gated_ell_kernel(const __grid_constant__ InitArgs a) {
     const FrameDev& F = a.F;
     int ix, iy;
-    tile_pixel(a.tile_w, bx, by, ix, iy);
+    tile_pixel(a.tile_w, ix, iy);
     if (ix >= F.W || iy >= F.H) return;
     const int pix = iy * F.W + ix;
     const ParamsDev& P = a.P;
@@ -283,7 +284,7 @@ __device__ __forceinline__ void initial_gated_body(const InitArgs& a, int bx, in
     TreeVerts T;
     for (int t = 0; t < P.n_cand; ++t) {
         sink.tree = t;
-        trace_tree<kEll ? 1 : 0>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
+        trace_tree<1>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
     }
     float outv = 0.f;
     uint32_t occ = 0u;
@@ -296,20 +297,127 @@ __device__ __forceinline__ void initial_gated_body(const InitArgs& a, int bx, in
     a.dst.occ[pix] = occ;
     if (a.out) a.out[pix] = outv;
 }
-template <bool kEll>
-__global__ void __launch_bounds__(128, kEll ? 4 : 6) initial_gated_kernel(const __grid_constant__ InitArgs a) {
-    initial_gated_body<kEll>(a, blockIdx.x, blockIdx.y);
+// Path trees in lanes: a block of 128 threads takes a small tile of pixels with one thread for each (pixel,
+// tree), which records its candidates and vertices in shared memory; then one thread per pixel replays
+// the streaming RIS in the trees' order -- the same trees, candidates, order and uniforms as one thread
+// walking the pixel's trees, without its chain of all of them.  Such a thread is bound by that chain's
+// latency (a 128 x 128 view has only 4 warps an SM), so a small view gains what the trees are parallel.
+constexpr int kLaneThreads = 128;
+struct LaneTile { int w, h; };   // pixels of a block; w * h * n_cand <= kLaneThreads
+static __host__ __device__ __forceinline__ LaneTile lane_tile(int n_cand) {
+    const int pixels = kLaneThreads / n_cand;   // at least 2 (kMaxCand = 64)
+    LaneTile t;
+    t.w = pixels >= 8 ? 8 : pixels >= 4 ? 4 : 2;
+    t.h = pixels / t.w;
+    return t;
 }
-__global__ void __launch_bounds__(128, 6) initial_gated_batch_kernel(const InitArgs* __restrict__ A, const int* __restrict__ blk0,
-                                                                     int n) {
+struct LaneTable {
+    float2 cand[kLaneThreads * kMaxDepth];   // (f / p, tau) of the candidate ending at vertex d of a thread's tree
+    float4 vtx[kLaneThreads * kMaxDepth];    // (tri bits, b1, b2, area pdf) of vertex d
+};
+struct LaneSink {
+    float2* cand;
+    float4* vtx;
+    __device__ void operator()(int k, float c, float tauv, const TreeVerts&, int) { cand[k - 1] = make_float2(c, tauv); }
+    __device__ void vertex(int d, const TreeVerts& T, float, float) {
+        const Surf& v = T.v[d];
+        vtx[d - 1] = make_float4(__int_as_float(v.tri), v.b1, v.b2, T.pdfA[d]);
+    }
+};
+__device__ __forceinline__ void initial_lanes_body(const InitArgs& a, int bx, int by, LaneTable& tab) {
+    const FrameDev& F = a.F;
+    const ParamsDev& P = a.P;
+    const int nc = P.n_cand, depth = P.depth;
+    const LaneTile tile = lane_tile(nc);
+    const int npx = tile.w * tile.h;
+    const int pl = (int)threadIdx.x / nc, t = (int)threadIdx.x % nc;
+    if (pl < npx) {
+        const int ix = bx * tile.w + pl % tile.w, iy = by * tile.h + pl / tile.w;
+        LaneSink sink;
+        sink.cand = tab.cand + threadIdx.x * kMaxDepth;
+        sink.vtx = tab.vtx + threadIdx.x * kMaxDepth;
+        for (int d = 0; d < depth; ++d) sink.cand[d] = make_float2(0.f, 0.f);
+        if (ix < F.W && iy < F.H) {
+            const int pix = iy * F.W + ix;
+            const float4 gb = F.gb[pix];
+            const uint32_t tri = __float_as_uint(gb.x);
+            Domain D = make_domain_hit(&F, tri != kNoHit, (int)tri, gb.y, gb.z, gb.w, F.L0, F.dL);
+            if (D.valid) {
+                TreeVerts T;
+                trace_tree<0, true>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
+            }
+        }
+    }
+    __syncthreads();
+    if ((int)threadIdx.x >= npx) return;
+    const int q = (int)threadIdx.x;
+    const int ix = bx * tile.w + q % tile.w, iy = by * tile.h + q / tile.w;
+    if (ix >= F.W || iy >= F.H) return;
+    const int pix = iy * F.W + ix;
+    a.dst.M[pix] = (float)nc;
+    const float4 gb = F.gb[pix];
+    const uint32_t tri = __float_as_uint(gb.x);
+    const float invN = 1.0f / (float)nc;
+    float S = 0.f, sel_tau = 0.f, outv = 0.f;
+    int sel_t = -1, sel_k = 0;
+    uint32_t occ = 0u;
+    if (tri != kNoHit) {
+        for (int u = 0; u < nc; ++u)
+            for (int d = (P.flags & 1u) ? 1 : 2; d <= depth; ++d) {
+                const float2 ac = tab.cand[(q * nc + u) * kMaxDepth + d - 1];
+                const float wv = invN * ac.x;
+                if (!(wv > 0.f)) continue;
+                const uint4 r = philox((uint32_t)pix, F.frame, ((uint32_t)u << 8) | (uint32_t)d, P_RIS, P.seed);
+                S += wv;
+                if (u01(r.x) * S < wv) { sel_t = u; sel_k = d; sel_tau = ac.y; }
+            }
+    }
+    if (sel_t >= 0) {
+        Domain D = make_domain_hit(&F, true, (int)tri, gb.y, gb.z, gb.w, F.L0, F.dL);
+        const GeomDev& g = F.g;
+        TreeVerts T;
+        T.v[1] = D.y1;
+        T.cls[1] = mat_class(load_mat(g, D.y1.mat));
+        T.pdfA[1] = 1.0f;
+        for (int j = 2; j <= sel_k; ++j) {
+            const float4 v = tab.vtx[(q * nc + sel_t) * kMaxDepth + j - 1];
+            T.v[j] = surf_at(g, __float_as_int(v.x), v.y, v.z);
+            T.cls[j] = mat_class(load_mat(g, T.v[j].mat));
+            T.pdfA[j] = v.w;
+        }
+        Rec r;
+        build_rec(D, T, sel_k, sel_t, (uint32_t)pix, F.frame, sel_tau, P, r);
+        store_tail(a.dst, (size_t)pix, r);
+        if (r.phat > 0.f) {
+            const float W = S / r.phat;
+            *res_at(a.dst, 0, (size_t)pix) = make_float4(W, r.phat, sel_tau, r.Lsuf);
+            occ = 1u;
+            outv = r.phat * W;
+        }
+    }
+    a.dst.occ[pix] = occ;
+    if (a.out) a.out[pix] = outv;
+}
+__global__ void __launch_bounds__(kLaneThreads, 6) initial_lanes_kernel(const __grid_constant__ InitArgs a) {
+    __shared__ LaneTable tab;
+    initial_lanes_body(a, blockIdx.x, blockIdx.y, tab);
+}
+__global__ void __launch_bounds__(kLaneThreads, 6) initial_lanes_batch_kernel(const InitArgs* __restrict__ A, const int* __restrict__ blk0,
+                                                                              int n) {
     __shared__ InitArgs s;
+    __shared__ LaneTable tab;
     const int j = batch_job(blk0, n);
     block_copy(&s, &A[j]);
     __syncthreads();
     if (s.wave) return;   // launched as the bounce wavefront after this kernel (the whole block)
     const int lb = (int)blockIdx.x - __ldg(&blk0[j]);
-    const int tx = (s.F.W + s.tile_w - 1) / s.tile_w;
-    initial_gated_body<false>(s, lb % tx, lb / tx);
+    const int tx = (s.F.W + lane_tile(s.P.n_cand).w - 1) / lane_tile(s.P.n_cand).w;
+    initial_lanes_body(s, lb % tx, lb / tx, tab);
+}
+// blocks of the lane form over a view
+int initial_lanes_blocks(int W, int H, int n_cand) {
+    const LaneTile t = lane_tile(n_cand);
+    return ((W + t.w - 1) / t.w) * ((H + t.h - 1) / t.h);
 }
 
 // 6 resident blocks per SM (80 registers): 1.08 against 1.11 ms at 5 blocks (96 registers) on the
@@ -523,6 +631,76 @@ __global__ void __launch_bounds__(128) tree_select_kernel(const __grid_constant_
     if (a.out) a.out[pix] = outv;
 }
 
+// The selection of the tree wavefront for histograms: every candidate streams into the reservoir of its own
+// bin (Sec. 4.5).  One warp per pixel, lane i the i-th candidate in the trees' order (at most
+// kMaxBinsPerPixel = 32, tested by the host): the lanes of a bin form its running sums by shuffles in that
+// order, the last accepted lane of a bin builds and stores its record.
+__global__ void __launch_bounds__(128) tree_select_bins_kernel(const __grid_constant__ InitArgs a, const TreeWaveDev w) {
+    const FrameDev& F = a.F;
+    const ParamsDev& P = a.P;
+    const int pix = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (pix >= F.W * F.H) return;
+    uint32_t* occ = a.dst.occ + (size_t)pix * a.dst.words;
+    for (int q = lane; q < a.dst.words; q += 32) occ[q] = 0u;
+    if (lane == 0) a.dst.M[pix] = (float)P.n_cand;
+    const float4 gb = F.gb[pix];
+    const uint32_t tri = __float_as_uint(gb.x);
+    if (tri == kNoHit) return;
+    const int kmin = (P.flags & 1u) ? 1 : 2, lengths = P.depth - kmin + 1;
+    const int n = lengths > 0 ? P.n_cand * lengths : 0;
+    const float invN = 1.0f / (float)P.n_cand;
+    int t = 0, d = 1, b = 0;
+    float wv = 0.f, tau = 0.f;
+    bool valid = false;
+    if (lane < n) {
+        t = lane / lengths;
+        d = kmin + lane % lengths;
+        const float2 ac = w.acand[((size_t)pix * w.nc + t) * w.depth + d - 1];
+        wv = invN * ac.x;
+        tau = ac.y;
+        const float fb = floorf((tau - F.L0) / F.dL);
+        valid = wv > 0.f && fb >= 0.f && fb < (float)F.B;
+        b = valid ? (int)fb : 0;
+    }
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, valid ? b : -1 - lane);
+    float S = 0.f, Sall = 0.f;
+    for (int j = 0; j < n; ++j) {
+        const float wj = __shfl_sync(0xFFFFFFFFu, wv, j);
+        if ((peers >> j) & 1u) {
+            Sall += wj;
+            if (j <= lane) S += wj;
+        }
+    }
+    bool acc = false;
+    if (valid) {
+        const uint4 u = philox((uint32_t)pix, F.frame, ((uint32_t)t << 8) | (uint32_t)d, P_RIS, P.seed);
+        acc = u01(u.x) * S < wv;
+    }
+    const unsigned won = __ballot_sync(0xFFFFFFFFu, acc) & peers;
+    __syncwarp();   // the occupancy words are zeroed before any lane sets a bit
+    if (!acc || 31 - __clz(won) != lane) return;
+    const GeomDev& g = F.g;
+    Domain D = make_domain_hit(&F, true, (int)tri, gb.y, gb.z, gb.w, F.L0, F.dL);
+    TreeVerts T;
+    T.v[1] = D.y1;
+    T.cls[1] = mat_class(load_mat(g, D.y1.mat));
+    T.pdfA[1] = 1.0f;
+    const size_t base = ((size_t)pix * w.nc + t) * w.depth;
+    for (int j = 2; j <= d; ++j) {
+        const float4 v = w.vtx[base + j - 1];
+        T.v[j] = surf_at(g, __float_as_int(v.x), v.y, v.z);
+        T.cls[j] = mat_class(load_mat(g, T.v[j].mat));
+        T.pdfA[j] = v.w;
+    }
+    Rec r;
+    build_rec(D, T, d, t, (uint32_t)pix, F.frame, tau, P, r);
+    const size_t idx = (size_t)pix * F.B + b;
+    store_tail(a.dst, idx, r);
+    if (!(r.phat > 0.f)) return;
+    *res_at(a.dst, 0, idx) = make_float4(Sall / r.phat, r.phat, tau, r.Lsuf);
+    atomicOr(&occ[b >> 5], 1u << (b & 31));
+}
+
 // --------------------------------------------------------------------------------------------
 // gated initial candidates as a bounce wavefront (TreeWaveDev): the same trees, candidates,
 // uniforms and order as initial_gated_kernel<false>, so the same reservoirs, with every lane of a
@@ -560,7 +738,7 @@ __device__ __forceinline__ void tw_vertex(const InitArgs& a, const TreeWaveDev& 
         const float fs = nee_eval(D, x, m, wi, lt, seg);
         if (fs > 0.f) {
             float tau = len + seg - D.o;
-            if (tau >= F.L0 && tau < F.L0 + F.dL) {
+            if (tau >= F.L0 && tau < (F.B > 0 ? F.L0 + F.B * F.dL : F.L0 + F.dL)) {
                 float c = beta * fs * lt;
                 if constexpr (kEll) {
                     if (d > 1) {
@@ -796,48 +974,68 @@ __global__ void __launch_bounds__(256) splat_kernel(const __grid_constant__ Spla
 // --------------------------------------------------------------------------------------------
 // plain path tracing (comparison method of Sec. 6)
 // --------------------------------------------------------------------------------------------
+// One thread per sample: a block takes blockDim.x / G pixels with G = min(spp, blockDim.x) samples of each at
+// a time, whose contributions stay in shared memory until one thread per pixel adds them in the samples'
+// order (the sum of one thread running through them).  With one thread per pixel, a 200 x 150 image had
+// 6 warps an SM, each waiting on its own chain of spp * depth traversals.
 struct PtSink {
-    float* row;
-    int B;
-    float t0, w, scale;
-    __device__ void operator()(int k, float c, float tau, const TreeVerts& T, int strategy) {
-        (void)k; (void)T; (void)strategy;
-        if (B > 0) {
-            float fb = floorf((tau - t0) / w);
-            if (!(fb >= 0.f && fb < (float)B)) return;
-            row[(int)fb] += scale * c;
-        } else {
-            row[0] += scale * c;
-        }
-    }
+    float2* cand;
+    __device__ void operator()(int k, float c, float tau, const TreeVerts&, int) { cand[k - 1] = make_float2(c, tau); }
 };
 
-__global__ void __launch_bounds__(128) pt_kernel(const __grid_constant__ PtArgs a) {
+constexpr int kPtThreads = 128;
+__global__ void __launch_bounds__(kPtThreads) pt_kernel(const __grid_constant__ PtArgs a) {
+    __shared__ float2 cand[kPtThreads * kMaxDepth];
     const FrameDev& F = a.F;
-    int ix = blockIdx.x * 16 + (threadIdx.x & 15), iy = blockIdx.y * 8 + (threadIdx.x >> 4);
-    if (ix >= F.W || iy >= F.H) return;
-    const int pix = iy * F.W + ix;
+    const ParamsDev& P = a.P;
+    const int G = a.spp < kPtThreads ? a.spp : kPtThreads, ppb = kPtThreads / G;
+    const int pl = (int)threadIdx.x / G, lane = (int)threadIdx.x % G;
+    const long long pix = (long long)blockIdx.x * ppb + pl;
+    const bool mine = pl < ppb && pix < (long long)F.W * F.H;
+    const int ix = mine ? (int)(pix % F.W) : 0, iy = mine ? (int)(pix / F.W) : 0;
     const int Bn = F.B > 0 ? F.B : 1;
-    float* row = a.out + (size_t)pix * Bn;
+    float* row = a.out + (size_t)(mine ? pix : 0) * Bn;
+    if (mine)
+        for (int b = lane; b < Bn; b += G) row[b] = 0.f;
     float acc = 0.f;
-    for (int b = 0; b < Bn; ++b) row[b] = 0.f;
+    const float scale = 1.0f / (float)a.spp;
+    const float glo = F.L0, ghi = F.B > 0 ? F.L0 + F.B * F.dL : F.L0 + F.dL;
     PtSink sink;
-    sink.B = F.B; sink.t0 = F.L0; sink.w = F.dL; sink.scale = 1.0f / (float)a.spp;
-    sink.row = F.B > 0 ? row : &acc;
-    float glo = F.L0, ghi = F.B > 0 ? F.L0 + F.B * F.dL : F.L0 + F.dL;
-    TreeVerts T;
-    for (int s = 0; s < a.spp; ++s) {
-        uint4 u = philox((uint32_t)pix, F.frame, (uint32_t)s, P_JITTER, a.P.seed);
-        float3 o, d;
-        primary_ray(F, ix, iy, u01(u.x), u01(u.y), o, d);
-        int tri; float b1, b2, t;
-        if (!traverse<false>(F.g, o, d, 3.0e38f, tri, b1, b2, t)) continue;
-        Surf s1 = surf_at(F.g, tri, b1, b2);
-        Domain D = make_domain_hit(&F, true, tri, b1, b2, len3(s1.p - o), F.L0, F.dL);
-        D.x0 = o;
-        trace_tree(D, a.P, (uint32_t)pix, F.frame, s, glo, ghi, T, sink);
+    sink.cand = cand + threadIdx.x * kMaxDepth;
+    for (int s0 = 0; s0 < a.spp; s0 += G) {
+        const int s = s0 + lane;
+        for (int d = 0; d < P.depth; ++d) sink.cand[d] = make_float2(0.f, 0.f);
+        if (mine && s < a.spp) {
+            uint4 u = philox((uint32_t)pix, F.frame, (uint32_t)s, P_JITTER, P.seed);
+            float3 o, d;
+            primary_ray(F, ix, iy, u01(u.x), u01(u.y), o, d);
+            int tri; float b1, b2, t;
+            if (traverse<false>(F.g, o, d, 3.0e38f, tri, b1, b2, t)) {
+                Surf s1 = surf_at(F.g, tri, b1, b2);
+                Domain D = make_domain_hit(&F, true, tri, b1, b2, len3(s1.p - o), F.L0, F.dL);
+                D.x0 = o;
+                TreeVerts T;
+                trace_tree(D, P, (uint32_t)pix, F.frame, s, glo, ghi, T, sink);
+            }
+        }
+        __syncthreads();   // the zeroed row and every sample's contributions
+        if (mine && lane == 0) {
+            const int ns = min(G, a.spp - s0);
+            for (int j = 0; j < ns; ++j)
+                for (int d = 0; d < P.depth; ++d) {
+                    const float2 c = cand[(threadIdx.x + j) * kMaxDepth + d];
+                    if (c.x == 0.f) continue;
+                    if (F.B > 0) {
+                        const float fb = floorf((c.y - F.L0) / F.dL);
+                        if (fb >= 0.f && fb < (float)F.B) row[(int)fb] += scale * c.x;
+                    } else {
+                        acc += scale * c.x;
+                    }
+                }
+        }
+        __syncthreads();
     }
-    if (F.B == 0) row[0] = acc;
+    if (mine && lane == 0 && F.B == 0) row[0] = acc;
 }
 
 // --------------------------------------------------------------------------------------------
@@ -861,7 +1059,6 @@ __global__ void laser_kernel(GeomDev g, float3 o, float3 dir, float power, Light
 // --------------------------------------------------------------------------------------------
 // host-side launchers
 // --------------------------------------------------------------------------------------------
-static inline dim3 pix_grid(int W, int H) { return dim3((W + 15) / 16, (H + 7) / 8); }
 static inline dim3 tile_grid(int W, int H, int tw, int th) { return dim3((W + tw - 1) / tw, (H + th - 1) / th); }
 
 // tile_w x tile_h pixel tiles, tile_w a power of two in [4, 32], tile_w * tile_h = 64 or 128
@@ -875,8 +1072,9 @@ cudaError_t launch_initial(const InitArgs& a, int tile_h, unsigned* err, cudaStr
     const dim3 grid = tile_grid(a.F.W, a.F.H, a.tile_w, tile_h);
     const int threads = a.tile_w * tile_h;
     if (a.F.B == 0) {
-        if (a.P.flags & kFlagEllipsoid) initial_gated_kernel<true><<<grid, threads, 0, s>>>(a);
-        else initial_gated_kernel<false><<<grid, threads, 0, s>>>(a);
+        const LaneTile t = lane_tile(a.P.n_cand);
+        if (a.P.flags & kFlagEllipsoid) initial_gated_ell_kernel<<<grid, threads, 0, s>>>(a);
+        else initial_lanes_kernel<<<tile_grid(a.F.W, a.F.H, t.w, t.h), kLaneThreads, 0, s>>>(a);
     } else {
         if (a.P.flags & kFlagEllipsoid) initial_kernel<true><<<grid, threads, 0, s>>>(a, err);
         else initial_kernel<false><<<grid, threads, 0, s>>>(a, err);
@@ -895,7 +1093,7 @@ cudaError_t launch_gbuffer_batch(const GbufArgs* A, const int* blk0, int n, int 
 }
 cudaError_t launch_initial_batch(const InitArgs* A, const int* blk0, int n, int blocks, cudaStream_t s) {
     note_launch();
-    initial_gated_batch_kernel<<<blocks, 128, 0, s>>>(A, blk0, n);
+    initial_lanes_batch_kernel<<<blocks, kLaneThreads, 0, s>>>(A, blk0, n);
     return cudaGetLastError();
 }
 
@@ -956,7 +1154,8 @@ cudaError_t launch_initial_tree_wave(const InitArgs& a, const TreeWaveDev& w, in
                          vis_blocks, s);
     if (e != cudaSuccess) return e;
     note_launch();
-    tree_select_kernel<false><<<tile_grid(a.F.W, a.F.H, a.tile_w, tile_h), a.tile_w * tile_h, 0, s>>>(a, w);
+    if (a.F.B > 0) tree_select_bins_kernel<<<((unsigned)a.F.W * (unsigned)a.F.H + 3u) / 4u, 128, 0, s>>>(a, w);
+    else tree_select_kernel<false><<<tile_grid(a.F.W, a.F.H, a.tile_w, tile_h), a.tile_w * tile_h, 0, s>>>(a, w);
     return cudaGetLastError();
 }
 
@@ -1007,7 +1206,8 @@ cudaError_t launch_splat(const SplatArgs& a, cudaStream_t s) {
 }
 cudaError_t launch_pt(const PtArgs& a, cudaStream_t s) {
     note_launch();
-    pt_kernel<<<pix_grid(a.F.W, a.F.H), 128, 0, s>>>(a);
+    const int G = a.spp < kPtThreads ? a.spp : kPtThreads, ppb = kPtThreads / G;
+    pt_kernel<<<(unsigned)(((long long)a.F.W * a.F.H + ppb - 1) / ppb), kPtThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 cudaError_t launch_laser(const GeomDev& g, float3 o, float3 d, float power, LightDev* out, cudaStream_t s) {
