@@ -40,6 +40,9 @@ cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const 
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
                                   uint32_t** prim_out, cudaStream_t s);
+cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
+                            int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut,
+                            int sms, cudaStream_t s);
 cudaError_t launch_etree(int nt, int P, const float4* tri, float4* node, cudaStream_t s);
 cudaError_t launch_refit(int n, const uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, const int* child,
                          const int* parent_int, const int* parent_leaf, uint32_t* counter, cudaStream_t s);
@@ -567,7 +570,14 @@ tof_status tof_bvh_build(tof_ctx* c, tof_scene id, const float* xf, int refit_on
         CK(launch_build_topology(S.nt, S.cent, S.bb, S.keys, S.vals, S.keys2, S.vals2, S.hist, S.child, S.parent_int,
                                  S.parent_leaf, &S.prim, s));
     }
-    CK(launch_refit(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, s));
+    const bool full = !S.built || !refit_only;
+    if (full && S.nt > 1) {
+        if (!c->sms) CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
+        CK(launch_treelets(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, S.keys2,
+                           S.vals2, S.bb + 6, c->sms, s));
+    } else {
+        CK(launch_refit(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, s));
+    }
     if (S.enode[slot]) CK(launch_etree(S.nt, S.eP, S.tri[slot], S.enode[slot], s));
     S.version[slot] = ++c->version_counter;
     S.xfh[slot] = xv;

@@ -246,8 +246,19 @@ __device__ __forceinline__ int delta(const uint32_t* __restrict__ k, int n, int 
     return __clz(a ^ b);
 }
 
+// Ranges of at most kTreelet leaves whose parent's is larger are listed as treelets (cuts[r] = (first leaf,
+// leaves | kRootLast where the Karras node of the range is numbered by its last leaf), *ncut of them).
+constexpr int kTreelet = 512;
+constexpr uint32_t kRootLast = 0x80000000u;
+__device__ __forceinline__ void list_cut(int first, int last, int code, uint32_t* __restrict__ cut_a, uint32_t* __restrict__ cut_m,
+                                         uint32_t* ncut) {
+    const uint32_t r = atomicAdd(ncut, 1u);
+    cut_a[r] = (uint32_t)first;
+    cut_m[r] = (uint32_t)(last - first + 1) | (code == last && last > first ? kRootLast : 0u);
+}
 __global__ void karras_kernel(int n, const uint32_t* __restrict__ keys, int* __restrict__ child, int* __restrict__ parent_int,
-                              int* __restrict__ parent_leaf) {
+                              int* __restrict__ parent_leaf, uint32_t* __restrict__ cut_a, uint32_t* __restrict__ cut_m,
+                              uint32_t* ncut) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
     int d = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) >= 0 ? 1 : -1;
@@ -276,6 +287,13 @@ __global__ void karras_kernel(int n, const uint32_t* __restrict__ keys, int* __r
     if (left < 0) parent_leaf[~left] = i; else parent_int[left] = i;
     if (right < 0) parent_leaf[~right] = i; else parent_int[right] = i;
     if (i == 0) parent_int[0] = -1;
+    const int first = min(i, j), last = max(i, j);
+    if (last - first + 1 > kTreelet) {
+        if (g - first + 1 <= kTreelet) list_cut(first, g, left, cut_a, cut_m, ncut);
+        if (last - g <= kTreelet) list_cut(g + 1, last, right, cut_a, cut_m, ncut);
+    } else if (i == 0) {
+        list_cut(0, n - 1, 0, cut_a, cut_m, ncut);
+    }
 }
 
 struct Box { float lo[3], hi[3]; };
@@ -332,6 +350,342 @@ __global__ void refit_kernel(int n, const uint32_t* __restrict__ prim, const flo
         N[2] = make_float4(b[0].lo[2], b[0].hi[2], b[1].lo[2], b[1].hi[2]);
         N[3] = make_float4(__int_as_float(c[0]), __int_as_float(c[1]), 0.f, 0.f);
         p = parent_int[p];
+    }
+}
+
+// ---- surface-area treelets ---------------------------------------------------------------------
+// A Morton-code hierarchy splits space in halves whatever lies in them: rays visit 1.25 to 2 times the
+// nodes that they do in one split by the surface area heuristic (host model, visits per ray: terrain with
+// spheres 36 against 29 for bounce rays and 40 against 31 for visibility, full top-down SAH 27 and 29;
+// confocal scan 18 against 11.5; box 13.6 against 7.2).  So the Morton order is cut into ranges of at most
+// 512 leaves, each is built anew top-down by one block -- every split of the sorted orders tried, all nodes
+// of a level at once, the triangles' boxes in shared memory -- and one block builds the levels above over
+// the ranges' roots in the same way (up to 1024 of them; more keep the Morton hierarchy there).  Bound by
+// the issue of the running-box shuffles over about 14 levels; ranges of 256 and 128 leaves: 121 and 205 us
+// for both kernels instead of 126.  Frames with the build: 512 x 512 2.73 -> 2.63 ms, 1024 x 1024 11.1 ->
+// 10.4; static scenes: path tracing 608 -> 446 us, 128 x 128 allocation-free 428 -> 361 us.
+// It writes boxes, children and leaf order itself, so a full build needs no bottom-up pass over all levels.
+// Node numbers: a range [a, a + m) owns the m - 1 numbers of its Karras nodes; its root keeps the Karras
+// root's, so that a Karras parent's link to it stays right.
+template <int N>
+struct Sweep {
+    float box[6][N];             // lo, hi of item i
+    float suf[6][N];             // box of positions p .. end of segment
+    unsigned long long best[N];  // per segment start: (cost, distance from the middle, position)
+    unsigned long long keys[N];
+    uint16_t ord[3][N];          // items sorted along each axis within their segment
+    uint16_t seg0[N], seg1[N];   // segment [seg0, seg1) of a position
+    uint16_t pre[3][N];          // items of the left side before a position of each order
+    uint8_t side[N], axis[N];    // of an item; of a segment's split, by its start
+    int link[N];                 // per segment start: 2 * parent + side of the node to come, or -1
+    float wup[3][N / 32][6], wdown[3][N / 32][6];
+    int wcnt[3][N / 32];
+    int root_split, open;        // open: leaves of the longest segment not yet split up
+};
+__device__ __forceinline__ float half_area(const float b[6]) {
+    const float x = b[3] - b[0], y = b[4] - b[1], z = b[5] - b[2];
+    return x * y + y * z + z * x;
+}
+__device__ __forceinline__ void grow(float b[6], const float o[6]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { b[k] = fminf(b[k], o[k]); b[3 + k] = fmaxf(b[3 + k], o[3 + k]); }
+}
+// barrier of the block's first nt threads (a multiple of 32): a range shorter than the block's threads
+// leaves the other warps out
+__device__ __forceinline__ void group_sync(int nt) { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); }
+// within its warp, the running box of a position's segment [s, e): from its start up to the position (kUp) or
+// from the position to its end
+template <bool kUp>
+__device__ __forceinline__ void run_boxes(int longest, int p, int s, int e, bool in, float b[6]) {
+    const int lane = p & 31;
+#pragma unroll 1
+    for (int o = 1; o < 32 && o < longest; o <<= 1) {
+        float n[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) n[k] = kUp ? __shfl_up_sync(0xFFFFFFFFu, b[k], o) : __shfl_down_sync(0xFFFFFFFFu, b[k], o);
+        if (in && (kUp ? lane >= o && p - o >= s : lane + o < 32 && p + o < e)) grow(b, n);
+    }
+}
+
+// Builds the hierarchy of items 0 .. m - 1 (m >= 2, boxes in S.box) with N threads.  number(split,
+// root_split) is the node that splits after position `split`; leaf(position, item) the child code of one item;
+// up(code, node) records a child's parent.  Levels from kMaxSweep on split in the middle, which bounds the
+// depth (coincident items).  all_axes: every split of the three orders is tried, else those of the order along
+// the segment's longest axis (a third of the work: 145 -> 77 us for 66k triangles, visits per ray up 2 %; a
+// scene of one range tries all, 12 % fewer visits in the 332-triangle box).
+constexpr int kMaxSweep = 16;
+template <int N, class Number, class Leaf, class Up>
+__device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, bool all_axes, float4* __restrict__ nodes, int* __restrict__ child, Number number, Leaf leaf,
+                                            Up up) {
+    const int p = threadIdx.x;
+    const int nt = (m + 31) & ~31;
+    if (p >= nt) return;
+    int pow2 = 2;
+    while (pow2 < m) pow2 <<= 1;
+    for (int ax = 0; ax < 3; ++ax) {
+        // centre, then item: an order of all items (bitonic sort; padding sorts last)
+        for (int i = p; i < pow2; i += nt) {
+            uint32_t c = 0xFFFFFFFFu;
+            if (i < m) c = fenc(S.box[ax][i] + S.box[3 + ax][i]);
+            S.keys[i] = ((unsigned long long)c << 16) | (uint32_t)(i < m ? i : 0xFFFF);
+        }
+        group_sync(nt);
+        for (int k = 2; k <= pow2; k <<= 1)
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int i = p; i < pow2 / 2; i += nt) {
+                    const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1)), hi = lo | j;
+                    const unsigned long long a = S.keys[lo], b = S.keys[hi];
+                    if ((a > b) == ((lo & k) == 0)) { S.keys[lo] = b; S.keys[hi] = a; }
+                }
+                group_sync(nt);
+            }
+        if (p < m) S.ord[ax][p] = (uint16_t)(S.keys[p] & 0xFFFFu);
+        group_sync(nt);
+    }
+    if (p < m) { S.seg0[p] = 0; S.seg1[p] = (uint16_t)m; }
+    if (p == 0) { S.link[0] = -1; S.root_split = -1; S.open = m; }
+    group_sync(nt);
+    for (int level = 0;; ++level) {
+        const bool have = p < m;
+        const int s = have ? S.seg0[p] : 0, e = have ? S.seg1[p] : 0;
+        const bool in = have && e - s > 1;   // an open segment
+        if (in && p == s) S.best[s] = ~0ull;
+        const int longest = S.open;   // leaves of the longest open segment
+        group_sync(nt);
+        if (p == 0) S.open = 0;
+        float L[6], R[6], bestc = 3.4e38f;
+        int bax = -1, longaxis = 0;
+        if (!all_axes && in) {
+            float ext = -1.0f;
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                const int i0 = S.ord[ax][s], i1 = S.ord[ax][e - 1];
+                const float x = (S.box[ax][i1] + S.box[3 + ax][i1]) - (S.box[ax][i0] + S.box[3 + ax][i0]);
+                if (x > ext) { ext = x; longaxis = ax; }
+            }
+        }
+        const bool any = __any_sync(0xFFFFFFFFu, in);
+#pragma unroll 1
+        for (int t = 0; t < (all_axes ? 3 : 1); ++t) {
+            const int ax = all_axes ? t : longaxis;
+            if (!any) {   // no open segment in this warp
+                group_sync(nt);
+                group_sync(nt);
+                continue;
+            }
+            const int item = in ? S.ord[ax][p] : 0;
+            float b[6], f[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) b[k] = f[k] = S.box[k][item];
+            run_boxes<true>(longest, p, s, e, in, f);
+            run_boxes<false>(longest, p, s, e, in, b);
+            // across warps: a segment's part in each warp it reaches over
+            if ((p & 31) == 31)
+#pragma unroll
+                for (int k = 0; k < 6; ++k) S.wup[t][p >> 5][k] = f[k];
+            if ((p & 31) == 0)
+#pragma unroll
+                for (int k = 0; k < 6; ++k) S.wdown[t][p >> 5][k] = b[k];
+            group_sync(nt);
+            if (in) {
+                for (int v = (p >> 5) - 1; v >= 0 && 32 * v + 31 >= s; --v) grow(f, S.wup[t][v]);
+                for (int v = (p >> 5) + 1; 32 * v < e; ++v) grow(b, S.wdown[t][v]);
+            }
+            if (have)
+#pragma unroll
+                for (int k = 0; k < 6; ++k) S.suf[k][p] = b[k];
+            group_sync(nt);
+            if (in && p + 1 < e) {
+                float r[6];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) r[k] = S.suf[k][p + 1];
+                const float c = level >= kMaxSweep ? 0.f : half_area(f) * (float)(p + 1 - s) + half_area(r) * (float)(e - 1 - p);
+                if (bax < 0 || c < bestc) {
+                    bestc = c; bax = ax;
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) { L[k] = f[k]; R[k] = r[k]; }
+                }
+            }
+        }
+        const uint32_t mid = (uint32_t)abs(2 * (p + 1 - s) - (e - s));
+        const unsigned long long key = ((unsigned long long)__float_as_uint(bestc) << 32) | (mid << 16) | (uint32_t)p;
+        if (in && bax >= 0) atomicMin(&S.best[s], key);
+        group_sync(nt);
+        const int cut = in ? (int)(S.best[s] & 0xFFFFu) : 0;   // the segment splits after this position
+        const bool winner = in && p == cut;
+        if (winner) {
+            if (level == 0) S.root_split = p;
+            const int id = number(p, level == 0 ? p : S.root_split);
+            nodes[4 * (size_t)id] = make_float4(L[0], L[3], L[1], L[4]);
+            nodes[4 * (size_t)id + 1] = make_float4(R[0], R[3], R[1], R[4]);
+            nodes[4 * (size_t)id + 2] = make_float4(L[2], L[5], R[2], R[5]);
+            const int link = S.link[s];
+            if (link >= 0) {
+                child[link] = id;
+                reinterpret_cast<int*>(nodes + 4 * (size_t)(link >> 1) + 3)[link & 1] = id;
+                up(id, link >> 1);
+            }
+            S.link[s] = 2 * id;        // an open left part keeps the start
+            S.link[p + 1] = 2 * id + 1;
+            S.axis[s] = (uint8_t)bax;
+            const int longer = max(p + 1 - s, e - 1 - p);
+            if (longer > 1) atomicMax(&S.open, longer);
+        }
+        group_sync(nt);
+        if (in) S.side[S.ord[S.axis[s]][p]] = p > cut;   // items up to the cut in the winning order go left
+        group_sync(nt);
+        // stable partition of the three orders
+        int item[3], before[3];
+        unsigned left = 0u;
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            item[ax] = in ? S.ord[ax][p] : 0;
+            const bool l = in && S.side[item[ax]] == 0;
+            const unsigned bal = __ballot_sync(0xFFFFFFFFu, l);
+            if (l) left |= 1u << ax;
+            if ((p & 31) == 0) S.wcnt[ax][p >> 5] = __popc(bal);
+            before[ax] = __popc(bal & ((1u << (p & 31)) - 1u));
+        }
+        group_sync(nt);
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            for (int v = 0; v < (p >> 5); ++v) before[ax] += S.wcnt[ax][v];
+            S.pre[ax][p] = (uint16_t)before[ax];
+        }
+        group_sync(nt);
+        if (in)
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                const int l = before[ax] - S.pre[ax][s];   // of the left side before this position
+                S.ord[ax][(left >> ax) & 1u ? s + l : cut + 1 + (p - s) - l] = (uint16_t)item[ax];
+            }
+        group_sync(nt);
+        if (in) {
+            const int ns = p <= cut ? s : cut + 1, ne = p <= cut ? cut + 1 : e;
+            S.seg0[p] = (uint16_t)ns;
+            S.seg1[p] = (uint16_t)ne;
+            if (ne - ns == 1) {   // one item left: a child of the node just written
+                const int link = S.link[p];
+                const int code = leaf(p, (int)S.ord[0][p]);
+                child[link] = code;
+                reinterpret_cast<int*>(nodes + 4 * (size_t)(link >> 1) + 3)[link & 1] = code;
+                up(code, link >> 1);
+            }
+        }
+        group_sync(nt);
+        if (!S.open) break;
+        group_sync(nt);
+    }
+}
+
+__global__ void __launch_bounds__(kTreelet) treelet_kernel(int n, uint32_t* __restrict__ prim, const float4* __restrict__ tri,
+                                                           float4* __restrict__ leaves, float4* __restrict__ nodes, int* __restrict__ child,
+                                                           int* __restrict__ parent_int, int* __restrict__ parent_leaf,
+                                                           const uint32_t* __restrict__ cut_a, const uint32_t* __restrict__ cut_m,
+                                                           const uint32_t* __restrict__ ncut) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    Sweep<kTreelet>& S = *reinterpret_cast<Sweep<kTreelet>*>(sm);
+    const int p = threadIdx.x;
+    const uint32_t R = *ncut;
+    for (uint32_t r = blockIdx.x; r < R; r += gridDim.x) {
+        const int a = (int)cut_a[r], m = (int)(cut_m[r] & ~kRootLast);
+        const bool last = (cut_m[r] & kRootLast) != 0u;
+        const int t = p < m ? (int)prim[a + p] : 0;   // item p's triangle
+        if (p < m) {
+            const Box b = tri_box(tri, t);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { S.box[k][p] = b.lo[k]; S.box[3 + k][p] = b.hi[k]; }
+        }
+        __syncthreads();
+        int pos = p;   // item p's leaf within the range
+        if (m > 1) {
+            // numbers a .. a + m - 1 without the end that is not the root's
+            const int base = last ? a + 1 : a, root = last ? a + m - 1 : a, at_root = root - base;
+            sweep_build<kTreelet>(
+                S, m, R == 1u, nodes, child,
+                [=](int split, int rs) { return split == rs ? root : split == at_root ? base + rs : base + split; },
+                [=](int q, int) { return ~(a + q); },
+                [=](int code, int node) {
+                    if (code < 0) parent_leaf[~code] = node;
+                    else parent_int[code] = node;
+                });
+            if (p < m) S.pre[0][S.ord[0][p]] = (uint16_t)p;
+            __syncthreads();
+            if (p < m) pos = S.pre[0][p];
+        }
+        if (p < m) {
+            const size_t l = (size_t)(a + pos);
+            prim[l] = (uint32_t)t;
+            const float4 v = tri[3 * (size_t)t];
+            leaves[3 * l] = make_float4(v.x, v.y, v.z, __int_as_float(t));
+            leaves[3 * l + 1] = tri[3 * (size_t)t + 1];
+            leaves[3 * l + 2] = tri[3 * (size_t)t + 2];
+        }
+        __syncthreads();
+    }
+}
+
+// the levels above the treelets, one block
+constexpr int kTopItems = 1024;
+__global__ void __launch_bounds__(kTopItems) treelet_top_kernel(int n, const uint32_t* __restrict__ prim, const float4* __restrict__ tri,
+                                                                float4* nodes, int* __restrict__ child, int* parent_int, int* parent_leaf,
+                                                                uint32_t* counter, const uint32_t* __restrict__ cut_a,
+                                                                const uint32_t* __restrict__ cut_m, const uint32_t* __restrict__ ncut) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    Sweep<kTopItems>& S = *reinterpret_cast<Sweep<kTopItems>*>(sm);
+    __shared__ int s_no_slot, s_slot0;   // the item without a free number; the item whose free number is 0
+    const int p = threadIdx.x;
+    const int R = (int)*ncut;
+    if (R == 1) return;
+    if (R <= kTopItems) {
+        if (p < R) {
+            const int a = (int)cut_a[p], m = (int)(cut_m[p] & ~kRootLast);
+            const bool last = (cut_m[p] & kRootLast) != 0u;
+            const Box b = m == 1 ? tri_box(tri, (int)prim[a]) : node_box(nodes + 4 * (size_t)(last ? a + m - 1 : a));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { S.box[k][p] = b.lo[k]; S.box[3 + k][p] = b.hi[k]; }
+            const int slot = last ? a : a + m - 1;   // the number of the range that none of its nodes has
+            if (slot == n - 1) s_no_slot = p;
+            if (slot == 0) s_slot0 = p;
+        }
+        __syncthreads();
+        const int none = s_no_slot, zero = s_slot0;
+        // R - 1 splits onto the R - 1 free numbers, the root's being 0
+        auto slot_item = [=](int split) { return split == none ? R - 1 : split; };
+        auto slot_of = [=](int item) { return (cut_m[item] & kRootLast) ? (int)cut_a[item] : (int)(cut_a[item] + (cut_m[item] & ~kRootLast)) - 1; };
+        const int zero_split = zero == R - 1 ? none : zero;
+        sweep_build<kTopItems>(
+            S, R, false, nodes, child,
+            [=](int split, int rs) { return split == rs ? 0 : slot_of(slot_item(split == zero_split ? rs : split)); },
+            [=](int, int item) {
+                const int a = (int)cut_a[item], m = (int)(cut_m[item] & ~kRootLast);
+                return m == 1 ? ~a : (cut_m[item] & kRootLast) ? a + m - 1 : a;
+            },
+            [=](int code, int node) {
+                if (code < 0) parent_leaf[~code] = node;
+                else parent_int[code] = node;
+            });
+        return;
+    }
+    // too many: the Morton hierarchy's own nodes above the treelets, bottom-up as in refit_kernel
+    for (int i = p; i < n - 1; i += kTopItems) counter[i] = 0u;
+    __syncthreads();
+    for (int r = p; r < R; r += kTopItems) {
+        const int a = (int)cut_a[r], m = (int)(cut_m[r] & ~kRootLast);
+        int q = m == 1 ? parent_leaf[a] : parent_int[(cut_m[r] & kRootLast) ? a + m - 1 : a];
+        int guard = n;
+        while (q >= 0 && --guard >= 0) {
+            if (arrive_acq_rel(&counter[q]) == 0u) break;
+            const int c[2] = {child[2 * q], child[2 * q + 1]};
+            Box b[2];
+            for (int k = 0; k < 2; ++k) b[k] = c[k] < 0 ? tri_box(tri, (int)prim[~c[k]]) : node_box(nodes + 4 * (size_t)c[k]);
+            float4* N = nodes + 4 * (size_t)q;
+            N[0] = make_float4(b[0].lo[0], b[0].hi[0], b[0].lo[1], b[0].hi[1]);
+            N[1] = make_float4(b[1].lo[0], b[1].hi[0], b[1].lo[1], b[1].hi[1]);
+            N[2] = make_float4(b[0].lo[2], b[0].hi[2], b[1].lo[2], b[1].hi[2]);
+            N[3] = make_float4(__int_as_float(c[0]), __int_as_float(c[1]), 0.f, 0.f);
+            q = parent_int[q];
+        }
     }
 }
 
@@ -411,7 +765,7 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
                                   uint32_t** prim_out, cudaStream_t s) {
     // centroid bounds start empty: encoded minima at 0xFFFFFFFF, maxima at 0
     cudaError_t e = cudaMemsetAsync(bb, 0xFF, 3 * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(bb + 3, 0, 3 * sizeof(uint32_t), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(bb + 3, 0, 4 * sizeof(uint32_t), s);   // and the number of treelets
     if (e != cudaSuccess) return e;
     note_launch();
     bounds_kernel<<<min(1024u, blocks(n, 256)), 256, 0, s>>>(n, cent, bb);
@@ -444,7 +798,7 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
         note_launch();
         e = cudaLaunchCooperativeKernel((const void*)radix_sort_coop_kernel, dim3(ntiles), dim3(256), args, 0, s);
         if (e != cudaSuccess) return e;
-        if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf); }
+        if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
         *prim_out = vi;
         return cudaGetLastError();
     }
@@ -459,8 +813,31 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
         t = vi; vi = vo; vo = t;
     }
     // after 4 passes the sorted keys / prims are back in keys / vals
-    if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf); }
+    if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
     *prim_out = vi;
+    return cudaGetLastError();
+}
+
+// boxes, leaf records and the treelets' topology of a full build (n > 1), after launch_build_topology
+cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
+                            int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut,
+                            int sms, cudaStream_t s) {
+    static std::atomic<bool> sized[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !sized[dev].load()) {
+        cudaError_t e = cudaFuncSetAttribute(treelet_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTreelet>));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(treelet_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTopItems>));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) sized[dev].store(true);
+    }
+    // ranges hold at least a few leaves each, mostly hundreds: a block takes several where there are many
+    const int grid = min((int)blocks(n, 64), 4 * sms);
+    note_launch(2);
+    treelet_kernel<<<grid, kTreelet, sizeof(Sweep<kTreelet>), s>>>(n, prim, tri, leaf, nodes, child, parent_int, parent_leaf, cut_a, cut_m, ncut);
+    treelet_top_kernel<<<1, kTopItems, sizeof(Sweep<kTopItems>), s>>>(n, prim, tri, nodes, child, parent_int, parent_leaf, counter, cut_a,
+                                                                      cut_m, ncut);
     return cudaGetLastError();
 }
 
