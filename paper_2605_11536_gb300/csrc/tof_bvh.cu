@@ -166,55 +166,70 @@ __global__ void __launch_bounds__(256) radix_scatter_kernel(const uint32_t* __re
     }
 }
 
-// The same four passes in one cooperative launch of one block per tile (all resident): per pass
-// the tile histograms, a grid-wide sync, each block's digit offsets -- the digit totals' exclusive
+// The same four passes in one cooperative launch of one block per tile of kCoopTile keys (all resident): per
+// pass the tile histograms, a grid-wide sync, each block's digit offsets -- the digit totals' exclusive
 // scan plus the digit's count in the earlier tiles, the global scan above restated per block --
 // the same stable scatter, and a grid-wide sync.  Sorted keys and values are those of the
-// separate launches (after four passes back in k0 / v0).
+// separate launches (after four passes back in k0 / v0).  Bound by the latency of its barriers and
+// dependent steps: a tile of 512 keys has two ranking rounds a pass where one of 2048 has eight, and its
+// keys stay in registers from the histogram to the scatter; more than kCoopTiles tiles take 2048, since each
+// block reads every tile's histogram.
+template <int kCoopTile>
 __global__ void __launch_bounds__(256) radix_sort_coop_kernel(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int n,
                                                               uint32_t* __restrict__ hist, int ntiles) {
     namespace cg = cooperative_groups;
     cg::grid_group grid = cg::this_grid();
+    constexpr int kRounds = kCoopTile / 256;
     __shared__ uint32_t h[256];
     __shared__ uint32_t base[256];
     __shared__ uint32_t wc[8][256];
+    __shared__ uint32_t wsum[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
+    const int t0 = blockIdx.x * kCoopTile;
     for (int shift = 0; shift < 32; shift += 8) {
         h[tid] = 0u;
         __syncthreads();
-        const int t0 = blockIdx.x * kTile;
-        for (int i = tid; i < kTile; i += 256) {
-            const int g = t0 + i;
-            if (g < n) atomicAdd(&h[(__ldcg(&ki[g]) >> shift) & 255u], 1u);
+        uint32_t key[kRounds];
+#pragma unroll
+        for (int r = 0; r < kRounds; ++r) {
+            const int g = t0 + r * 256 + tid;
+            key[r] = g < n ? __ldcg(&ki[g]) : 0u;
+            if (g < n) atomicAdd(&h[(key[r] >> shift) & 255u], 1u);
         }
         __syncthreads();
-        hist[tid * ntiles + blockIdx.x] = h[tid];
+        hist[blockIdx.x * 256 + tid] = h[tid];
         __threadfence();
         grid.sync();
         uint32_t tot = 0u, before = 0u;
+#pragma unroll 8
         for (int t = 0; t < ntiles; ++t) {
-            const uint32_t c = __ldcg(&hist[tid * ntiles + t]);
+            const uint32_t c = __ldcg(&hist[t * 256 + tid]);
             tot += c;
             if (t < (int)blockIdx.x) before += c;
         }
-        h[tid] = tot;
-        __syncthreads();
-        for (int off = 1; off < 256; off <<= 1) {   // inclusive scan of the digit totals
-            const uint32_t v = tid >= off ? h[tid - off] : 0u;
-            __syncthreads();
-            h[tid] += v;
-            __syncthreads();
+        // exclusive scan of the digit totals
+        uint32_t incl = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += v;
         }
-        base[tid] = h[tid] - tot + before;
-        for (int r = 0; r < kTile / 256; ++r) {
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        uint32_t low = 0u;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) low += w < warp ? wsum[w] : 0u;
+        base[tid] = low + incl - tot + before;
+#pragma unroll
+        for (int r = 0; r < kRounds; ++r) {
             for (int k = 0; k < 8; ++k) wc[k][tid] = 0u;
             __syncthreads();
             const int i = t0 + r * 256 + tid;
             const bool valid = i < n;
-            const uint32_t key = valid ? __ldcg(&ki[i]) : 0u;
-            const uint32_t dg = (key >> shift) & 255u;
+            const uint32_t val = valid ? __ldcg(&vi[i]) : 0u;
+            const uint32_t dg = (key[r] >> shift) & 255u;
             const uint32_t peers = __match_any_sync(0xFFFFFFFFu, valid ? dg : 256u + (uint32_t)lane);
             const uint32_t rank = __popc(peers & lt);
             if (valid && rank == 0) wc[warp][dg] = __popc(peers);
@@ -222,14 +237,16 @@ __global__ void __launch_bounds__(256) radix_sort_coop_kernel(uint32_t* k0, uint
             if (valid) {
                 uint32_t off = base[dg] + rank;
                 for (int w = 0; w < warp; ++w) off += wc[w][dg];
-                ko[off] = key;
-                vo[off] = __ldcg(&vi[i]);
+                ko[off] = key[r];
+                vo[off] = val;
             }
-            __syncthreads();
-            uint32_t add = 0;
-            for (int w = 0; w < 8; ++w) add += wc[w][tid];
-            base[tid] += add;
-            __syncthreads();
+            if (r + 1 < kRounds) {
+                __syncthreads();
+                uint32_t add = 0;
+                for (int w = 0; w < 8; ++w) add += wc[w][tid];
+                base[tid] += add;
+                __syncthreads();
+            }
         }
         __threadfence();
         grid.sync();
@@ -762,7 +779,7 @@ cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const 
 // full build of the hierarchy (prim order, children, parents) from the centroids
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
-                                  uint32_t** prim_out, cudaStream_t s) {
+                                  uint32_t** prim_out, float4* scratch, cudaStream_t s) {
     // centroid bounds start empty: encoded minima at 0xFFFFFFFF, maxima at 0
     cudaError_t e = cudaMemsetAsync(bb, 0xFF, 3 * sizeof(uint32_t), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(bb + 3, 0, 4 * sizeof(uint32_t), s);   // and the number of treelets
@@ -785,18 +802,33 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
             int sms = 0, per = 0, coop = 0;
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, radix_sort_coop_kernel, 256, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, radix_sort_coop_kernel<2048>, 256, 0);
             cudaGetLastError();
             coop_blocks[dev].store(coop ? sms * per : 0);
             coop_known[dev].store(true);
         }
         coop_cap = coop_blocks[dev].load();
     }
+    // tiles of 512 keys up to kCoopTiles of them; their histograms (2 B a key) lie in the centroids' memory, which
+    // the Morton codes were the last to read
+    constexpr int kCoopTiles = 192;
+    const int small = (n + 511) / 512;
+    if (small <= kCoopTiles && small <= coop_cap && n >= 512) {
+        int nn = n, nt = small;
+        uint32_t* hh = reinterpret_cast<uint32_t*>(scratch);
+        void* args[] = {&ki, &vi, &ko, &vo, &nn, &hh, &nt};
+        note_launch();
+        e = cudaLaunchCooperativeKernel((const void*)radix_sort_coop_kernel<512>, dim3(small), dim3(256), args, 0, s);
+        if (e != cudaSuccess) return e;
+        if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
+        *prim_out = vi;
+        return cudaGetLastError();
+    }
     if (ntiles <= coop_cap) {
         int nn = n, nt = ntiles;
         void* args[] = {&ki, &vi, &ko, &vo, &nn, &hist, &nt};
         note_launch();
-        e = cudaLaunchCooperativeKernel((const void*)radix_sort_coop_kernel, dim3(ntiles), dim3(256), args, 0, s);
+        e = cudaLaunchCooperativeKernel((const void*)radix_sort_coop_kernel<2048>, dim3(ntiles), dim3(256), args, 0, s);
         if (e != cudaSuccess) return e;
         if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
         *prim_out = vi;
