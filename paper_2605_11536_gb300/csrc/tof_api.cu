@@ -50,7 +50,7 @@ cudaError_t launch_gbuffer_batch(const GbufArgs* A, const int* blk0, int n, int 
 int initial_lanes_blocks(int W, int H, int n_cand);
 cudaError_t launch_initial_batch(const InitArgs* A, const int* blk0, int n, int blocks, cudaStream_t s);
 cudaError_t launch_reuse_batch(const ReuseJob* J, int n, const int* blk_slots, int nblk_slots, const int* blk_units,
-                               int nblk_units, int persist_blocks, int vis_blocks, cudaStream_t s);
+                               int nblk_units, int persist_blocks, int shift_blocks, int vis_blocks, cudaStream_t s);
 }  // namespace tof
 
 using namespace tof;
@@ -158,7 +158,7 @@ struct tof_ctx {
     unsigned* d_err = nullptr;   // device error word (kErr* bits), set by kernels
     unsigned* h_err = nullptr;   // pinned host mirror of it, copied after every render on its stream
     float* d_scratch = nullptr;  // laser spot of plain PT renders
-    int persist_blocks = 0;      // resident blocks of the merge and the batched reuse stages (all SMs)
+    int persist_blocks = 0;      // resident blocks of the merge and the emission (all SMs)
     int shift_blocks = 0;        // resident blocks of the shift kernels (all SMs)
     int ell_blocks = 0;          // resident blocks of the ellipsoidal placement kernel (all SMs)
     int hit_blocks = 0;          // resident blocks of the wavefront closest-hit kernel (all SMs)
@@ -1289,7 +1289,8 @@ static cudaError_t staged_launch(tof_ctx* c, const StagedGroup& G, unsigned char
     }
     for (size_t k = 0; k < G.rec.pass.size() && e == cudaSuccess; ++k)
         e = launch_reuse_batch((const ReuseJob*)(d + G.o_p[k]), (int)G.rec.pass[k].size(), (const int*)(d + G.o_s[k]),
-                               G.bs[k].back(), (const int*)(d + G.o_u[k]), G.bu[k].back(), c->persist_blocks, c->vis_blocks, q);
+                               G.bs[k].back(), (const int*)(d + G.o_u[k]), G.bu[k].back(), c->persist_blocks, c->shift_blocks,
+                               c->vis_blocks, q);
     return e;
 }
 

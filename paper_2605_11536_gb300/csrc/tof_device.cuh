@@ -411,7 +411,8 @@ static __device__ __forceinline__ bool trav_round(const float4* __restrict__ nod
 }
 
 // The n rays of a queue, traced by a persistent grid: Q::load(i, o, d, tmax) reads ray i, Q::done(ray)
-// takes its answer.  kAny: whether anything is hit; else the closest hit.
+// takes its answer.  kAny: whether anything is hit; else the closest hit.  `warp`: the warp's place among the
+// grid's (its share of a short queue).
 //
 // Bound by issue (the min / max of the slab tests and the divergence of a warp's rays), the L1's data path
 // (node_test) and, with few rays, by the longest ray's chain of node visits.
@@ -427,8 +428,10 @@ static __device__ __forceinline__ bool trav_round(const float4* __restrict__ nod
 // kernels 826 -> 710 us; 1024 x 1024 12.0 -> 11.2 ms.
 constexpr int kQueueRun = 8;
 constexpr uint32_t kAloneRays = 4;
+// the warp's place in its grid
+static __device__ __forceinline__ uint32_t grid_warp() { return blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); }
 template <bool kAny, class Q>
-static __device__ __forceinline__ void trace_queue(const GeomDev& g, uint32_t n, uint32_t* fetch, uint32_t min_rays, Q& q) {
+static __device__ __forceinline__ void trace_queue(const GeomDev& g, uint32_t n, uint32_t* fetch, uint32_t min_rays, uint32_t warp, Q& q) {
     const float4* __restrict__ nodes = g.nodes;
     const float4* __restrict__ leaf = g.leaf;
     const int nt = g.nt;
@@ -444,7 +447,7 @@ static __device__ __forceinline__ void trace_queue(const GeomDev& g, uint32_t n,
     uint32_t pool = 0, pool_end = 0;
     bool drained = n <= warps * chunk;
     if (drained) {
-        pool = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * chunk;
+        pool = warp * chunk;
         pool_end = min(pool + chunk, n);
         if (pool >= n) return;
     }

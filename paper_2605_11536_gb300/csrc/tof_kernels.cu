@@ -816,7 +816,7 @@ __global__ void __launch_bounds__(128, 8) tw_hit_kernel(const GeomDev gref, cons
                                                      uint32_t cap, uint32_t* fetch, float4* __restrict__ hits) {
     HitQueue q;
     q.rays = rays; q.hits = hits; q.cur = 0;
-    trace_queue<false>(gref, min(*counter, cap), fetch, kAloneRays, q);
+    trace_queue<false>(gref, min(*counter, cap), fetch, kAloneRays, grid_warp(), q);
 }
 
 // the hits of the round towards vertex d: one thread per ray

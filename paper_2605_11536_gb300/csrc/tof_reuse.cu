@@ -292,7 +292,7 @@ struct Later {
 };
 
 template <bool kWalk, bool kSame>
-__device__ __forceinline__ void shift_fwd_body(const ReuseArgs& a, const WaveDev& w) {
+__device__ __forceinline__ void shift_fwd_body(const ReuseArgs& a, const WaveDev& w, uint32_t warp) {
     __shared__ uint32_t later_list[4][64];
     ShiftStats st = {0, 0, 0, 0, 0};
     const uint32_t ntask = min(w.counters[1], (uint32_t)w.cap_units * (uint32_t)(w.slots - 1));
@@ -301,7 +301,7 @@ __device__ __forceinline__ void shift_fwd_body(const ReuseArgs& a, const WaveDev
     Later later;
     later.list = later_list[threadIdx.x >> 5];
     later.n = 0;
-    for (uint32_t t0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);; t0 += gridDim.x * blockDim.x) {
+    for (uint32_t t0 = warp * 32u;; t0 += gridDim.x * blockDim.x) {
         const bool more = t0 < ntask;
         if (!more || later.n >= 32) {
             if (lane < min(later.n, 32)) {
@@ -363,7 +363,7 @@ __device__ __forceinline__ void shift_fwd_body(const ReuseArgs& a, const WaveDev
 }
 template <bool kWalk, bool kSame>
 __global__ void __launch_bounds__(128, kShiftBlocks) shift_fwd_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w) {
-    shift_fwd_body<kWalk, kSame>(a, w);
+    shift_fwd_body<kWalk, kSame>(a, w, grid_warp());
 }
 
 // --------------------------------------------------------------------------------------------
@@ -390,13 +390,13 @@ struct SegQueue {
 
 __device__ __forceinline__ void vis_body(const GeomDev& gref, const float4* __restrict__ rays, const uint32_t* counter,
                                          uint32_t cap, uint32_t* fetch, float* target, StatsDev* stats, int stat, int ray_stat,
-                                         uint32_t min_rays) {
+                                         uint32_t min_rays, uint32_t warp) {
     const uint32_t n = min(*counter, cap);
     if (stats && ray_stat >= 0 && blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(&stats->v[ray_stat], (unsigned long long)n);
     const int lane = threadIdx.x & 31;
     SegQueue q;
     q.rays = rays; q.target = target; q.lost = 0; q.tgt = 0;
-    trace_queue<true>(gref, n, fetch, min_rays, q);
+    trace_queue<true>(gref, n, fetch, min_rays, warp, q);
     const unsigned long long lost = q.lost;
     if (stats && stat >= 0) {
         unsigned long long x = lost;
@@ -407,7 +407,7 @@ __device__ __forceinline__ void vis_body(const GeomDev& gref, const float4* __re
 __global__ void __launch_bounds__(128, 8) vis_kernel(const GeomDev g, const float4* __restrict__ rays, const uint32_t* counter,
                                                   uint32_t cap, uint32_t* fetch, float* target, StatsDev* stats, int stat,
                                                   int ray_stat) {
-    vis_body(g, rays, counter, cap, fetch, target, stats, stat, ray_stat, kAloneRays);
+    vis_body(g, rays, counter, cap, fetch, target, stats, stat, ray_stat, kAloneRays, grid_warp());
 }
 
 // --------------------------------------------------------------------------------------------
@@ -415,11 +415,11 @@ __global__ void __launch_bounds__(128, 8) vis_kernel(const GeomDev g, const floa
 // the other reused domains (pairwise MIS needs none: it pairs the canonical domain with each
 // reused one)
 // --------------------------------------------------------------------------------------------
-__device__ __forceinline__ void emit_inv_body(const ReuseArgs& a, const WaveDev& w) {
+__device__ __forceinline__ void emit_inv_body(const ReuseArgs& a, const WaveDev& w, uint32_t warp) {
     const uint32_t ntask = min(w.counters[1], (uint32_t)w.cap_units * (uint32_t)(w.slots - 1));
     const int S = w.slots;
     const bool pairwise = (a.P.flags & kFlagPairwiseMis) != 0u;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < ntask; t += gridDim.x * blockDim.x) {
+    for (uint32_t t = warp * 32u + (threadIdx.x & 31u); t < ntask; t += gridDim.x * blockDim.x) {
         uint32_t task = w.fwd[t];
         uint32_t u = task >> 4;
         int s = (int)(task & 15u);
@@ -436,7 +436,7 @@ __device__ __forceinline__ void emit_inv_body(const ReuseArgs& a, const WaveDev&
     }
 }
 __global__ void __launch_bounds__(128) emit_inv_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w) {
-    emit_inv_body(a, w);
+    emit_inv_body(a, w, grid_warp());
 }
 
 // --------------------------------------------------------------------------------------------
@@ -478,7 +478,7 @@ __device__ __noinline__ void shift_inv_general(const ReuseArgs& a, const WaveDev
 // tasks [t0, t1) of the list; their visibility segments go to `rays` (counter rcount, capacity rcap)
 template <bool kWalk, bool kSame>
 __device__ __forceinline__ void shift_inv_body(const ReuseArgs& a, const WaveDev& w, uint32_t t0, uint32_t t1, float4* rays,
-                                               uint32_t* rcount, uint32_t rcap) {
+                                               uint32_t* rcount, uint32_t rcap, uint32_t warp) {
     __shared__ uint32_t later_list[4][64];
     const int S = w.slots;
     const int lane = threadIdx.x & 31;
@@ -486,7 +486,7 @@ __device__ __forceinline__ void shift_inv_body(const ReuseArgs& a, const WaveDev
     Later later;
     later.list = later_list[threadIdx.x >> 5];
     later.n = 0;
-    for (uint32_t tw = t0 + blockIdx.x * blockDim.x + (threadIdx.x & ~31u);; tw += gridDim.x * blockDim.x) {
+    for (uint32_t tw = t0 + warp * 32u;; tw += gridDim.x * blockDim.x) {
         const bool more = tw < t1;
         if (!more || later.n >= 32) {
             if (lane < min(later.n, 32)) shift_inv_general<kWalk>(a, w, later.list[later.n - 1 - lane], rays, rcount, rcap);
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(128, kShiftBlocks) shift_inv_kernel(const __gr
                                                           const uint32_t* lo, const uint32_t* hi, float4* rays, uint32_t* rcount,
                                                           uint32_t rcap) {
     const uint32_t cap = inv_task_cap(w);
-    shift_inv_body<kWalk, kSame>(a, w, lo ? min(*lo, cap) : 0u, min(*hi, cap), rays, rcount, rcap);
+    shift_inv_body<kWalk, kSame>(a, w, lo ? min(*lo, cap) : 0u, min(*hi, cap), rays, rcount, rcap, grid_warp());
 }
 
 // --------------------------------------------------------------------------------------------
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(128, kShiftBlocks) shift_inv_kernel(const __gr
 // same running sum and comparisons as one thread would make); the group then copies the selected
 // record plane by plane.
 // --------------------------------------------------------------------------------------------
-__device__ __forceinline__ void reuse_merge_body(const ReuseArgs& a, const WaveDev& w) {
+__device__ __forceinline__ void reuse_merge_body(const ReuseArgs& a, const WaveDev& w, uint32_t warp) {
     const uint32_t nunits = min(w.counters[0], (uint32_t)w.cap_units);
     const int S = w.slots;
     const FrameDev& C = a.cur;
@@ -571,10 +571,10 @@ __device__ __forceinline__ void reuse_merge_body(const ReuseArgs& a, const WaveD
     const int g0 = lane & ~(G - 1);               // first lane of the group
     const unsigned gmask = (G == 32 ? 0xFFFFFFFFu : ((1u << G) - 1u)) << g0;
     const uint32_t groups = gridDim.x * (blockDim.x / G);
-    const uint32_t first = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const uint32_t first = (warp * 32u + lane) / G;
     // every lane of a warp runs the same number of iterations (the group index advances by the same
     // stride for all groups of the warp), so the warp-synchronous shuffles below see full groups
-    const uint32_t warp_first = (blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / G;
+    const uint32_t warp_first = warp * 32u / G;
     for (uint32_t base = warp_first; base < nunits; base += groups) {
         const uint32_t u = first + (base - warp_first);
         const bool unit_ok = u < nunits;
@@ -714,15 +714,20 @@ __device__ __forceinline__ void reuse_merge_body(const ReuseArgs& a, const WaveD
     }
 }
 __global__ void __launch_bounds__(128) reuse_merge_kernel(const __grid_constant__ ReuseArgs a, const __grid_constant__ WaveDev w) {
-    reuse_merge_body(a, w);
+    reuse_merge_body(a, w, grid_warp());
 }
 
 // --------------------------------------------------------------------------------------------
 // a reuse pass over all instances of a batch (tof_render_batch): one launch per stage.  Per-pixel
 // stages map each block to its instance through blk0 (first block of each instance); persistent
-// stages run over the instances one after another, every block pulling its share of each instance's
+// stages run over the instances one after another, every warp pulling its share of each instance's
 // tasks (the instances are independent, so no block waits for another).  Each block copies the
 // instance's argument record to shared memory.
+// An instance is seldom as long as the grid (a 128 x 128 view lists some 20k tasks, the grid has 78k or
+// 156k lanes), so its shares start at the warp where the last instance's ended: the grid fills up evenly
+// instead of its first warps taking a share of every instance (batch of 32 views 13.99 -> 13.60 ms).  The
+// shifts' grid is what is resident at their four blocks an SM; twice that, the merge's, held back the next
+// group's kernels behind blocks with nothing to do (14.17 -> 13.55 ms; a quarter less: 13.9).
 // --------------------------------------------------------------------------------------------
 __global__ void reuse_reset_batch_kernel(const ReuseJob* __restrict__ J, int n) {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * kWaveCounters; t += gridDim.x * blockDim.x)
@@ -747,41 +752,54 @@ __global__ void __launch_bounds__(128) reuse_units_batch_kernel(const ReuseJob* 
 template <int kStage>
 __global__ void __launch_bounds__(128, kStage == 0 || kStage == 3 ? kShiftBlocks : 8) reuse_persist_batch_kernel(const ReuseJob* __restrict__ J, int n) {
     __shared__ ReuseJob s;
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    uint32_t warp = grid_warp();
     for (int j = 0; j < n; ++j) {
         __syncthreads();
         block_copy(&s, &J[j]);
         __syncthreads();
         const ReuseArgs& a = s.a;
         const WaveDev& w = s.w;
+        uint32_t ntask;
         if constexpr (kStage == 0) {
-            if (a.temporal) shift_fwd_body<false, false>(a, w);
-            else shift_fwd_body<false, true>(a, w);
-        }
-        else if constexpr (kStage == 1)
-            vis_body(a.cur.g, w.rays, &w.counters[4], w.ray_cap, &w.counters[6], w.py, a.stats, 4, a.temporal ? -1 : 8, 32u);
-        else if constexpr (kStage == 2) emit_inv_body(a, w);
-        else if constexpr (kStage == 3)
-            {
-                if (a.temporal) shift_inv_body<false, false>(a, w, 0u, min(w.counters[2], inv_task_cap(w)), w.rays, &w.counters[5], w.ray_cap);
-                else shift_inv_body<false, true>(a, w, 0u, min(w.counters[2], inv_task_cap(w)), w.rays, &w.counters[5], w.ray_cap);
-            }
-        else if constexpr (kStage == 4)
+            ntask = min(w.counters[1], (uint32_t)w.cap_units * (uint32_t)(w.slots - 1));
+            if (a.temporal) shift_fwd_body<false, false>(a, w, warp);
+            else shift_fwd_body<false, true>(a, w, warp);
+        } else if constexpr (kStage == 1) {
+            ntask = min(w.counters[4], w.ray_cap);
+            vis_body(a.cur.g, w.rays, &w.counters[4], w.ray_cap, &w.counters[6], w.py, a.stats, 4, a.temporal ? -1 : 8, 32u, warp);
+        } else if constexpr (kStage == 2) {
+            ntask = min(w.counters[1], (uint32_t)w.cap_units * (uint32_t)(w.slots - 1));
+            emit_inv_body(a, w, warp);
+        } else if constexpr (kStage == 3) {
+            ntask = min(w.counters[2], inv_task_cap(w));
+            if (a.temporal) shift_inv_body<false, false>(a, w, 0u, ntask, w.rays, &w.counters[5], w.ray_cap, warp);
+            else shift_inv_body<false, true>(a, w, 0u, ntask, w.rays, &w.counters[5], w.ray_cap, warp);
+        } else if constexpr (kStage == 4) {
+            ntask = min(w.counters[5], w.ray_cap);
             vis_body(a.temporal ? a.prev.g : a.cur.g, w.rays, &w.counters[5], w.ray_cap, &w.counters[7], w.terms, a.stats, -1,
-                     a.temporal ? -1 : 9, 32u);
-        else reuse_merge_body(a, w);
+                     a.temporal ? -1 : 9, 32u, warp);
+        } else {
+            const uint32_t per = 32u / (w.slots <= 2 ? 2u : w.slots <= 4 ? 4u : w.slots <= 8 ? 8u : 16u);
+            ntask = (min(w.counters[0], (uint32_t)w.cap_units) + per - 1u) / per * 32u;
+            reuse_merge_body(a, w, warp);
+        }
+        // the next instance's shares start where this one's ended
+        const uint32_t used = (ntask + 31u) / 32u % warps;
+        warp = warp >= used ? warp - used : warp + warps - used;
     }
 }
 
 cudaError_t launch_reuse_batch(const ReuseJob* J, int n, const int* blk_slots, int nblk_slots, const int* blk_units,
-                               int nblk_units, int persist_blocks, int vis_blocks, cudaStream_t s) {
+                               int nblk_units, int persist_blocks, int shift_blocks, int vis_blocks, cudaStream_t s) {
     note_launch(9);
     reuse_reset_batch_kernel<<<(n * kWaveCounters + 127) / 128, 128, 0, s>>>(J, n);
     reuse_slots_batch_kernel<<<nblk_slots, 128, 0, s>>>(J, blk_slots, n);
     reuse_units_batch_kernel<<<nblk_units, 128, 0, s>>>(J, blk_units, n);
-    reuse_persist_batch_kernel<0><<<persist_blocks, 128, 0, s>>>(J, n);
+    reuse_persist_batch_kernel<0><<<shift_blocks, 128, 0, s>>>(J, n);
     reuse_persist_batch_kernel<1><<<vis_blocks, 128, 0, s>>>(J, n);
     reuse_persist_batch_kernel<2><<<persist_blocks, 128, 0, s>>>(J, n);
-    reuse_persist_batch_kernel<3><<<persist_blocks, 128, 0, s>>>(J, n);
+    reuse_persist_batch_kernel<3><<<shift_blocks, 128, 0, s>>>(J, n);
     reuse_persist_batch_kernel<4><<<vis_blocks, 128, 0, s>>>(J, n);
     reuse_persist_batch_kernel<5><<<persist_blocks, 128, 0, s>>>(J, n);
     return cudaGetLastError();
