@@ -41,7 +41,7 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
                                   uint32_t** prim_out, float4* scratch, cudaStream_t s);
 cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
-                            int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut,
+                            int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut, float4* boxes,
                             int sms, cudaStream_t s);
 cudaError_t launch_etree(int nt, int P, const float4* tri, float4* node, cudaStream_t s);
 cudaError_t launch_refit(int n, const uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, const int* child,
@@ -574,7 +574,7 @@ tof_status tof_bvh_build(tof_ctx* c, tof_scene id, const float* xf, int refit_on
     if (full && S.nt > 1) {
         if (!c->sms) CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
         CK(launch_treelets(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, S.keys2,
-                           S.vals2, S.bb + 6, c->sms, s));
+                           S.vals2, S.bb + 6, S.cent, c->sms, s));
     } else {
         CK(launch_refit(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, s));
     }
