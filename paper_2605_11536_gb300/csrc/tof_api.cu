@@ -113,6 +113,8 @@ struct ViewH {
     uint32_t geom_version[2] = {0, 0};
     int cur = 0;
     int prev_final = -1;
+    size_t prev_bins = 0;        // at most so many of a pixel's bins hold a sample in res[prev_final]
+    bool recorded = false;       // a render of it was recorded into a user's graph: its replays are not seen here
     bool has_prev = false;
     StatsDev* stats = nullptr;
     cudaStream_t last_stream = nullptr;
@@ -266,6 +268,14 @@ static ParamsDev to_dev(const tof_params* p, uint64_t seed) {
     return d;
 }
 
+// candidates of a pixel's initial stage
+static int initial_candidates(const tof_params* p) {
+    const int kmin = (p->flags & TOF_FLAG_DIRECT) ? 1 : 2;
+    int lengths = p->depth - kmin + 1;
+    if (p->flags & TOF_FLAG_ELLIPSOID) lengths += p->depth - 1;   // one ellipsoidal candidate per vertex below depth
+    return lengths > 0 ? p->n_cand * lengths : 0;
+}
+
 static tof_status check_params(tof_ctx* c, const tof_params* p, int transient) {
     if (!p) return fail(c, TOF_EINVAL, "params is NULL");
     if (p->depth < 1 || p->depth > kMaxDepth) return fail(c, TOF_EINVAL, "depth %d outside [1, %d]", p->depth, kMaxDepth);
@@ -291,12 +301,9 @@ static tof_status check_params(tof_ctx* c, const tof_params* p, int transient) {
             return fail(c, TOF_EINVAL, "shrink_fine %d outside [0, n_cand - 1]", p->shrink_fine);
     }
     if (transient) {
-        int kmin = (p->flags & TOF_FLAG_DIRECT) ? 1 : 2;
-        int lengths = p->depth - kmin + 1;
-        if (p->flags & TOF_FLAG_ELLIPSOID) lengths += p->depth - 1;   // one ellipsoidal candidate per vertex below depth
-        if (lengths > 0 && p->n_cand * lengths > kMaxBinsPerPixel)
+        if (initial_candidates(p) > kMaxBinsPerPixel)
             return fail(c, TOF_EINVAL, "transient: n_cand * path lengths = %d exceeds %d candidates per pixel",
-                        p->n_cand * lengths, kMaxBinsPerPixel);
+                        initial_candidates(p), kMaxBinsPerPixel);
     }
     return TOF_OK;
 }
@@ -778,10 +785,12 @@ static bool tree_wave_ready(const ViewH& V, const tof_params* p) {
 // a histogram's initial stage runs as the wavefront in direct renders, where its scratch (2 KB a pixel with 8
 // trees of depth 4, against 300 B a bin of the view itself) is to be had; batches and the served form, which
 // account their views' memory beforehand, keep the single kernel
-static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p) {
+static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p, bool capturing) {
     if (c->in_batch || g_rec) return false;
     const std::string before = c->err;
     const size_t paths = (size_t)V.W * V.H * (size_t)p->n_cand;
+    // nothing is allocated while the stream is being captured
+    if (capturing && !(V.tw_paths >= paths && V.tw.nc == p->n_cand && V.tw.depth == p->depth)) return false;
     if (V.tw_denied && paths >= V.tw_denied) return false;
     if (ensure_tree_wave(c, V, p->n_cand, p->depth) == TOF_OK) return true;
     V.tw_denied = paths;   // not tried again at every frame
@@ -846,8 +855,8 @@ static tof_status ensure_side(tof_ctx* c, ViewH& V) {
 }
 
 // one reuse pass as a wavefront; transient passes run in pixel chunks so that a chunk's merge
-// units (at most B per pixel) never exceed the scratch capacity
-static tof_status reuse_pass(tof_ctx* c, ViewH& V, const ReuseArgs& ra, const WaveDev* fixed, cudaStream_t s) {
+// units (at most `bins` per pixel) never exceed the scratch capacity
+static tof_status reuse_pass(tof_ctx* c, ViewH& V, const ReuseArgs& ra, size_t bins, const WaveDev* fixed, cudaStream_t s) {
     const int S = ra.binpass ? 3 : ra.temporal ? 2 : 1 + ra.P.n_spatial;
     const size_t npix = (size_t)V.W * V.H;
     const size_t Bn = V.B > 0 ? (size_t)V.B : 1;
@@ -866,7 +875,7 @@ static tof_status reuse_pass(tof_ctx* c, ViewH& V, const ReuseArgs& ra, const Wa
     w.rays2 = beside ? V.rays2 : nullptr;
     w.ray2_cap = beside ? V.ray2_cap : 0u;
     if (!fixed) w.cap_units = V.wave_cap;
-    size_t chunk = V.B > 0 ? (size_t)V.wave_cap / Bn : npix;
+    size_t chunk = V.B > 0 ? (size_t)V.wave_cap / (bins < 1 ? 1 : bins < Bn ? bins : Bn) : npix;
     if (chunk < 1) chunk = 1;
     for (size_t p0 = 0; p0 < npix; p0 += chunk) {
         size_t p1 = p0 + chunk < npix ? p0 + chunk : npix;
@@ -947,6 +956,14 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     mark(V, 1, s);
     V.ran[0] = true;
 
+    bool capturing = false;
+    if (B > 0 && !c->in_batch && !g_rec) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+        else capturing = cap != cudaStreamCaptureStatusNone;
+        V.recorded = V.recorded || capturing;
+    }
+
     // temporal reuse needs the previous frame's geometry still resident
     bool temporal = params->temporal && V.has_prev && V.prev_final >= 0 &&
                     S.version[V.geom_slot[1 - fc]] == V.geom_version[1 - fc];
@@ -984,7 +1001,7 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
             CK(launch_initial_ell_wave(ia, V.ell, V.tune.tile_h, eb, vb, s));
         }
     } else if (use_tree_wave(V, B, params, fixed_wave != nullptr) &&
-               (B > 0 ? hist_tree_wave(c, V, params) : !(c->in_batch || g_rec) || tree_wave_ready(V, params))) {
+               (B > 0 ? hist_tree_wave(c, V, params, capturing) : !(c->in_batch || g_rec) || tree_wave_ready(V, params))) {
         // a batch uses the wavefront only where prepare_job allocated its scratch (large views)
         TRY(ensure_tree_wave(c, V, params->n_cand, params->depth));
         TRY(persist_init(c));
@@ -1009,6 +1026,15 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     V.ran[1] = true;
     int src = out_of(stage);
     ++stage;
+    // How many of a pixel's bins can hold a sample bounds a pass's merge units: at first one per candidate,
+    // then the bins of everything that a pass merges.  A histogram of 1024 bins is far from full in a
+    // capture's first frames, so its passes take larger chunks of the same scratch: 10 instead of 20 in three
+    // frames of 128 x 128 pixels and 8 trees, 3.70 -> 2.71 ms (a chunk's kernels last as long as their longest
+    // rays).  Of a graph, whose replays the host does not see, nothing is assumed but B.
+    const size_t all_bins = B > 0 ? (size_t)B : 1;
+    const bool bounded = B > 0 && !V.recorded && !c->in_batch && !g_rec;
+    auto bins_of = [&](size_t x) { return bounded && x < all_bins ? x : all_bins; };
+    size_t bins = bins_of((size_t)initial_candidates(params));
     ReuseArgs ra;
     memset(&ra, 0, sizeof(ra));
     ra.cur = F; ra.P = P; ra.stats = V.stats;
@@ -1020,7 +1046,8 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
         ra.temporal = 1; ra.pass = 0;
         ra.geom_static = V.geom_version[1 - fc] == S.version[S.cur];
         ra.out = (stage == stages - 1 && B == 0) ? out : nullptr;
-        TRY(reuse_pass(c, V, ra, fixed_wave, s));
+        bins = bins_of(bins + V.prev_bins);
+        TRY(reuse_pass(c, V, ra, bins, fixed_wave, s));
         src = out_of(stage);
         ++stage;
         V.ran[2] = true;
@@ -1034,7 +1061,8 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
         ra.dst = V.res[out_of(stage)].dev();
         ra.temporal = 0; ra.binpass = 1; ra.pass = 8; ra.geom_static = 1;
         ra.out = nullptr;
-        TRY(reuse_pass(c, V, ra, fixed_wave, s));
+        bins = bins_of(3 * bins);
+        TRY(reuse_pass(c, V, ra, bins, fixed_wave, s));
         ra.binpass = 0;
         src = out_of(stage);
         ++stage;
@@ -1048,7 +1076,8 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
             ra.dst = V.res[out_of(stage)].dev();
             ra.temporal = 0; ra.pass = 1 + it; ra.geom_static = 1;
             ra.out = (stage == stages - 1 && B == 0) ? out : nullptr;
-            TRY(reuse_pass(c, V, ra, fixed_wave, s));
+            bins = bins_of(bins * (size_t)(1 + params->n_spatial));
+            TRY(reuse_pass(c, V, ra, bins, fixed_wave, s));
             src = out_of(stage);
             ++stage;
             V.ran[3] = true;
@@ -1069,6 +1098,7 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     V.geom_version[fc] = S.version[S.cur];
     V.cur = fc;
     V.prev_final = src;
+    V.prev_bins = bins;
     V.has_prev = true;
     return TOF_OK;
 }
