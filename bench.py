@@ -209,7 +209,7 @@ def run_ours(args, rank, world):
     flush = torch.empty(256 * 1024 * 1024 // 4, device=dev)
     xf32 = [np.ascontiguousarray(sc.xforms[f].reshape(-1), dtype=np.float32) for f in range(nf)]
 
-    # a full LBVH build every frame: 0.23 ms for 66k triangles, against refits of the first frame's
+    # a full LBVH build every frame: 0.2 ms for 66k triangles, against refits of the first frame's
     # hierarchy whose SAH cost doubles as the spheres turn (traversal 1.4x slower on average)
     def frame(f, refit):
         tof.tof_bvh_build(ctx, sid, xf32[f % nf], refit_only=refit, stream=sptr)

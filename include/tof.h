@@ -182,7 +182,8 @@ tof_status tof_scene_destroy(tof_ctx* ctx, tof_scene scene);
 /* Place the objects (row-major 3x4 object-to-world matrices, nobj*12 floats) and build the GPU
  * LBVH (Morton codes, radix sort, hierarchy, bounds).  Not in the paper, which traces rays with
  * the GPU's ray-tracing hardware through DXR (Sec. 6); GB300 has no such units, so the library
- * builds its own hierarchy (Karras 2012 construction over 30-bit Morton codes).  refit_only = 1 keeps the hierarchy and
+ * builds its own hierarchy (Karras 2012 construction over 30-bit Morton codes, its ranges of up to
+ * 512 leaves and the levels above them rebuilt by the surface area heuristic).  refit_only = 1 keeps the hierarchy and
  * refits bounds after rigid motion: cheaper to build, but the hierarchy's quality decays as objects
  * move away from where it was built (a full build of 66k triangles takes about 0.2 ms on GB300 and
  * pays for itself within a few frames of motion).  Call once per frame before rendering it: the library keeps

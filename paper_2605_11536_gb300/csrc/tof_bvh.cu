@@ -4,10 +4,14 @@
 // RT cores, so visibility runs on a software LBVH built here:
 //   xform_kernel    rigid 3x4 object transform of every triangle corner, per frame
 //   bounds / morton 30-bit Morton codes of triangle centroids in the centroid bounds (cubic cells)
-//   radix sort      4 stable 8-bit LSD passes (tile histograms, one scan, ranked scatter)
-//   karras_kernel   binary radix tree over the sorted codes (Karras, HPG 2012), ties broken by index
-//   refit_kernel    leaf records in leaf order and bottom-up child boxes (one atomic per node;
-//                   the second arriving thread continues, no thread waits)
+//   radix sort      4 stable 8-bit LSD passes (tile histograms, offsets, ranked scatter), one cooperative
+//                   launch where its blocks can all be resident
+//   karras_kernel   binary radix tree over the sorted codes (Karras, HPG 2012), ties broken by index; lists
+//                   the ranges of at most 512 leaves below which it is rebuilt
+//   range_box / treelet / treelet_top_kernel   those ranges, and the levels above them, top-down by the surface
+//                   area heuristic; leaf records in leaf order
+//   refit_kernel    (refits, one triangle) leaf records and bottom-up child boxes of the hierarchy as it is (one
+//                   atomic per node; the second arriving thread continues, no thread waits)
 //   etree_*_kernel  the ellipsoidal connection's hierarchy over triangle index ranges (boxes and
 //                   areas, bottom-up: 8 levels per block in shared memory, then one block)
 #include <cstdio>
@@ -377,9 +381,9 @@ __global__ void refit_kernel(int n, const uint32_t* __restrict__ prim, const flo
 // confocal scan 18 against 11.5; box 13.6 against 7.2).  So the Morton order is cut into ranges of at most
 // 512 leaves, each is built anew top-down by one block -- every split of the sorted orders tried, all nodes
 // of a level at once, the triangles' boxes in shared memory -- and one block builds the levels above over
-// the ranges' roots in the same way (up to 1024 of them; more keep the Morton hierarchy there).  Bound by
+// the ranges' boxes in the same way, beside them (up to 1024 of them; more keep the Morton hierarchy there).  Bound by
 // the issue of the running-box shuffles over about 14 levels; ranges of 256 and 128 leaves: 121 and 205 us
-// for both kernels instead of 126.  Frames with the build: 512 x 512 2.73 -> 2.63 ms, 1024 x 1024 11.1 ->
+// for both kernels one after the other instead of 126.  Frames with the build: 512 x 512 2.73 -> 2.63 ms, 1024 x 1024 11.1 ->
 // 10.4; static scenes: path tracing 608 -> 446 us, 128 x 128 allocation-free 428 -> 361 us.
 // It writes boxes, children and leaf order itself, so a full build needs no bottom-up pass over all levels.
 // Node numbers: a range [a, a + m) owns the m - 1 numbers of its Karras nodes; its root keeps the Karras

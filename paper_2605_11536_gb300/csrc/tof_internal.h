@@ -131,7 +131,7 @@ struct InitArgs {
     float* out;              // gated image if this is the last stage (else null)
     int tile_w;
     int wave;                // a staged batch runs this instance's initial stage as the bounce
-                             // wavefront: initial_gated_batch_kernel skips it
+                             // wavefront: initial_lanes_batch_kernel skips it
 };
 
 struct ReuseArgs {

@@ -2,10 +2,11 @@
 //
 //   gbuffer_kernel   primary visibility, one jittered ray per pixel            (Sec. 3.2 setup)
 //   initial_kernel   path trees with NEE, streaming RIS into per-bin reservoirs (stage (1), Sec. 4.5);
-//                    direct gated renders run it as a bounce wavefront (tw_*_kernel)
+//                    direct renders run it as a bounce wavefront (tw_*_kernel), the allocation-free form
+//                    and a batch's small views with a thread per tree (initial_lanes_*_kernel)
 //   (temporal and spatial reuse, stages (2) and (3), are in tof_reuse.cu)
 //   splat_kernel     transient histogram H[px, b] = f(y_b) W_b                  (stage (4), Sec. 4.5)
-//   pt_kernel        plain gated / transient path tracing (the comparison of Sec. 6)
+//   pt_kernel        plain gated / transient path tracing, a thread per sample (the comparison of Sec. 6)
 //   laser_kernel     resolves the collimated laser's spot (Sec. 5 "Light Source")
 // The gated image is written by the last stage's kernels (final shading fused into them).
 #include "tof_device.cuh"
@@ -703,7 +704,7 @@ __global__ void __launch_bounds__(128) tree_select_bins_kernel(const __grid_cons
 
 // --------------------------------------------------------------------------------------------
 // gated initial candidates as a bounce wavefront (TreeWaveDev): the same trees, candidates,
-// uniforms and order as initial_gated_kernel<false>, so the same reservoirs, with every lane of a
+// uniforms and order as initial_lanes_kernel, so the same reservoirs, with every lane of a
 // warp on the same step.  In the single kernel a warp's 32 path trees diverge in depth, in
 // traversal length and in whether a candidate needs a light segment, and most lanes idle:
 //   tw_start_kernel   one thread per path: vertex 1 (the G-buffer hit), its NEE candidate, the
