@@ -1131,8 +1131,8 @@ def main():
             "spatial_merge": BYTES["spatial_merge"] * r["npix"]}
     ell, walk = int(bool(args.flags & 256)), int(bool(args.flags & 64))
     kernels = {"gbuffer": "gbuffer_kernel", "initial": ELL_WAVE if ell else TREE_WAVE, "temporal": "temporal pass (8 kernels)",
-               "spatial_setup": "reuse_slots_kernel + reuse_units_kernel", "spatial_fwd_shift": "shift_fwd_kernel<%d>" % walk,
-               "spatial_fwd_vis": "vis_kernel (forward segments) + emit_inv_kernel", "spatial_inv_shift": "shift_inv_kernel<%d>" % walk,
+               "spatial_setup": "reuse_slots_kernel + reuse_units_kernel", "spatial_fwd_shift": "shift_fwd_kernel<%d, 1>" % walk,
+               "spatial_fwd_vis": "vis_kernel (forward segments) + emit_inv_kernel", "spatial_inv_shift": "shift_inv_kernel<%d, 1>" % walk,
                "spatial_inv_vis": "vis_kernel (inverse segments)", "spatial_merge": "reuse_merge_kernel"}
     src = _src_hash()
     traffic = NCU_TRAFFIC if src == NCU_TRAFFIC_SRC else {}
