@@ -72,15 +72,15 @@ BYTES = {
 # kernel changes; the hash below ties the figures to the sources they were captured on.
 ELL_WAVE = "ell_trees_kernel + ell_place_kernel + ell_select_kernel"
 TREE_WAVE = "tw_start_kernel + 3 x (tw_hit_kernel + tw_shade_kernel) + vis_kernel + tree_select_kernel"
-NCU_TRAFFIC_SRC = "ac8af494847f"   # _src_hash() of the sources the figures below were captured on
+NCU_TRAFFIC_SRC = "529488b1c205"   # _src_hash() of the sources the figures below were captured on
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch (one stage for the initial wavefront),
-# frame 5 (profiles/launches_dynamic_gated_512.md, profiles/tree_wavefront_dynamic_gated_512.md)
-NCU_TRAFFIC = {TREE_WAVE: 306.09e6, "shift_inv_kernel<0>": 185.79e6 + 380.14e6, "shift_fwd_kernel<0>": 166.26e6 + 240.34e6,
-               "vis_kernel (inverse segments)": 87.57e6 + 2.90e6, "reuse_merge_kernel": 115.84e6 + 7.45e6}
+# frame 5 (profiles/kernels_dynamic_gated_512.md)
+NCU_TRAFFIC = {TREE_WAVE: 314.17e6, "shift_inv_kernel<0, 1>": 100.11e6 + 64.68e6, "shift_fwd_kernel<0, 1>": 50.45e6 + 41.55e6,
+               "vis_kernel (inverse segments)": 88.74e6 + 2.95e6, "reuse_merge_kernel": 115.86e6 + 7.44e6}
 # L1 / L2 sector hit rates (%) and active lanes per warp instruction of the traversal-bound kernels,
 # from the same capture (the initial wavefront's first closest-hit round)
-NCU_HIT = {"tw_hit_kernel": [87.5, 72.0, 12.1], "shift_fwd_kernel<0>": [42.0, 45.1, 20.4],
-           "shift_inv_kernel<0>": [46.9, 64.8, 22.1], "vis_kernel": [94.8, 67.2, 13.5]}
+NCU_HIT = {"tw_hit_kernel": [79.8, 69.5, 14.6], "shift_fwd_kernel<0, 1>": [49.8, 58.9, 19.5],
+           "shift_inv_kernel<0, 1>": [64.4, 51.8, 21.1], "vis_kernel": [91.4, 65.9, 16.5]}
 
 
 def _peaks():
