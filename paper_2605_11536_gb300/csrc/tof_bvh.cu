@@ -430,13 +430,15 @@ __device__ __forceinline__ void run_boxes(int longest, int p, int s, int e, bool
 
 // Builds the hierarchy of items 0 .. m - 1 (m >= 2, boxes in S.box) with N threads.  number(split,
 // root_split) is the node that splits after position `split`; leaf(position, item) the child code of one item;
-// up(code, node) records a child's parent.  Levels from kMaxSweep on split in the middle, which bounds the
-// depth (coincident items).  all_axes: every split of the three orders is tried, else those of the order along
+// up(code, node) records a child's parent.  Levels from `sweeps` on split in the middle, which bounds the
+// depth (coincident items): 16 and 9 levels in a range of 512, 16 and 10 above 1024 ranges, 51 of the 64 that a
+// traversal's stack holds.  Below the Morton hierarchy's own top, which can be 30 levels and the logarithm of its
+// ranges deep, 8 and 9 levels.  all_axes: every split of the three orders is tried, else those of the order along
 // the segment's longest axis (a third of the work: 145 -> 77 us for 66k triangles, visits per ray up 2 %; a
 // scene of one range tries all, 12 % fewer visits in the 332-triangle box).
-constexpr int kMaxSweep = 16;
+constexpr int kMaxSweep = 16, kMortonSweep = 8;
 template <int N, class Number, class Leaf, class Up>
-__device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, bool all_axes, float4* __restrict__ nodes, int* __restrict__ child, Number number, Leaf leaf,
+__device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, bool all_axes, int sweeps, float4* __restrict__ nodes, int* __restrict__ child, Number number, Leaf leaf,
                                             Up up) {
     const int p = threadIdx.x;
     const int nt = (m + 31) & ~31;
@@ -520,7 +522,7 @@ __device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, bool all_axes, f
                 float r[6];
 #pragma unroll
                 for (int k = 0; k < 6; ++k) r[k] = S.suf[k][p + 1];
-                const float c = level >= kMaxSweep ? 0.f : half_area(f) * (float)(p + 1 - s) + half_area(r) * (float)(e - 1 - p);
+                const float c = level >= sweeps ? 0.f : half_area(f) * (float)(p + 1 - s) + half_area(r) * (float)(e - 1 - p);
                 if (bax < 0 || c < bestc) {
                     bestc = c; bax = ax;
 #pragma unroll
@@ -664,7 +666,7 @@ __global__ void __launch_bounds__(kTreelet) treelet_kernel(int n, uint32_t* __re
             // numbers a .. a + m - 1 without the end that is not the root's
             const int base = last ? a + 1 : a, root = last ? a + m - 1 : a, at_root = root - base;
             sweep_build<kTreelet>(
-                S, m, R == 1u, nodes, child,
+                S, m, R == 1u, R == 1u || top_by_area((int)R, n) ? kMaxSweep : kMortonSweep, nodes, child,
                 [=](int split, int rs) { return split == rs ? root : split == at_root ? base + rs : base + split; },
                 [=](int q, int) { return ~(a + q); },
                 [=](int code, int node) {
@@ -723,7 +725,7 @@ __global__ void __launch_bounds__(kTopItems) treelet_top_kernel(int n, const uin
         auto slot_of = [=](int item) { return (cut_m[item] & kRootLast) ? (int)cut_a[item] : (int)(cut_a[item] + (cut_m[item] & ~kRootLast)) - 1; };
         const int zero_split = zero == R - 1 ? none : zero;
         sweep_build<kTopItems>(
-            S, R, false, nodes, child,
+            S, R, false, kMaxSweep, nodes, child,
             [=](int split, int rs) { return split == rs ? 0 : slot_of(slot_item(split == zero_split ? rs : split)); },
             [=](int, int item) {
                 const int a = (int)cut_a[item], m = (int)(cut_m[item] & ~kRootLast);
