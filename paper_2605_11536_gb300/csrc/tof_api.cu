@@ -139,6 +139,7 @@ struct ViewH {
     void* ell_ptrs[9] = {nullptr};
     TreeWaveDev tw;              // the gated initial stage's bounce wavefront
     size_t tw_paths = 0;         // pixels x trees it holds
+    size_t tw_bytes = 0;         // of a histogram view: what it takes, given back when other scratch needs the room
     size_t tw_denied = 0;        // pixels x trees of a histogram view that there was no room for
     void* tw_ptrs[9] = {nullptr};
     tof_tuning tune = {16, 8, 0, TOF_LAYOUT_SOA};   // launch shapes and reservoir layout (autotuner)
@@ -152,6 +153,8 @@ struct tof_ctx {
     int device = 0;
     uint64_t budget = 0;
     uint64_t used = 0;
+    uint64_t optional = 0;       // of `used`: histogram views' wavefront scratch, which a render can do without
+    bool keep_optional = false;  // it is not given back (its own allocation, or the caller's stream is being captured)
     std::string err;
     std::vector<SceneH> scenes;
     std::vector<ViewH> views;
@@ -192,15 +195,22 @@ static tof_status fail(tof_ctx* c, tof_status st, const char* fmt, ...) {
     return st;
 }
 
+static bool give_back_optional(tof_ctx* c);
+
 template <class T>
 static tof_status dalloc(tof_ctx* c, T** p, size_t bytes, const char* what) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
+    if (c->budget && c->used + bytes > c->budget) give_back_optional(c);
     if (c->budget && c->used + bytes > c->budget)
         return fail(c, TOF_EBUDGET, "%s: %zu bytes exceed the HBM budget (%llu of %llu used)", what, bytes,
                     (unsigned long long)c->used, (unsigned long long)c->budget);
     void* q = nullptr;
     cudaError_t e = cudaMalloc(&q, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        if (give_back_optional(c)) e = cudaMalloc(&q, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(c, TOF_ENOMEM, "%s: cudaMalloc(%zu) failed: %s", what, bytes, cudaGetErrorString(e));
@@ -222,6 +232,34 @@ static void dfree(tof_ctx* c, void* p) {
         }
     cudaFree(p);
 }
+
+static void free_tree_wave(tof_ctx* c, ViewH& V) {
+    for (void*& p : V.tw_ptrs) { dfree(c, p); p = nullptr; }
+    c->optional -= V.tw_bytes;
+    V.tw_bytes = 0;
+    V.tw_paths = 0;
+}
+// Frees the histogram views' wavefront scratch (hist_tree_wave), which must not take the room of anything
+// that a call cannot do without; such a view keeps to the single kernel from then on.  False if there is
+// none.  (cudaFree waits for the kernels that use it; a recorded graph may still run with its own.)
+static bool give_back_optional(tof_ctx* c) {
+    if (!c->optional || c->keep_optional) return false;
+    bool any = false;
+    for (ViewH& V : c->views)
+        if (V.alive && V.tw_bytes && !V.recorded) {
+            V.tw_denied = 1;
+            free_tree_wave(c, V);
+            any = true;
+        }
+    return any;
+}
+
+struct KeepOptional {
+    tof_ctx* c;
+    bool before;
+    KeepOptional(tof_ctx* c_, bool keep) : c(c_), before(c_->keep_optional) { c->keep_optional = before || keep; }
+    ~KeepOptional() { c->keep_optional = before; }
+};
 
 #define CK(call)                                                                                     \
     do {                                                                                             \
@@ -632,7 +670,7 @@ tof_status tof_view_destroy(tof_ctx* c, tof_view id) {
     for (int k = 0; k < 3; ++k) { dfree(c, V.res[k].planes); dfree(c, V.res[k].M); dfree(c, V.res[k].occ); }
     for (void* p : V.wave_ptrs) dfree(c, p);
     for (void* p : V.ell_ptrs) dfree(c, p);
-    for (void* p : V.tw_ptrs) dfree(c, p);
+    free_tree_wave(c, V);
     dfree(c, V.rays2);
     if (V.side) cudaStreamDestroy(V.side);
     if (V.side_fork) cudaEventDestroy(V.side_fork);
@@ -729,8 +767,7 @@ static tof_status ensure_ell_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
 static tof_status ensure_tree_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
     const size_t paths = (size_t)V.W * V.H * (size_t)nc, slots = paths * (size_t)depth;
     if (V.tw_paths >= paths && V.tw.nc == nc && V.tw.depth == depth) return TOF_OK;
-    for (void*& p : V.tw_ptrs) { dfree(c, p); p = nullptr; }
-    V.tw_paths = 0;
+    free_tree_wave(c, V);
     TreeWaveDev& w = V.tw;
     w = TreeWaveDev();
     w.nc = nc; w.depth = depth;
@@ -783,8 +820,9 @@ static bool tree_wave_ready(const ViewH& V, const tof_params* p) {
 }
 
 // a histogram's initial stage runs as the wavefront in direct renders, where its scratch (2 KB a pixel with 8
-// trees of depth 4, against 300 B a bin of the view itself) is to be had; batches and the served form, which
-// account their views' memory beforehand, keep the single kernel
+// trees of depth 4, against 300 B a bin of the view itself) is to be had beside everything that the context's
+// calls cannot do without (give_back_optional); batches and the served form, which account their views'
+// memory beforehand, keep the single kernel
 static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p, bool capturing) {
     if (c->in_batch || g_rec) return false;
     const std::string before = c->err;
@@ -792,7 +830,15 @@ static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p, bool captu
     // nothing is allocated while the stream is being captured
     if (capturing && !(V.tw_paths >= paths && V.tw.nc == p->n_cand && V.tw.depth == p->depth)) return false;
     if (V.tw_denied && paths >= V.tw_denied) return false;
-    if (ensure_tree_wave(c, V, p->n_cand, p->depth) == TOF_OK) return true;
+    const KeepOptional keep(c, true);
+    const uint64_t held = c->used - V.tw_bytes;
+    const tof_status st = ensure_tree_wave(c, V, p->n_cand, p->depth);
+    if (st == TOF_OK) {
+        c->optional -= V.tw_bytes;
+        V.tw_bytes = c->used - held;
+        c->optional += V.tw_bytes;
+        return true;
+    }
     V.tw_denied = paths;   // not tried again at every frame
     c->err = before;
     return false;
@@ -937,6 +983,14 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     if (!g_no_marks) TRY(pending_err(c));
     cudaStream_t s = (cudaStream_t)stream;
     V.last_stream = s;
+    bool capturing = false;
+    if (!c->in_batch && !g_rec) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+        else capturing = cap != cudaStreamCaptureStatusNone;
+        V.recorded = V.recorded || capturing;
+    }
+    const KeepOptional keep(c, capturing);   // nothing is freed while the stream is being captured
 
     const int fc = V.has_prev ? 1 - V.cur : V.cur;
     FrameDev F = make_frame(S, S.cur, sensor, emitter, L0, dL, B, frame, V.gb[fc], V.laser[fc], c->d_err);
@@ -955,14 +1009,6 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     }
     mark(V, 1, s);
     V.ran[0] = true;
-
-    bool capturing = false;
-    if (B > 0 && !c->in_batch && !g_rec) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-        else capturing = cap != cudaStreamCaptureStatusNone;
-        V.recorded = V.recorded || capturing;
-    }
 
     // temporal reuse needs the previous frame's geometry still resident
     bool temporal = params->temporal && V.has_prev && V.prev_final >= 0 &&
@@ -1179,6 +1225,9 @@ __attribute__((visibility("hidden"))) int tof_internal_scene_objects(tof_ctx* c,
     if (!c || id < 0 || id >= (int)c->scenes.size() || !c->scenes[id].alive) return -1;
     return c->scenes[id].nobj;
 }
+
+// device bytes of a context without the scratch that it gives back when other allocations need the room
+__attribute__((visibility("hidden"))) uint64_t tof_internal_required_bytes(tof_ctx* c) { return c ? c->used - c->optional : 0; }
 
 // validate one job of a batch and allocate its view's scratch (allocation is not allowed inside the
 // capture)

@@ -17,6 +17,7 @@
 
 extern "C" {
 __attribute__((visibility("hidden"))) tof_status tof_internal_prepare_job(tof_ctx* c, const tof_job* job);
+__attribute__((visibility("hidden"))) uint64_t tof_internal_required_bytes(tof_ctx* c);
 __attribute__((visibility("hidden"))) tof_status tof_internal_render_batch(tof_ctx* c, const tof_job* jobs, uint32_t n,
                                                                          void* stream, int slot);
 }
@@ -204,7 +205,7 @@ static bool evict_one(tof_server* s, int32_t keep) {
 static tof_status admit_view(tof_server* s, int32_t sid, const tof_job& job, bool* fits) {
     StreamS& st = s->streams[sid];
     *fits = false;
-    const uint64_t before = tof_device_bytes(s->ctx);
+    const uint64_t before = tof_internal_required_bytes(s->ctx);
     tof_view v;
     tof_status rc = tof_view_create(s->ctx, st.scene, st.W, st.H, st.B, &v);
     if (rc == TOF_OK) {
@@ -215,7 +216,7 @@ static tof_status admit_view(tof_server* s, int32_t sid, const tof_job& job, boo
     }
     if (rc == TOF_EBUDGET || rc == TOF_ENOMEM) return TOF_OK;   // the context's own bound: defer
     if (rc != TOF_OK) return rc;
-    const uint64_t bytes = tof_device_bytes(s->ctx) - before;
+    const uint64_t bytes = tof_internal_required_bytes(s->ctx) - before;
     while (s->budget && s->resident + bytes > s->budget)
         if (!evict_one(s, sid)) break;
     if (s->budget && s->resident + bytes > s->budget) {
