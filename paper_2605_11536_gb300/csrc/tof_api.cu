@@ -827,8 +827,9 @@ static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p, bool captu
     if (c->in_batch || g_rec) return false;
     const std::string before = c->err;
     const size_t paths = (size_t)V.W * V.H * (size_t)p->n_cand;
-    // nothing is allocated while the stream is being captured
-    if (capturing && !(V.tw_paths >= paths && V.tw.nc == p->n_cand && V.tw.depth == p->depth)) return false;
+    const bool fits = V.tw_paths >= paths && V.tw.nc == p->n_cand && V.tw.depth == p->depth;
+    // nothing is allocated while the stream is being captured, and what a recorded graph may run with stays
+    if (!fits && (capturing || (V.recorded && V.tw_paths))) return false;
     if (V.tw_denied && paths >= V.tw_denied) return false;
     const KeepOptional keep(c, true);
     const uint64_t held = c->used - V.tw_bytes;
