@@ -139,6 +139,7 @@ struct ViewH {
     void* ell_ptrs[9] = {nullptr};
     TreeWaveDev tw;              // the gated initial stage's bounce wavefront
     size_t tw_paths = 0;         // pixels x trees it holds
+    size_t tw_slots = 0;         // pixels x trees x depth it holds
     size_t tw_bytes = 0;         // of a histogram view: what it takes, given back when other scratch needs the room
     size_t tw_denied = 0;        // pixels x trees of a histogram view that there was no room for
     void* tw_ptrs[9] = {nullptr};
@@ -237,7 +238,7 @@ static void free_tree_wave(tof_ctx* c, ViewH& V) {
     for (void*& p : V.tw_ptrs) { dfree(c, p); p = nullptr; }
     c->optional -= V.tw_bytes;
     V.tw_bytes = 0;
-    V.tw_paths = 0;
+    V.tw_paths = V.tw_slots = 0;
 }
 // Frees the histogram views' wavefront scratch (hist_tree_wave), which must not take the room of anything
 // that a call cannot do without; such a view keeps to the single kernel from then on.  False if there is
@@ -764,9 +765,21 @@ static tof_status ensure_ell_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
 // (re)allocate the bounce wavefront of the gated initial stage for nc trees of the given depth: per
 // (pixel, tree) 24 B per vertex (record and candidate), 32 B of path state, 80 B of rays and hits
 // and a queued light segment (about 240 MB for 512 x 512, 4 trees, depth 4)
+static bool tree_wave_fits(const ViewH& V, int nc, int depth) {
+    const size_t paths = (size_t)V.W * V.H * (size_t)nc;
+    if (V.B > 0) return V.tw_paths >= paths && V.tw_slots >= paths * (size_t)depth;
+    return V.tw_paths >= paths && V.tw.nc == nc && V.tw.depth == depth;
+}
 static tof_status ensure_tree_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
-    const size_t paths = (size_t)V.W * V.H * (size_t)nc, slots = paths * (size_t)depth;
-    if (V.tw_paths >= paths && V.tw.nc == nc && V.tw.depth == depth) return TOF_OK;
+    size_t paths = (size_t)V.W * V.H * (size_t)nc, slots = paths * (size_t)depth;
+    if (tree_wave_fits(V, nc, depth)) {
+        V.tw.nc = nc; V.tw.depth = depth;
+        return TOF_OK;
+    }
+    if (V.B > 0) {   // a histogram's is optional and grows; a gated view holds what its last frame needs
+        paths = std::max(paths, V.tw_paths);
+        slots = std::max(slots, V.tw_slots);
+    }
     free_tree_wave(c, V);
     TreeWaveDev& w = V.tw;
     w = TreeWaveDev();
@@ -792,6 +805,7 @@ static tof_status ensure_tree_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
     }
     for (int k = 0; k < 9; ++k) V.tw_ptrs[k] = ps[k];
     V.tw_paths = paths;
+    V.tw_slots = slots;
     return TOF_OK;
 }
 
@@ -827,10 +841,10 @@ static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p, bool captu
     if (c->in_batch || g_rec) return false;
     const std::string before = c->err;
     const size_t paths = (size_t)V.W * V.H * (size_t)p->n_cand;
-    const bool fits = V.tw_paths >= paths && V.tw.nc == p->n_cand && V.tw.depth == p->depth;
+    const bool fits = tree_wave_fits(V, p->n_cand, p->depth);
     // nothing is allocated while the stream is being captured, and what a recorded graph may run with stays
     if (!fits && (capturing || (V.recorded && V.tw_paths))) return false;
-    if (V.tw_denied && paths >= V.tw_denied) return false;
+    if (!fits && V.tw_denied && paths >= V.tw_denied) return false;
     const KeepOptional keep(c, true);
     const uint64_t held = c->used - V.tw_bytes;
     const tof_status st = ensure_tree_wave(c, V, p->n_cand, p->depth);

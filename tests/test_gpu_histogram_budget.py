@@ -100,3 +100,25 @@ def test_a_later_view_takes_the_wavefronts_room():
         assert tof.tof_device_bytes(ctx) == need
     finally:
         tof.tof_destroy(ctx)
+
+
+def test_changing_trees_and_depth_allocates_once():
+    import torch
+    from paper_2605_11536_gb300 import tof
+    sc = _scene(0, 0)
+    ctx, sid = _context(sc, 0)
+    try:
+        view, other = (tof.tof_view_create(ctx, sid, W, H, B) for _ in range(2))
+        out = torch.full((2, W * H * B), -1.0, device="cuda")
+        seen = []
+        for f, (trees, depth) in enumerate([(8, 2), (4, 5), (8, 2), (4, 5), (1, 3), (8, 2)]):
+            sc.params.n_cand, sc.params.depth = trees, depth
+            tof.tof_render_transient(ctx, sid, view, sc.sensors[0], sc.emitters[0], BINS, sc.params, 3, f, out[0].data_ptr())
+            seen.append(tof.tof_device_bytes(ctx))
+            tof.tof_render_batch(ctx, [tof.job(sid, other, sc.sensors[0], sc.emitters[0], sc.params, 3, f, out[1].data_ptr(), bins=BINS)])
+            tof.tof_sync(ctx)
+            a = out.cpu().numpy()
+            np.testing.assert_array_equal(a[0], a[1])   # in a batch: the single kernel
+        assert seen[2:] == [seen[2]] * 4, seen
+    finally:
+        tof.tof_destroy(ctx)
