@@ -230,6 +230,7 @@ struct PtArgs {
     FrameDev F;
     ParamsDev P;
     int spp;
+    int ppb;                 // pixels of a block (set by the launch)
     float* out;
 };
 
