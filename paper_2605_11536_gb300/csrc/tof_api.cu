@@ -47,7 +47,8 @@ cudaError_t launch_etree(int nt, int P, const float4* tri, float4* node, cudaStr
 cudaError_t launch_refit(int n, const uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, const int* child,
                          const int* parent_int, const int* parent_leaf, uint32_t* counter, cudaStream_t s);
 cudaError_t launch_gbuffer_batch(const GbufArgs* A, const int* blk0, int n, int blocks, cudaStream_t s);
-int initial_lanes_blocks(int W, int H, int n_cand);
+void initial_lanes_tile(long long npix, int nc, int sms, int* w, int* h);
+int initial_lanes_blocks(const InitArgs& a);
 cudaError_t launch_initial_batch(const InitArgs* A, const int* blk0, int n, int blocks, cudaStream_t s);
 cudaError_t launch_reuse_batch(const ReuseJob* J, int n, const int* blk_slots, int nblk_slots, const int* blk_units,
                                int nblk_units, int persist_blocks, int shift_blocks, int vis_blocks, cudaStream_t s);
@@ -719,6 +720,7 @@ struct BatchRec {
     std::vector<WaveRec> wave;
     std::vector<std::vector<ReuseJob>> pass;   // pass[q]: every instance's q-th reuse pass
     size_t q = 0;                              // the current instance's next pass
+    long long npix = 0;                        // pixels of all instances
 };
 // staged batches: while set, render() records each stage's arguments instead of launching them
 static BatchRec* g_rec = nullptr;
@@ -1042,6 +1044,8 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     ia.F = F; ia.dst = V.res[out_of(stage)].dev(); ia.P = P;
     ia.out = (stage == stages - 1 && B == 0) ? out : nullptr;
     ia.tile_w = V.tune.tile_w;
+    if (!c->sms) CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
+    initial_lanes_tile(g_rec ? g_rec->npix : (long long)V.W * V.H, params->n_cand, c->sms, &ia.lane_w, &ia.lane_h);
     if (B == 0 && params->shrink_k > 1.f) {
         CK(launch_initial_shrink(ia, V.tune.tile_h, s));
     } else if (use_ell_wave(V, B, params, fixed_wave != nullptr)) {
@@ -1329,7 +1333,7 @@ static size_t staged_layout(StagedGroup& G, size_t off) {
         const int tw = g.tile_w, th = 128 / tw;
         G.bpix[j + 1] = G.bpix[j] + ((g.F.W + tw - 1) / tw) * ((g.F.H + th - 1) / th);
         // an instance that runs the bounce wavefront needs no blocks here
-        G.binit[j + 1] = G.binit[j] + (G.rec.init[j].wave ? 0 : initial_lanes_blocks(g.F.W, g.F.H, g.P.n_cand));
+        G.binit[j + 1] = G.binit[j] + (G.rec.init[j].wave ? 0 : initial_lanes_blocks(G.rec.init[j]));
     }
     G.o_g = off;
     off = al256h(off + sizeof(GbufArgs) * nj);
@@ -1430,6 +1434,7 @@ static tof_status render_batch_staged(tof_ctx* c, const tof_job* jobs, uint32_t 
         load[best] += cost[i];
     }
     std::vector<StagedGroup> G(NG);
+    for (uint32_t i = 0; i < n; ++i) G[group[i]].rec.npix += (long long)c->views[jobs[i].view].W * c->views[jobs[i].view].H;
     g_no_marks = true;
     tof_status st = TOF_OK;
     for (uint32_t i = 0; i < n && st == TOF_OK; ++i) {

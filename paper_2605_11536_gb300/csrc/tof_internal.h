@@ -132,6 +132,7 @@ struct InitArgs {
     int tile_w;
     int wave;                // a staged batch runs this instance's initial stage as the bounce
                              // wavefront: initial_lanes_batch_kernel skips it
+    int lane_w, lane_h;      // pixel tile of the lane form (initial_lanes_tile)
 };
 
 struct ReuseArgs {

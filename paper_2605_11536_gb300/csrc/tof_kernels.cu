@@ -299,106 +299,134 @@ __global__ void __launch_bounds__(128, 4) initial_gated_ell_kernel(const __grid_
     a.dst.occ[pix] = occ;
     if (a.out) a.out[pix] = outv;
 }
-// Path trees in lanes: a block of 128 threads takes a small tile of pixels with one thread for each (pixel,
-// tree), which records its candidates and vertices in shared memory; then one thread per pixel replays
-// the streaming RIS in the trees' order -- the same trees, candidates, order and uniforms as one thread
-// walking the pixel's trees, without its chain of all of them.  Such a thread is bound by that chain's
-// latency (a 128 x 128 view has only 4 warps an SM), so a small view gains what the trees are parallel.
+// Path trees in lanes: a block of 128 threads takes a small tile of pixels (InitArgs::lane_w x lane_h) and runs
+// their trees through its threads, one each, 128 at a time; a thread records its tree's candidates and vertices
+// in shared memory, then one thread per pixel replays the streaming RIS in the trees' order -- the same
+// trees, candidates, order and uniforms as one thread walking the pixel's trees, without its chain of all of
+// them.  Such a thread is bound by that chain's latency (a 128 x 128 view has only 4 warps an SM), so a
+// small view gains what the trees are parallel.  A pixel's trees may reach into a second round, whose first
+// thread goes on with the selection (LaneTable::carry), so that tree counts that do not divide 128 leave few
+// threads idle (initial_lanes_tile); the replay looks only at trees with a candidate, since the block waits
+// for it.
 constexpr int kLaneThreads = 128;
-struct LaneTile { int w, h; };   // pixels of a block; w * h * n_cand <= kLaneThreads
-static __host__ __device__ __forceinline__ LaneTile lane_tile(int n_cand) {
-    const int pixels = kLaneThreads / n_cand;   // at least 2 (kMaxCand = 64)
-    LaneTile t;
-    t.w = pixels >= 8 ? 8 : pixels >= 4 ? 4 : 2;
-    t.h = pixels / t.w;
-    return t;
-}
+struct LaneCarry {
+    float S, tau;
+    int t, k;
+    float4 vtx[kMaxDepth];
+};
 struct LaneTable {
     float2 cand[kLaneThreads * kMaxDepth];   // (f / p, tau) of the candidate ending at vertex d of a thread's tree
     float4 vtx[kLaneThreads * kMaxDepth];    // (tri bits, b1, b2, area pdf) of vertex d
+    uint8_t masks[kLaneThreads];             // bit d - 1: a thread's tree has a candidate ending at vertex d
+    uint32_t any[kLaneThreads / 32];         // per warp, the lanes with candidates
+    LaneCarry carry[2];                      // the selection of the pixel that a round leaves off in, by the round's parity
 };
 struct LaneSink {
-    float2* cand;
-    float4* vtx;
-    __device__ void operator()(int k, float c, float tauv, const TreeVerts&, int) { cand[k - 1] = make_float2(c, tauv); }
+    LaneTable& tab;   // nothing of it in registers over the tree
+    __device__ void operator()(int k, float c, float tauv, const TreeVerts&, int) {
+        tab.cand[threadIdx.x * kMaxDepth + k - 1] = make_float2(c, tauv);
+        tab.masks[threadIdx.x] |= (uint8_t)(1u << (k - 1));
+    }
     __device__ void vertex(int d, const TreeVerts& T, float, float) {
         const Surf& v = T.v[d];
-        vtx[d - 1] = make_float4(__int_as_float(v.tri), v.b1, v.b2, T.pdfA[d]);
+        tab.vtx[threadIdx.x * kMaxDepth + d - 1] = make_float4(__int_as_float(v.tri), v.b1, v.b2, T.pdfA[d]);
     }
 };
 __device__ __forceinline__ void initial_lanes_body(const InitArgs& a, int bx, int by, LaneTable& tab) {
     const FrameDev& F = a.F;
     const ParamsDev& P = a.P;
-    const int nc = P.n_cand, depth = P.depth;
-    const LaneTile tile = lane_tile(nc);
-    const int npx = tile.w * tile.h;
-    const int pl = (int)threadIdx.x / nc, t = (int)threadIdx.x % nc;
-    if (pl < npx) {
-        const int ix = bx * tile.w + pl % tile.w, iy = by * tile.h + pl / tile.w;
-        LaneSink sink;
-        sink.cand = tab.cand + threadIdx.x * kMaxDepth;
-        sink.vtx = tab.vtx + threadIdx.x * kMaxDepth;
-        for (int d = 0; d < depth; ++d) sink.cand[d] = make_float2(0.f, 0.f);
-        if (ix < F.W && iy < F.H) {
+    const int tid = (int)threadIdx.x;
+#pragma unroll 1
+    for (int f0 = 0;; f0 += kLaneThreads) {
+        tab.masks[tid] = 0;
+        if (f0 + tid < a.lane_w * a.lane_h * P.n_cand) {
+            const int nc = P.n_cand, tw = a.lane_w;
+            const int pl = (f0 + tid) / nc, t = (f0 + tid) % nc;
+            const int ix = bx * tw + pl % tw, iy = by * a.lane_h + pl / tw;
+            if (ix < F.W && iy < F.H) {
+                const int pix = iy * F.W + ix;
+                const float4 gb = F.gb[pix];
+                const uint32_t tri = __float_as_uint(gb.x);
+                Domain D = make_domain_hit(&F, tri != kNoHit, (int)tri, gb.y, gb.z, gb.w, F.L0, F.dL);
+                if (D.valid) {
+                    TreeVerts T;
+                    LaneSink sink{tab};
+                    trace_tree<0, true>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
+                }
+            }
+        }
+        const uint32_t got = __ballot_sync(0xFFFFFFFFu, tab.masks[tid] != 0);
+        if ((tid & 31) == 0) tab.any[tid >> 5] = got;
+        __syncthreads();
+        const int nc = P.n_cand, tw = a.lane_w, npx = tw * a.lane_h;
+        const float invN = 1.0f / (float)nc;
+        const int q = f0 / nc + tid;   // a pixel of this round
+        const int ix = bx * tw + q % tw, iy = by * a.lane_h + q / tw;
+        if (q < npx && q * nc < f0 + kLaneThreads && ix < F.W && iy < F.H) {
             const int pix = iy * F.W + ix;
-            const float4 gb = F.gb[pix];
-            const uint32_t tri = __float_as_uint(gb.x);
-            Domain D = make_domain_hit(&F, tri != kNoHit, (int)tri, gb.y, gb.z, gb.w, F.L0, F.dL);
-            if (D.valid) {
-                TreeVerts T;
-                trace_tree<0, true>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
+            const int base = q * nc - f0;   // the thread of the pixel's first tree (negative: in the round before)
+            const LaneCarry& left = tab.carry[(f0 / kLaneThreads) & 1];
+            const float4* sel_vtx = left.vtx;
+            float S = 0.f, sel_tau = 0.f;
+            int sel_t = -1, sel_k = 0;
+            if (base < 0) { S = left.S; sel_tau = left.tau; sel_t = left.t; sel_k = left.k; }
+            const int lo = max(base, 0), hi = min(base + nc, kLaneThreads);
+            for (int w = lo >> 5; w <= (hi - 1) >> 5; ++w) {
+                uint32_t bits = tab.any[w];
+                if (w == lo >> 5) bits &= 0xFFFFFFFFu << (lo & 31);
+                if (w == (hi - 1) >> 5) bits &= 0xFFFFFFFFu >> (31 - ((hi - 1) & 31));
+                for (; bits; bits &= bits - 1u) {
+                    const int j = 32 * w + __ffs(bits) - 1, u = j - base;
+                    for (uint32_t m = tab.masks[j]; m; m &= m - 1u) {
+                        const int d = __ffs(m);
+                        const float2 ac = tab.cand[j * kMaxDepth + d - 1];
+                        const float wv = invN * ac.x;
+                        if (!(wv > 0.f)) continue;
+                        const uint4 r = philox((uint32_t)pix, F.frame, ((uint32_t)u << 8) | (uint32_t)d, P_RIS, P.seed);
+                        S += wv;
+                        if (u01(r.x) * S < wv) { sel_t = u; sel_k = d; sel_tau = ac.y; sel_vtx = tab.vtx + j * kMaxDepth; }
+                    }
+                }
+            }
+            if (base + nc > kLaneThreads) {   // the next round goes on
+                LaneCarry& c = tab.carry[(f0 / kLaneThreads + 1) & 1];
+                c.S = S; c.tau = sel_tau; c.t = sel_t; c.k = sel_k;
+                for (int j = 2; j <= sel_k; ++j) c.vtx[j - 1] = sel_vtx[j - 1];
+            } else {
+                float outv = 0.f;
+                uint32_t occ = 0u;
+                a.dst.M[pix] = (float)nc;
+                if (sel_t >= 0) {
+                    const float4 gb = F.gb[pix];
+                    Domain D = make_domain_hit(&F, true, __float_as_int(gb.x), gb.y, gb.z, gb.w, F.L0, F.dL);
+                    const GeomDev& g = F.g;
+                    TreeVerts T;
+                    T.v[1] = D.y1;
+                    T.cls[1] = mat_class(load_mat(g, D.y1.mat));
+                    T.pdfA[1] = 1.0f;
+                    for (int j = 2; j <= sel_k; ++j) {
+                        const float4 v = sel_vtx[j - 1];
+                        T.v[j] = surf_at(g, __float_as_int(v.x), v.y, v.z);
+                        T.cls[j] = mat_class(load_mat(g, T.v[j].mat));
+                        T.pdfA[j] = v.w;
+                    }
+                    Rec r;
+                    build_rec(D, T, sel_k, sel_t, (uint32_t)pix, F.frame, sel_tau, P, r);
+                    store_tail(a.dst, (size_t)pix, r);
+                    if (r.phat > 0.f) {
+                        const float W = S / r.phat;
+                        *res_at(a.dst, 0, (size_t)pix) = make_float4(W, r.phat, sel_tau, r.Lsuf);
+                        occ = 1u;
+                        outv = r.phat * W;
+                    }
+                }
+                a.dst.occ[pix] = occ;
+                if (a.out) a.out[pix] = outv;
             }
         }
+        if (f0 + kLaneThreads >= npx * nc) break;
+        __syncthreads();
     }
-    __syncthreads();
-    if ((int)threadIdx.x >= npx) return;
-    const int q = (int)threadIdx.x;
-    const int ix = bx * tile.w + q % tile.w, iy = by * tile.h + q / tile.w;
-    if (ix >= F.W || iy >= F.H) return;
-    const int pix = iy * F.W + ix;
-    a.dst.M[pix] = (float)nc;
-    const float4 gb = F.gb[pix];
-    const uint32_t tri = __float_as_uint(gb.x);
-    const float invN = 1.0f / (float)nc;
-    float S = 0.f, sel_tau = 0.f, outv = 0.f;
-    int sel_t = -1, sel_k = 0;
-    uint32_t occ = 0u;
-    if (tri != kNoHit) {
-        for (int u = 0; u < nc; ++u)
-            for (int d = (P.flags & 1u) ? 1 : 2; d <= depth; ++d) {
-                const float2 ac = tab.cand[(q * nc + u) * kMaxDepth + d - 1];
-                const float wv = invN * ac.x;
-                if (!(wv > 0.f)) continue;
-                const uint4 r = philox((uint32_t)pix, F.frame, ((uint32_t)u << 8) | (uint32_t)d, P_RIS, P.seed);
-                S += wv;
-                if (u01(r.x) * S < wv) { sel_t = u; sel_k = d; sel_tau = ac.y; }
-            }
-    }
-    if (sel_t >= 0) {
-        Domain D = make_domain_hit(&F, true, (int)tri, gb.y, gb.z, gb.w, F.L0, F.dL);
-        const GeomDev& g = F.g;
-        TreeVerts T;
-        T.v[1] = D.y1;
-        T.cls[1] = mat_class(load_mat(g, D.y1.mat));
-        T.pdfA[1] = 1.0f;
-        for (int j = 2; j <= sel_k; ++j) {
-            const float4 v = tab.vtx[(q * nc + sel_t) * kMaxDepth + j - 1];
-            T.v[j] = surf_at(g, __float_as_int(v.x), v.y, v.z);
-            T.cls[j] = mat_class(load_mat(g, T.v[j].mat));
-            T.pdfA[j] = v.w;
-        }
-        Rec r;
-        build_rec(D, T, sel_k, sel_t, (uint32_t)pix, F.frame, sel_tau, P, r);
-        store_tail(a.dst, (size_t)pix, r);
-        if (r.phat > 0.f) {
-            const float W = S / r.phat;
-            *res_at(a.dst, 0, (size_t)pix) = make_float4(W, r.phat, sel_tau, r.Lsuf);
-            occ = 1u;
-            outv = r.phat * W;
-        }
-    }
-    a.dst.occ[pix] = occ;
-    if (a.out) a.out[pix] = outv;
 }
 __global__ void __launch_bounds__(kLaneThreads, 6) initial_lanes_kernel(const __grid_constant__ InitArgs a) {
     __shared__ LaneTable tab;
@@ -413,13 +441,31 @@ __global__ void __launch_bounds__(kLaneThreads, 6) initial_lanes_batch_kernel(co
     __syncthreads();
     if (s.wave) return;   // launched as the bounce wavefront after this kernel (the whole block)
     const int lb = (int)blockIdx.x - __ldg(&blk0[j]);
-    const int tx = (s.F.W + lane_tile(s.P.n_cand).w - 1) / lane_tile(s.P.n_cand).w;
+    const int tx = (s.F.W + s.lane_w - 1) / s.lane_w;
     initial_lanes_body(s, lb % tx, lb / tx, tab);
 }
-// blocks of the lane form over a view
-int initial_lanes_blocks(int W, int H, int n_cand) {
-    const LaneTile t = lane_tile(n_cand);
-    return ((W + t.w - 1) / t.w) * ((H + t.h - 1) / t.h);
+// A block's tile for nc trees a pixel in launches of npix pixels on sms SMs: the number of pixels with the fewest
+// rounds over the launch (blocks / resident blocks rounded up, times a block's rounds), of equals the
+// smallest; rows of 8 pixels where they divide it (their records share lines), else the squarest shape that is
+// at least as wide as high.  32 views of 250 x 250, ms, a thread per pixel / whole pixels in one round / this: 21 trees
+// 21.9 / 24.6 / 19.5, 43 trees 40.1 / 47.0 / 37.6, 64 trees 57.1 / - / 50.9; one 128 x 128 view, us: 33 trees 1384 / 575 /
+// 492, 43 trees 1703 / 592 / 549.
+void initial_lanes_tile(long long npix, int nc, int sms, int* w, int* h) {
+    const long long resident = 6ll * (sms > 0 ? sms : 1);
+    long long best = -1;
+    const int first = kLaneThreads / nc;   // at least 2 (kMaxCand = 64)
+    for (int k = first; k <= first + 8; ++k) {
+        int tw = k % 8 == 0 && k <= 64 ? 8 : 0;
+        for (int d = 1; d <= 16 && !tw; ++d)
+            if (k % d == 0 && d * d >= k) tw = d;
+        if (!tw) continue;
+        const long long waves = ((npix + k - 1) / k + resident - 1) / resident;
+        const long long rounds = ((long long)k * nc + kLaneThreads - 1) / kLaneThreads;
+        if (best < 0 || waves * rounds < best) { best = waves * rounds; *w = tw; *h = k / tw; }
+    }
+}
+int initial_lanes_blocks(const InitArgs& a) {
+    return ((a.F.W + a.lane_w - 1) / a.lane_w) * ((a.F.H + a.lane_h - 1) / a.lane_h);
 }
 
 // 6 resident blocks per SM (80 registers): 1.08 against 1.11 ms at 5 blocks (96 registers) on the
@@ -1107,9 +1153,8 @@ cudaError_t launch_initial(const InitArgs& a, int tile_h, unsigned* err, cudaStr
     const dim3 grid = tile_grid(a.F.W, a.F.H, a.tile_w, tile_h);
     const int threads = a.tile_w * tile_h;
     if (a.F.B == 0) {
-        const LaneTile t = lane_tile(a.P.n_cand);
         if (a.P.flags & kFlagEllipsoid) initial_gated_ell_kernel<<<grid, threads, 0, s>>>(a);
-        else initial_lanes_kernel<<<tile_grid(a.F.W, a.F.H, t.w, t.h), kLaneThreads, 0, s>>>(a);
+        else initial_lanes_kernel<<<tile_grid(a.F.W, a.F.H, a.lane_w, a.lane_h), kLaneThreads, 0, s>>>(a);
     } else {
         if (a.P.flags & kFlagEllipsoid) initial_kernel<true><<<grid, threads, 0, s>>>(a, err);
         else initial_kernel<false><<<grid, threads, 0, s>>>(a, err);
