@@ -240,9 +240,10 @@ tof_status tof_render_gated_noalloc(tof_ctx* ctx, tof_scene scene, tof_view view
 
 /* Render one transient frame (Sec. 4.5): per-bin reservoirs, per-bin temporal / spatial reuse,
  * and the histogram out_hist_dev[H*W*B] (bin fastest, float32).  Without the ellipsoidal connection,
- * views of up to 16M pixels x trees run the initial stage as the bounce wavefront where there is room
- * for its scratch (144 + 24 * depth bytes per pixel and tree, counted by tof_device_bytes); without room, and
- * in batches, a single kernel that needs none gives the same histograms.  The scratch is given back when
+ * views of up to 16M pixels x trees run the initial stage as the bounce wavefront where that is the faster form
+ * (8 path trees and more, fewer in small views or with long paths) and there is room for its scratch
+ * (144 + 24 * depth bytes per pixel and tree, counted by tof_device_bytes); otherwise, and in batches, a single
+ * kernel that needs none gives the same histograms.  The scratch is given back when
  * any other allocation of the context would not fit otherwise, and the view keeps to the single kernel
  * from then on. */
 tof_status tof_render_transient(tof_ctx* ctx, tof_scene scene, tof_view view, const tof_sensor* sensor,

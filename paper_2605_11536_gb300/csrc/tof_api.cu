@@ -839,8 +839,16 @@ static bool tree_wave_ready(const ViewH& V, const tof_params* p) {
 // trees of depth 4, against 300 B a bin of the view itself) is to be had beside everything that the context's
 // calls cannot do without (give_back_optional); batches and the served form, which account their views'
 // memory beforehand, keep the single kernel
+// With few path trees the single kernel, one thread's chain of n_cand trees, is shorter than the wavefront's
+// 2 * depth + 1 launches and queues.  A frame's time, single kernel / wavefront, us (confocal scan; closed
+// box; box of glossy and mirror walls): 1 tree of depth 4, 64 x 64 99 / 204; 104 / 175; 119 / 186, 3 trees 197 / 236; 216 / 185;
+// 322 / 198; 4 trees 245 / 249; 272 / 192; 427 / 203, 256 x 256 372 / 474; 550 / 559; 1083 / 609; 6 trees 513 / 537; 808 / 665; 1742 / 729; 6
+// trees of depth 2, 256 x 256 349 / 340; 272 / 319; 323 / 317, 8 trees of depth 2 436 / 375; 348 / 349; 413 / 345.
+static bool hist_wave_pays(const ViewH& V, const tof_params* p) {
+    return p->n_cand >= 8 || (p->n_cand >= 6 && p->depth >= 3) || (p->n_cand >= 4 && (size_t)V.W * V.H <= 80 * 80);
+}
 static bool hist_tree_wave(tof_ctx* c, ViewH& V, const tof_params* p, bool capturing) {
-    if (c->in_batch || g_rec) return false;
+    if (c->in_batch || g_rec || !hist_wave_pays(V, p)) return false;
     const std::string before = c->err;
     const size_t paths = (size_t)V.W * V.H * (size_t)p->n_cand;
     const bool fits = tree_wave_fits(V, p->n_cand, p->depth);

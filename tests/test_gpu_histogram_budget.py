@@ -122,3 +122,18 @@ def test_changing_trees_and_depth_allocates_once():
         assert seen[2:] == [seen[2]] * 4, seen
     finally:
         tof.tof_destroy(ctx)
+
+
+@pytest.mark.parametrize("trees,depth,wave", [(1, 5, False), (3, 4, False), (4, 4, True), (8, 4, True)])
+def test_few_trees_take_the_single_kernel(trees, depth, wave):
+    from paper_2605_11536_gb300 import tof
+    sc = _scene(0, 0)
+    sc.params.n_cand, sc.params.depth = trees, depth
+    ctx, sid = _context(sc, 0)
+    try:
+        vid = tof.tof_view_create(ctx, sid, W, H, B)
+        before = tof.tof_device_bytes(ctx)
+        assert np.count_nonzero(_frames(sc, ctx, sid, vid, 1)) > 20
+        assert (tof.tof_device_bytes(ctx) > before) == wave
+    finally:
+        tof.tof_destroy(ctx)

@@ -30,18 +30,18 @@ def test_a_recorded_frame_keeps_its_scratch(recorded_with_scratch):
 
         ref, out, rec = (torch.full((W * H * B,), -1.0, device="cuda") for _ in range(3))
         if not recorded_with_scratch:   # the reuse scratch alone, by the form that takes no other
-            p.n_cand, p.depth = 3, 3
+            p.n_cand, p.depth = 4, 3
             tof.tof_render_batch(ctx, [tof.job(sid, vid, sc.sensors[0], sc.emitters[0], p, 3, 5, ref.data_ptr(), bins=bins)])
         else:
-            render(3, 3, 5, ref)
+            render(4, 3, 5, ref)
         tof.tof_sync(ctx)
         held = tof.tof_device_bytes(ctx)
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph):
-            render(3, 3, 5, rec, torch.cuda.current_stream().cuda_stream)
+            render(4, 3, 5, rec, torch.cuda.current_stream().cuda_stream)
         assert tof.tof_device_bytes(ctx) == held
         seen = []
-        for trees, depth in ((8, 4), (2, 4), (8, 2), (3, 3)):
+        for trees, depth in ((8, 4), (5, 4), (8, 2), (4, 3)):
             render(trees, depth, 5, out)
             tof.tof_sync(ctx)
             seen.append(tof.tof_device_bytes(ctx))
@@ -55,7 +55,7 @@ def test_a_recorded_frame_keeps_its_scratch(recorded_with_scratch):
             graph.replay()
             torch.cuda.synchronize()
             np.testing.assert_array_equal(rec.cpu().numpy(), ref.cpu().numpy())
-        np.testing.assert_array_equal(out.cpu().numpy(), ref.cpu().numpy())   # (3, 3) again
+        np.testing.assert_array_equal(out.cpu().numpy(), ref.cpu().numpy())   # (4, 3) again
     finally:
         torch.cuda.synchronize()
         tof.tof_destroy(ctx)
