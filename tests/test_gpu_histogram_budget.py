@@ -126,6 +126,7 @@ def test_changing_trees_and_depth_allocates_once():
 
 @pytest.mark.parametrize("trees,depth,wave", [(1, 5, False), (3, 4, False), (4, 4, True), (8, 4, True)])
 def test_few_trees_take_the_single_kernel(trees, depth, wave):
+    import torch
     from paper_2605_11536_gb300 import tof
     sc = _scene(0, 0)
     sc.params.n_cand, sc.params.depth = trees, depth
@@ -133,7 +134,12 @@ def test_few_trees_take_the_single_kernel(trees, depth, wave):
     try:
         vid = tof.tof_view_create(ctx, sid, W, H, B)
         before = tof.tof_device_bytes(ctx)
-        assert np.count_nonzero(_frames(sc, ctx, sid, vid, 1)) > 20
+        img = _frames(sc, ctx, sid, vid, 1)[0]
         assert (tof.tof_device_bytes(ctx) > before) == wave
+        out = torch.full((W * H * B,), -1.0, device="cuda")   # a batch: always the single kernel
+        tof.tof_render_batch(ctx, [tof.job(sid, vid, sc.sensors[0], sc.emitters[0], sc.params, 3, 0, out.data_ptr(), bins=BINS)])
+        tof.tof_sync(ctx)
+        np.testing.assert_array_equal(img, out.cpu().numpy())
+        assert img.any()
     finally:
         tof.tof_destroy(ctx)
