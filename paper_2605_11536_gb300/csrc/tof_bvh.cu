@@ -5,7 +5,7 @@
 //   xform_kernel    rigid 3x4 object transform of every triangle corner, per frame
 //   bounds / morton 30-bit Morton codes of triangle centroids in the centroid bounds (cubic cells)
 //   radix sort      4 stable 8-bit LSD passes (tile histograms, offsets, ranked scatter), one cooperative
-//                   launch where its blocks can all be resident
+//                   launch up to 307k triangles
 //   karras_kernel   binary radix tree over the sorted codes (Karras, HPG 2012), ties broken by index; lists
 //                   the ranges of at most 512 leaves below which it is rebuilt
 //   range_box / treelet / treelet_top_kernel   those ranges, and the levels above them, top-down by the surface
@@ -118,32 +118,56 @@ __global__ void __launch_bounds__(256) radix_hist_kernel(const uint32_t* __restr
     hist[threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive scan of n words in place (single block of 1024 threads)
-__global__ void __launch_bounds__(1024) scan_kernel(uint32_t* __restrict__ data, int n) {
-    __shared__ uint32_t part[1024];
-    int per = (n + 1023) / 1024;
-    int b = threadIdx.x * per, e = min(n, b + per);
-    uint32_t s = 0;
-    for (int i = b; i < e; ++i) s += data[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        uint32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+// exclusive scan of a block's 256 values; all = their sum
+__device__ __forceinline__ uint32_t scan256(uint32_t x, uint32_t* wsum, uint32_t& all) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += v;
     }
-    uint32_t run = part[threadIdx.x] - s;
-    for (int i = b; i < e; ++i) { uint32_t v = data[i]; data[i] = run; run += v; }
+    __syncthreads();   // wsum's last values are read
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t low = 0u;
+    all = 0u;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        low += w < warp ? wsum[w] : 0u;
+        all += wsum[w];
+    }
+    return low + incl - x;
+}
+// one digit's counts over the tiles (row) become each tile's offset within the digit; returns their sum
+__device__ __forceinline__ uint32_t scan_digit(uint32_t* row, int ntiles, uint32_t* wsum) {
+    uint32_t run = 0u;
+    for (int t0 = 0; t0 < ntiles; t0 += 256) {
+        const int t = t0 + (int)threadIdx.x;
+        uint32_t all;
+        const uint32_t before = scan256(t < ntiles ? __ldcg(&row[t]) : 0u, wsum, all);
+        if (t < ntiles) row[t] = run + before;
+        run += all;
+    }
+    return run;
+}
+// a block per digit (one block for all 256 * ntiles counts: 1.74 ms of a 4M-triangle sort's four passes)
+__global__ void __launch_bounds__(256) radix_scan_kernel(uint32_t* __restrict__ hist, uint32_t* __restrict__ totals, int ntiles) {
+    __shared__ uint32_t wsum[8];
+    const uint32_t sum = scan_digit(hist + (size_t)blockIdx.x * ntiles, ntiles, wsum);
+    if (threadIdx.x == 0) totals[blockIdx.x] = sum;
 }
 
 __global__ void __launch_bounds__(256) radix_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                                             uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, int n,
-                                                            int shift, const uint32_t* __restrict__ offs, int ntiles) {
+                                                            int shift, const uint32_t* __restrict__ offs,
+                                                            const uint32_t* __restrict__ totals, int ntiles) {
     __shared__ uint32_t base[256];
+    __shared__ uint32_t wsum[8];
     __shared__ uint32_t wc[8][256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = offs[tid * ntiles + blockIdx.x];
+    uint32_t all;
+    base[tid] = scan256(totals[tid], wsum, all) + offs[(size_t)tid * ntiles + blockIdx.x];
     const uint32_t lt = (1u << lane) - 1u;
     for (int r = 0; r < kTile / 256; ++r) {
         for (int k = 0; k < 8; ++k) wc[k][tid] = 0u;
@@ -170,15 +194,15 @@ __global__ void __launch_bounds__(256) radix_scatter_kernel(const uint32_t* __re
     }
 }
 
-// The same four passes in one cooperative launch of one block per tile of kCoopTile keys (all resident): per
-// pass the tile histograms, a grid-wide sync, each block's digit offsets -- the digit totals' exclusive
-// scan plus the digit's count in the earlier tiles, the global scan above restated per block --
-// the same stable scatter, and a grid-wide sync.  Sorted keys and values are those of the
-// separate launches (after four passes back in k0 / v0).  Bound by the latency of its barriers and
-// dependent steps: a tile of 512 keys has two ranking rounds a pass where one of 2048 has eight, and its
-// keys stay in registers from the histogram to the scatter; more than kCoopTiles tiles take 2048, since each
-// block reads every tile's histogram.
-template <int kCoopTile>
+// The same four passes in one cooperative launch of one block per tile of 512 keys (all resident): per
+// pass the tile histograms, a grid-wide sync, each tile's digit offsets, the same stable scatter, and a
+// grid-wide sync.  Sorted keys and values are those of the separate launches (after four passes back in k0 / v0).
+// Bound by the latency of its barriers and dependent steps: a tile of 512 keys has two ranking rounds a pass
+// where one of 2048 has eight, and its keys stay in registers from the histogram to the scatter.  Offsets:
+// every block adds up all tiles' histograms itself, or (kScan) the digits' rows are scanned by a block
+// each, a third grid-wide sync for a time that does not grow with the tiles (kAddTiles).
+constexpr int kCoopTile = 512;
+template <bool kScan>
 __global__ void __launch_bounds__(256) radix_sort_coop_kernel(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int n,
                                                               uint32_t* __restrict__ hist, int ntiles) {
     namespace cg = cooperative_groups;
@@ -191,6 +215,7 @@ __global__ void __launch_bounds__(256) radix_sort_coop_kernel(uint32_t* k0, uint
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
+    uint32_t* const totals = hist + (size_t)256 * ntiles;   // kScan
     const int t0 = blockIdx.x * kCoopTile;
     for (int shift = 0; shift < 32; shift += 8) {
         h[tid] = 0u;
@@ -203,29 +228,28 @@ __global__ void __launch_bounds__(256) radix_sort_coop_kernel(uint32_t* k0, uint
             if (g < n) atomicAdd(&h[(key[r] >> shift) & 255u], 1u);
         }
         __syncthreads();
-        hist[blockIdx.x * 256 + tid] = h[tid];
+        hist[kScan ? (size_t)tid * ntiles + blockIdx.x : (size_t)blockIdx.x * 256 + tid] = h[tid];
         __threadfence();
         grid.sync();
-        uint32_t tot = 0u, before = 0u;
+        uint32_t tot = 0u, before = 0u, all;
+        if constexpr (kScan) {
+            for (int d = blockIdx.x; d < 256; d += gridDim.x) {
+                const uint32_t sum = scan_digit(hist + (size_t)d * ntiles, ntiles, wsum);
+                if (tid == 0) totals[d] = sum;
+            }
+            __threadfence();
+            grid.sync();
+            tot = __ldcg(&totals[tid]);
+            before = __ldcg(&hist[(size_t)tid * ntiles + blockIdx.x]);
+        } else {
 #pragma unroll 8
-        for (int t = 0; t < ntiles; ++t) {
-            const uint32_t c = __ldcg(&hist[t * 256 + tid]);
-            tot += c;
-            if (t < (int)blockIdx.x) before += c;
+            for (int t = 0; t < ntiles; ++t) {
+                const uint32_t c = __ldcg(&hist[t * 256 + tid]);
+                tot += c;
+                if (t < (int)blockIdx.x) before += c;
+            }
         }
-        // exclusive scan of the digit totals
-        uint32_t incl = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane == 31) wsum[warp] = incl;
-        __syncthreads();
-        uint32_t low = 0u;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) low += w < warp ? wsum[w] : 0u;
-        base[tid] = low + incl - tot + before;
+        base[tid] = scan256(tot, wsum, all) + before;
 #pragma unroll
         for (int r = 0; r < kRounds; ++r) {
             for (int k = 0; k < 8; ++k) wc[k][tid] = 0u;
@@ -831,6 +855,30 @@ cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const 
     return cudaGetLastError();
 }
 
+// blocks of the cooperative sort (a form of it) that are resident at once, found once per device and process
+static int sort_blocks(const void* kernel, int form) {
+    static std::atomic<int> known[2][64];   // 1 + the number
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 0;
+    int v = known[form][dev].load();
+    if (!v) {
+        int sms = 0, per = 0, coop = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, 0);
+        cudaGetLastError();
+        v = 1 + (coop ? sms * per : 0);
+        known[form][dev].store(v);
+    }
+    return v - 1;
+}
+// Which sort, us for n triangles (every block adds up the histograms / rows scanned / separate launches, three a pass):
+// 10k 28 / 60 / 60, 40k 39 / 43 / 61, 66k 42 / 41 / 62, 98k 62 / 44 / 62, 198k 93 / 51 / 63, 270k 147 / 58 / 61, 400k 274 / 75 / 65;
+// separate 1M 83, 2M 113.  (Tiles of 2048 keys in one launch, as of old for more than 98,304: 198k 82, 400k 130, 1M 268;
+// tiles of 1024 with scanned rows: 400k 62, elsewhere slower than the best of these.)
+constexpr int kAddTiles = 110, kScanTiles = 600;
+
 // full build of the hierarchy (prim order, children, parents) from the centroids
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
@@ -843,61 +891,29 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
     bounds_kernel<<<min(1024u, blocks(n, 256)), 256, 0, s>>>(n, cent, bb);
     note_launch();
     morton_kernel<<<blocks(n, 256), 256, 0, s>>>(n, cent, bb, keys, vals);
-    int ntiles = (n + kTile - 1) / kTile;
     uint32_t *ki = keys, *vi = vals, *ko = keys2, *vo = vals2;
-    // one cooperative launch when every tile's block can be resident at once
-    // resident blocks of the cooperative sort on each device (found once per device and process)
-    static std::atomic<int> coop_blocks[64];
-    static std::atomic<bool> coop_known[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int coop_cap = 0;
-    if (dev >= 0 && dev < 64) {
-        if (!coop_known[dev].load()) {
-            int sms = 0, per = 0, coop = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, radix_sort_coop_kernel<2048>, 256, 0);
-            cudaGetLastError();
-            coop_blocks[dev].store(coop ? sms * per : 0);
-            coop_known[dev].store(true);
+    // the histograms (and the scans' totals) lie in the centroids' memory, which the Morton codes were the last to
+    // read: at most 2 B a key and 1 KB of its 16 B a key
+    uint32_t* counts = n >= 512 ? reinterpret_cast<uint32_t*>(scratch) : hist;
+    int nt = (n + kCoopTile - 1) / kCoopTile;
+    const void* sort = nt <= kAddTiles ? (const void*)radix_sort_coop_kernel<false> : (const void*)radix_sort_coop_kernel<true>;
+    if (nt <= kScanTiles && nt <= sort_blocks(sort, nt <= kAddTiles ? 0 : 1)) {
+        int nn = n;
+        void* args[] = {&ki, &vi, &ko, &vo, &nn, &counts, &nt};
+        note_launch();
+        e = cudaLaunchCooperativeKernel(sort, dim3(nt), dim3(256), args, 0, s);
+        if (e != cudaSuccess) return e;
+    } else {
+        const int ntiles = (n + kTile - 1) / kTile;
+        uint32_t* totals = counts + (size_t)256 * ntiles;
+        for (int shift = 0; shift < 32; shift += 8) {
+            note_launch(3);
+            radix_hist_kernel<<<ntiles, 256, 0, s>>>(ki, n, shift, counts, ntiles);
+            radix_scan_kernel<<<256, 256, 0, s>>>(counts, totals, ntiles);
+            radix_scatter_kernel<<<ntiles, 256, 0, s>>>(ki, vi, ko, vo, n, shift, counts, totals, ntiles);
+            uint32_t* t = ki; ki = ko; ko = t;
+            t = vi; vi = vo; vo = t;
         }
-        coop_cap = coop_blocks[dev].load();
-    }
-    // tiles of 512 keys up to kCoopTiles of them; their histograms (2 B a key) lie in the centroids' memory, which
-    // the Morton codes were the last to read
-    constexpr int kCoopTiles = 192;
-    const int small = (n + 511) / 512;
-    if (small <= kCoopTiles && small <= coop_cap && n >= 512) {
-        int nn = n, nt = small;
-        uint32_t* hh = reinterpret_cast<uint32_t*>(scratch);
-        void* args[] = {&ki, &vi, &ko, &vo, &nn, &hh, &nt};
-        note_launch();
-        e = cudaLaunchCooperativeKernel((const void*)radix_sort_coop_kernel<512>, dim3(small), dim3(256), args, 0, s);
-        if (e != cudaSuccess) return e;
-        if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
-        *prim_out = vi;
-        return cudaGetLastError();
-    }
-    if (ntiles <= coop_cap) {
-        int nn = n, nt = ntiles;
-        void* args[] = {&ki, &vi, &ko, &vo, &nn, &hist, &nt};
-        note_launch();
-        e = cudaLaunchCooperativeKernel((const void*)radix_sort_coop_kernel<2048>, dim3(ntiles), dim3(256), args, 0, s);
-        if (e != cudaSuccess) return e;
-        if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
-        *prim_out = vi;
-        return cudaGetLastError();
-    }
-    for (int shift = 0; shift < 32; shift += 8) {
-        note_launch();
-        radix_hist_kernel<<<ntiles, 256, 0, s>>>(ki, n, shift, hist, ntiles);
-        note_launch();
-        scan_kernel<<<1, 1024, 0, s>>>(hist, 256 * ntiles);
-        note_launch();
-        radix_scatter_kernel<<<ntiles, 256, 0, s>>>(ki, vi, ko, vo, n, shift, hist, ntiles);
-        uint32_t* t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
     }
     // after 4 passes the sorted keys / prims are back in keys / vals
     if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
