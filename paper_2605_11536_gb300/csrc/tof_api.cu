@@ -39,7 +39,7 @@ cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const 
                          const float* xf, float4* tri_out, float4* cent, cudaStream_t s);
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
-                                  uint32_t** prim_out, float4* scratch, cudaStream_t s);
+                                  uint32_t* counter, uint32_t** prim_out, float4* scratch, cudaStream_t s);
 cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
                             int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut, float4* boxes,
                             int sms, cudaStream_t s);
@@ -615,7 +615,7 @@ tof_status tof_bvh_build(tof_ctx* c, tof_scene id, const float* xf, int refit_on
     CK(launch_xform(S.nt, S.vloc, S.tris, S.triobj, S.objmat, S.xf, S.tri[slot], S.cent, s));
     if (!S.built || !refit_only) {
         CK(launch_build_topology(S.nt, S.cent, S.bb, S.keys, S.vals, S.keys2, S.vals2, S.hist, S.child, S.parent_int,
-                                 S.parent_leaf, &S.prim, S.cent, s));
+                                 S.parent_leaf, S.counter, &S.prim, S.cent, s));
     }
     const bool full = !S.built || !refit_only;
     if (full && S.nt > 1) {

@@ -303,9 +303,10 @@ __device__ __forceinline__ void list_cut(int first, int last, int code, uint32_t
 }
 __global__ void karras_kernel(int n, const uint32_t* __restrict__ keys, int* __restrict__ child, int* __restrict__ parent_int,
                               int* __restrict__ parent_leaf, uint32_t* __restrict__ cut_a, uint32_t* __restrict__ cut_m,
-                              uint32_t* ncut) {
+                              uint32_t* ncut, uint32_t* __restrict__ counter) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
+    if (counter) counter[i] = 0u;
     int d = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) >= 0 ? 1 : -1;
     int dmin = delta(keys, n, i, i - d);
     int lmax = 2;
@@ -719,12 +720,35 @@ __global__ void __launch_bounds__(kTreelet) treelet_kernel(int n, uint32_t* __re
 // what follows it in the stream finds both.  Both are chains of short barriers on few SMs (66k triangles: 75 and
 // 49 us), so side by side they take little more than the longer: 301 x 203 frame 1.311 -> 1.284 ms, four served
 // streams 6.39 -> 6.28, the boxes' own launch included.
+// Of more than kTopItems ranges the Morton hierarchy's own nodes above stay, their boxes found bottom-up as in
+// refit_kernel: by treelet_top_kernel's block in a scene of up to kClimbBlock triangles, by morton_top_kernel
+// in a larger one (4M triangles: 753 us in one block).
+constexpr int kClimbBlock = 1 << 18;
+__device__ __forceinline__ void climb_range(int r, int n, const uint32_t* prim, const float4* __restrict__ tri, float4* nodes, const int* child,
+                                            const int* parent_int, const int* parent_leaf, uint32_t* counter,
+                                            const uint32_t* __restrict__ cut_a, const uint32_t* __restrict__ cut_m) {
+    const int a = (int)cut_a[r], m = (int)(cut_m[r] & ~kRootLast);
+    int q = m == 1 ? parent_leaf[a] : parent_int[(cut_m[r] & kRootLast) ? a + m - 1 : a];
+    int guard = n;
+    while (q >= 0 && --guard >= 0) {
+        if (arrive_acq_rel(&counter[q]) == 0u) break;
+        const int c[2] = {child[2 * q], child[2 * q + 1]};
+        Box b[2];
+        for (int k = 0; k < 2; ++k) b[k] = c[k] < 0 ? tri_box(tri, (int)prim[~c[k]]) : node_box(nodes + 4 * (size_t)c[k]);
+        float4* N = nodes + 4 * (size_t)q;
+        N[0] = make_float4(b[0].lo[0], b[0].hi[0], b[0].lo[1], b[0].hi[1]);
+        N[1] = make_float4(b[1].lo[0], b[1].hi[0], b[1].lo[1], b[1].hi[1]);
+        N[2] = make_float4(b[0].lo[2], b[0].hi[2], b[1].lo[2], b[1].hi[2]);
+        N[3] = make_float4(__int_as_float(c[0]), __int_as_float(c[1]), 0.f, 0.f);
+        q = parent_int[q];
+    }
+}
 __device__ __forceinline__ void wait_for_treelets() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __global__ void __launch_bounds__(kTopItems) treelet_top_kernel(int n, const uint32_t* prim, const float4* __restrict__ tri,
                                                                 const float4* __restrict__ boxes, float4* nodes, int* child,
                                                                 int* parent_int, int* parent_leaf, uint32_t* counter,
                                                                 const uint32_t* __restrict__ cut_a, const uint32_t* __restrict__ cut_m,
-                                                                const uint32_t* __restrict__ ncut) {
+                                                                const uint32_t* __restrict__ ncut, bool climb) {
     extern __shared__ __align__(16) unsigned char sm[];
     Sweep<kTopItems>& S = *reinterpret_cast<Sweep<kTopItems>*>(sm);
     __shared__ int s_no_slot, s_slot0;   // the item without a free number; the item whose free number is 0
@@ -763,26 +787,20 @@ __global__ void __launch_bounds__(kTopItems) treelet_top_kernel(int n, const uin
         return;
     }
     wait_for_treelets();
-    // too many: the Morton hierarchy's own nodes above the treelets, bottom-up as in refit_kernel
+    if (!climb) return;
     for (int i = p; i < n - 1; i += kTopItems) counter[i] = 0u;
     __syncthreads();
-    for (int r = p; r < R; r += kTopItems) {
-        const int a = (int)cut_a[r], m = (int)(cut_m[r] & ~kRootLast);
-        int q = m == 1 ? parent_leaf[a] : parent_int[(cut_m[r] & kRootLast) ? a + m - 1 : a];
-        int guard = n;
-        while (q >= 0 && --guard >= 0) {
-            if (arrive_acq_rel(&counter[q]) == 0u) break;
-            const int c[2] = {child[2 * q], child[2 * q + 1]};
-            Box b[2];
-            for (int k = 0; k < 2; ++k) b[k] = c[k] < 0 ? tri_box(tri, (int)prim[~c[k]]) : node_box(nodes + 4 * (size_t)c[k]);
-            float4* N = nodes + 4 * (size_t)q;
-            N[0] = make_float4(b[0].lo[0], b[0].hi[0], b[0].lo[1], b[0].hi[1]);
-            N[1] = make_float4(b[1].lo[0], b[1].hi[0], b[1].lo[1], b[1].hi[1]);
-            N[2] = make_float4(b[0].lo[2], b[0].hi[2], b[1].lo[2], b[1].hi[2]);
-            N[3] = make_float4(__int_as_float(c[0]), __int_as_float(c[1]), 0.f, 0.f);
-            q = parent_int[q];
-        }
-    }
+    for (int r = p; r < R; r += kTopItems) climb_range(r, n, prim, tri, nodes, child, parent_int, parent_leaf, counter, cut_a, cut_m);
+}
+// the same over the whole GPU, with the counters zeroed before it (karras_kernel)
+__global__ void __launch_bounds__(256) morton_top_kernel(int n, const uint32_t* prim, const float4* __restrict__ tri, float4* nodes, const int* child,
+                                                         const int* parent_int, const int* parent_leaf, uint32_t* counter,
+                                                         const uint32_t* __restrict__ cut_a, const uint32_t* __restrict__ cut_m,
+                                                         const uint32_t* __restrict__ ncut) {
+    const int R = (int)*ncut;
+    if (R == 1 || top_by_area(R, n)) return;
+    for (int r = blockIdx.x * 256 + threadIdx.x; r < R; r += gridDim.x * 256)
+        climb_range(r, n, prim, tri, nodes, child, parent_int, parent_leaf, counter, cut_a, cut_m);
 }
 
 // ---- ellipsoidal-connection hierarchy (Sec. 5 "Ellipsoidal Path Connection": nodes weighted by
@@ -882,7 +900,7 @@ constexpr int kAddTiles = 110, kScanTiles = 600;
 // full build of the hierarchy (prim order, children, parents) from the centroids
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
-                                  uint32_t** prim_out, float4* scratch, cudaStream_t s) {
+                                  uint32_t* counter, uint32_t** prim_out, float4* scratch, cudaStream_t s) {
     // centroid bounds start empty: encoded minima at 0xFFFFFFFF, maxima at 0
     cudaError_t e = cudaMemsetAsync(bb, 0xFF, 3 * sizeof(uint32_t), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(bb + 3, 0, 4 * sizeof(uint32_t), s);   // and the number of treelets
@@ -916,7 +934,7 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
         }
     }
     // after 4 passes the sorted keys / prims are back in keys / vals
-    if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6); }
+    if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6, n > kClimbBlock ? counter : nullptr); }
     *prim_out = vi;
     return cudaGetLastError();
 }
@@ -935,6 +953,7 @@ cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* le
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) sized[dev].store(true);
     }
+    const bool climb = n > kClimbBlock;   // by a kernel of its own
     // ranges hold at least a few leaves each, mostly hundreds: a block takes several where there are many
     const int grid = min((int)blocks(n, 64), 4 * sms);
     note_launch(3);
@@ -946,9 +965,14 @@ cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* le
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1); cfg.blockDim = dim3(kTopItems); cfg.dynamicSmemBytes = sizeof(Sweep<kTopItems>); cfg.stream = s;
     cfg.attrs = beside; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, treelet_top_kernel, n, (const uint32_t*)prim, tri, (const float4*)boxes, nodes, child, parent_int,
-                                             parent_leaf, counter, cut_a, cut_m, ncut);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, treelet_top_kernel, n, (const uint32_t*)prim, tri, (const float4*)boxes, nodes, child, parent_int,
+                                             parent_leaf, counter, cut_a, cut_m, ncut, !climb);
     if (e != cudaSuccess) return e;
+    if (climb) {
+        note_launch();
+        morton_top_kernel<<<min((int)blocks(n, 64 * 256), 4 * sms), 256, 0, s>>>(n, prim, tri, nodes, child, parent_int, parent_leaf, counter, cut_a,
+                                                                                 cut_m, ncut);
+    }
     return cudaGetLastError();
 }
 
