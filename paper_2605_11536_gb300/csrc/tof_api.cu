@@ -36,13 +36,16 @@ cudaError_t launch_splat(const SplatArgs& a, cudaStream_t s);
 cudaError_t launch_pt(const PtArgs& a, cudaStream_t s);
 cudaError_t launch_laser(const GeomDev& g, float3 o, float3 d, float power, LightDev* out, cudaStream_t s);
 cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const uint32_t* triobj, const uint32_t* objmat,
-                         const float* xf, float4* tri_out, float4* cent, cudaStream_t s);
+                         const float* xf, float4* tri_out, float4* cent, uint32_t* bb, cudaStream_t s);
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
                                   uint32_t* counter, uint32_t** prim_out, float4* scratch, cudaStream_t s);
 cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
                             int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut, float4* boxes,
                             int sms, cudaStream_t s);
+bool whole_build(int n);
+cudaError_t launch_whole(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int, int* parent_leaf,
+                         cudaStream_t s);
 cudaError_t launch_etree(int nt, int P, const float4* tri, float4* node, cudaStream_t s);
 cudaError_t launch_refit(int n, const uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, const int* child,
                          const int* parent_int, const int* parent_leaf, uint32_t* counter, cudaStream_t s);
@@ -612,17 +615,20 @@ tof_status tof_bvh_build(tof_ctx* c, tof_scene id, const float* xf, int refit_on
     if (S.built && S.xfh[S.cur] == xv) return TOF_OK;   // static between frames
     int slot = S.built ? 1 - S.cur : 0;
     CK(cudaMemcpyAsync(S.xf, xf, sizeof(float) * 12 * S.nobj, cudaMemcpyHostToDevice, s));
-    CK(launch_xform(S.nt, S.vloc, S.tris, S.triobj, S.objmat, S.xf, S.tri[slot], S.cent, s));
-    if (!S.built || !refit_only) {
+    CK(launch_xform(S.nt, S.vloc, S.tris, S.triobj, S.objmat, S.xf, S.tri[slot], S.cent, S.bb, s));
+    const bool full = !S.built || !refit_only;
+    if (full && whole_build(S.nt)) {
+        S.prim = S.vals;
+        CK(launch_whole(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, s));
+    } else if (full) {
         CK(launch_build_topology(S.nt, S.cent, S.bb, S.keys, S.vals, S.keys2, S.vals2, S.hist, S.child, S.parent_int,
                                  S.parent_leaf, S.counter, &S.prim, S.cent, s));
     }
-    const bool full = !S.built || !refit_only;
-    if (full && S.nt > 1) {
+    if (full && S.nt > 1 && !whole_build(S.nt)) {
         if (!c->sms) CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
         CK(launch_treelets(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, S.keys2,
                            S.vals2, S.bb + 6, S.cent, c->sms, s));
-    } else {
+    } else if (!full || S.nt == 1) {
         CK(launch_refit(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, s));
     }
     if (S.enode[slot]) CK(launch_etree(S.nt, S.eP, S.tri[slot], S.enode[slot], s));

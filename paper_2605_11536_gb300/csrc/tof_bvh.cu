@@ -29,10 +29,13 @@ __device__ __forceinline__ float3 fx3(const float* M, float3 p, int r) {
 }
 
 // per triangle: world corners -> (v0, mat), (e1), (e2); centroid
+// (and the empty centroid bounds, encoded minima at 0xFFFFFFFF and maxima at 0, and the number of treelets)
 __global__ void xform_kernel(int nt, const float* __restrict__ vloc, const uint32_t* __restrict__ tris,
                              const uint32_t* __restrict__ triobj, const uint32_t* __restrict__ objmat,
-                             const float* __restrict__ xf, float4* __restrict__ tri_out, float4* __restrict__ cent) {
+                             const float* __restrict__ xf, float4* __restrict__ tri_out, float4* __restrict__ cent,
+                             uint32_t* __restrict__ bb) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 7) bb[t] = t < 3 ? 0xFFFFFFFFu : 0u;
     if (t >= nt) return;
     uint32_t o = triobj[t];
     const float* M = xf + 12 * (size_t)o;
@@ -294,6 +297,7 @@ __device__ __forceinline__ int delta(const uint32_t* __restrict__ k, int n, int 
 // Ranges of at most kTreelet leaves whose parent's is larger are listed as treelets (cuts[r] = (first leaf,
 // leaves | kRootLast where the Karras node of the range is numbered by its last leaf), *ncut of them).
 constexpr int kTreelet = 512;
+constexpr int kWhole = 1024;   // a scene of so many triangles is one range (whole_kernel)
 constexpr uint32_t kRootLast = 0x80000000u;
 __device__ __forceinline__ void list_cut(int first, int last, int code, uint32_t* __restrict__ cut_a, uint32_t* __restrict__ cut_m,
                                          uint32_t* ncut) {
@@ -406,27 +410,26 @@ __global__ void refit_kernel(int n, const uint32_t* __restrict__ prim, const flo
 // confocal scan 18 against 11.5; box 13.6 against 7.2).  So the Morton order is cut into ranges of at most
 // 512 leaves, each is built anew top-down by one block -- every split of the sorted orders tried, all nodes
 // of a level at once, the triangles' boxes in shared memory -- and one block builds the levels above over
-// the ranges' boxes in the same way, beside them (up to 1024 of them; more keep the Morton hierarchy there).  Bound by
-// the issue of the running-box shuffles over about 14 levels; ranges of 256 and 128 leaves: 121 and 205 us
-// for both kernels one after the other instead of 126.  Frames with the build: 512 x 512 2.73 -> 2.63 ms, 1024 x 1024 11.1 ->
-// 10.4; static scenes: path tracing 608 -> 446 us, 128 x 128 allocation-free 428 -> 361 us.
+// the ranges' boxes in the same way, beside them (up to 1024 of them; more keep the Morton hierarchy there).
+// Frames with the build: 512 x 512 2.73 -> 2.63 ms, 1024 x 1024 11.1 -> 10.4; static scenes: path tracing 608 ->
+// 446 us, 128 x 128 allocation-free 428 -> 361 us.  A build alone, us, bottom-up boxes of the Morton hierarchy / first
+// form of this / now: 312 triangles 87 / 130 / 63, 968 101 / 116 / 80, 5000 130 / 119 / 104, 66k 163 / 169 / 150, 198k 214 /
+// 304 / 205, 270k 266 / 392 / 271, 646k 819 / 807 / 499, 4M 2629 / 4850 / 2090.
 // It writes boxes, children and leaf order itself, so a full build needs no bottom-up pass over all levels.
 // Node numbers: a range [a, a + m) owns the m - 1 numbers of its Karras nodes; its root keeps the Karras
 // root's, so that a Karras parent's link to it stays right.
 template <int N>
 struct Sweep {
-    float box[6][N];             // lo, hi of item i
-    float suf[6][N];             // box of positions p .. end of segment
-    unsigned long long best[N];  // per segment start: (cost, distance from the middle, position)
-    unsigned long long keys[N];
-    uint16_t ord[3][N];          // items sorted along each axis within their segment
-    uint16_t seg0[N], seg1[N];   // segment [seg0, seg1) of a position
-    uint16_t pre[3][N];          // items of the left side before a position of each order
-    uint8_t side[N], axis[N];    // of an item; of a segment's split, by its start
-    int link[N];                 // per segment start: 2 * parent + side of the node to come, or -1
+    float box[6][N];                  // lo, hi of item i
+    uint32_t keys[3][N];              // the sort's exchange
+    unsigned long long best[N];       // per segment start: (cost and distance from the middle, axis, position)
+    uint16_t ord[3][N];               // items sorted along each axis within their segment
+    uint16_t seg0[N], seg1[N];        // segment [seg0, seg1) of a position
+    uint8_t side[N];                  // of an item: right of its segment's split
+    int link[N];                      // per segment start: 2 * parent + side of the node to come, or -1
     float wup[3][N / 32][6], wdown[3][N / 32][6];
-    int wcnt[3][N / 32];
-    int root_split, open;        // open: leaves of the longest segment not yet split up
+    uint32_t bal[3][N / 32];          // per warp and axis: the positions whose item goes left
+    int root_split, open[2];          // open: leaves of the longest segment to split, by the level's parity
 };
 __device__ __forceinline__ float half_area(const float b[6]) {
     const float x = b[3] - b[0], y = b[4] - b[1], z = b[5] - b[2];
@@ -439,129 +442,172 @@ __device__ __forceinline__ void grow(float b[6], const float o[6]) {
 // barrier of the block's first nt threads (a multiple of 32): a range shorter than the block's threads
 // leaves the other warps out
 __device__ __forceinline__ void group_sync(int nt) { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); }
-// within its warp, the running box of a position's segment [s, e): from its start up to the position (kUp) or
-// from the position to its end
+// the running box of a lane's segment within its warp, over the `before` lanes below it that are in the segment
+// (kUp) or the `before` lanes above it
 template <bool kUp>
-__device__ __forceinline__ void run_boxes(int longest, int p, int s, int e, bool in, float b[6]) {
-    const int lane = p & 31;
+__device__ __forceinline__ void run_boxes(int reach, int before, float b[6]) {
 #pragma unroll 1
-    for (int o = 1; o < 32 && o < longest; o <<= 1) {
+    for (int o = 1; o < 32 && o < reach; o <<= 1) {
         float n[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) n[k] = kUp ? __shfl_up_sync(0xFFFFFFFFu, b[k], o) : __shfl_down_sync(0xFFFFFFFFu, b[k], o);
-        if (in && (kUp ? lane >= o && p - o >= s : lane + o < 32 && p + o < e)) grow(b, n);
+        if (before >= o) grow(b, n);
     }
 }
 
 // Builds the hierarchy of items 0 .. m - 1 (m >= 2, boxes in S.box) with N threads.  number(split,
 // root_split) is the node that splits after position `split`; leaf(position, item) the child code of one item;
 // up(code, node) records a child's parent.  Levels from `sweeps` on split in the middle, which bounds the
-// depth (coincident items): 16 and 9 levels in a range of 512, 16 and 10 above 1024 ranges, 51 of the 64 that a
+// depth (coincident items): 16 and 10 levels in a range of 512, 16 and 11 above 1024 ranges, 53 of the 64 that a
 // traversal's stack holds.  Below the Morton hierarchy's own top, which can be 30 levels and the logarithm of its
-// ranges deep, 8 and 9 levels.  all_axes: every split of the three orders is tried, else those of the order along
-// the segment's longest axis (a third of the work: 145 -> 77 us for 66k triangles, visits per ray up 2 %; a
-// scene of one range tries all, 12 % fewer visits in the 332-triangle box).
+// ranges deep, 8 and 10 levels.  kAll: every split of the three orders is tried, else those of the order along
+// the segment's longest axis (a third of the work, visits per ray up 2 %; a scene of at most 512 triangles
+// tries all, 12 % fewer visits in the 332-triangle box).
+// Bound by issue (62 % active with three blocks an SM; some 10k instructions a warp over about 14 levels, a third of
+// them the running boxes) and its chain of barriers, so: the three orders are sorted together, keys in
+// registers, barriers only for exchanges between warps; a level has five barriers (eleven at first); the best
+// split of a segment is found by shuffles with one shared atomic for each warp and segment; 40 registers.
+// treelet_kernel 66k triangles 71 -> 57 us, 198k 130 -> 93, 4M 2.08 -> 1.7 ms.
 constexpr int kMaxSweep = 16, kMortonSweep = 8;
-template <int N, class Number, class Leaf, class Up>
-__device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, bool all_axes, int sweeps, float4* __restrict__ nodes, int* __restrict__ child, Number number, Leaf leaf,
+template <int N, bool kAll, class Number, class Leaf, class Up>
+__device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, int sweeps, float4* __restrict__ nodes, int* __restrict__ child, Number number, Leaf leaf,
                                             Up up) {
-    const int p = threadIdx.x;
+    const int p = threadIdx.x, lane = p & 31, warp = p >> 5;
+    int pow2 = 32;
+    while (pow2 < m) pow2 <<= 1;
+    if (p >= pow2) return;
+    {   // centre (in 2^22 steps of the items' extent), then item: an order of all items along each axis (bitonic
+        // sort; padding sorts last)
+        uint32_t key[3];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            const float c = p < m ? S.box[ax][p] + S.box[3 + ax][p] : 0.f;
+            const uint32_t lo = __reduce_min_sync(0xFFFFFFFFu, p < m ? fenc(c) : 0xFFFFFFFFu);
+            const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, p < m ? fenc(c) : 0u);
+            if (lane == 0) { S.keys[ax][warp] = lo; S.keys[ax][N / 2 + warp] = hi; }
+        }
+        group_sync(pow2);
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            const uint32_t lo = __reduce_min_sync(0xFFFFFFFFu, lane < pow2 / 32 ? S.keys[ax][lane] : 0xFFFFFFFFu);
+            const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, lane < pow2 / 32 ? S.keys[ax][N / 2 + lane] : 0u);
+            const float c = p < m ? S.box[ax][p] + S.box[3 + ax][p] : 0.f, l = fdec(lo), w = fdec(hi) - l;
+            const uint32_t q = (uint32_t)fminf(fmaxf((c - l) / fmaxf(w, 1e-30f) * 4194304.f, 0.f), 4194302.f);
+            key[ax] = p < m ? (q << 10) | (uint32_t)p : 0xFFFFFFFFu;
+        }
+        group_sync(pow2);
+#pragma unroll 1
+        for (int k = 2; k <= pow2; k <<= 1)
+#pragma unroll 1
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                const bool low = ((p & k) == 0) == ((p & j) == 0);   // this place keeps the lower key
+                uint32_t o[3];
+                if (j >= 32) {
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) S.keys[ax][p] = key[ax];
+                    group_sync(pow2);
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) o[ax] = S.keys[ax][p ^ j];
+                    group_sync(pow2);
+                } else {
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) o[ax] = __shfl_xor_sync(0xFFFFFFFFu, key[ax], j);
+                }
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) key[ax] = low ? min(key[ax], o[ax]) : max(key[ax], o[ax]);
+            }
+        if (p < m)
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) S.ord[ax][p] = (uint16_t)(key[ax] & 1023u);
+    }
     const int nt = (m + 31) & ~31;
     if (p >= nt) return;
-    int pow2 = 2;
-    while (pow2 < m) pow2 <<= 1;
-    for (int ax = 0; ax < 3; ++ax) {
-        // centre, then item: an order of all items (bitonic sort; padding sorts last)
-        for (int i = p; i < pow2; i += nt) {
-            uint32_t c = 0xFFFFFFFFu;
-            if (i < m) c = fenc(S.box[ax][i] + S.box[3 + ax][i]);
-            S.keys[i] = ((unsigned long long)c << 16) | (uint32_t)(i < m ? i : 0xFFFF);
-        }
-        group_sync(nt);
-        for (int k = 2; k <= pow2; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = p; i < pow2 / 2; i += nt) {
-                    const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1)), hi = lo | j;
-                    const unsigned long long a = S.keys[lo], b = S.keys[hi];
-                    if ((a > b) == ((lo & k) == 0)) { S.keys[lo] = b; S.keys[hi] = a; }
-                }
-                group_sync(nt);
-            }
-        if (p < m) S.ord[ax][p] = (uint16_t)(S.keys[p] & 0xFFFFu);
-        group_sync(nt);
-    }
     if (p < m) { S.seg0[p] = 0; S.seg1[p] = (uint16_t)m; }
-    if (p == 0) { S.link[0] = -1; S.root_split = -1; S.open = m; }
+    if (p == 0) { S.link[0] = -1; S.root_split = -1; S.open[0] = m; S.best[0] = ~0ull; }
     group_sync(nt);
+#pragma unroll 1
     for (int level = 0;; ++level) {
-        const bool have = p < m;
-        const int s = have ? S.seg0[p] : 0, e = have ? S.seg1[p] : 0;
-        const bool in = have && e - s > 1;   // an open segment
-        if (in && p == s) S.best[s] = ~0ull;
-        const int longest = S.open;   // leaves of the longest open segment
-        group_sync(nt);
-        if (p == 0) S.open = 0;
-        float L[6], R[6], bestc = 3.4e38f;
-        int bax = -1, longaxis = 0;
-        if (!all_axes && in) {
+        if (S.open[level & 1] <= 1) break;   // leaves of the longest segment
+        if (p == 0) S.open[(level + 1) & 1] = 0;
+        const int s = p < m ? S.seg0[p] : 0, e = p < m ? S.seg1[p] : 0;
+        const bool in = e - s > 1;   // a segment to split
+        // lanes of the segment below and above this one in the warp
+        const int below = in ? min(lane, p - s) : 0, above = in ? min(31 - lane, e - 1 - p) : 0;
+        const int reach = __reduce_max_sync(0xFFFFFFFFu, in ? e - s : 0);   // the warp's longest segment
+        if (reach == 0) {   // none in this warp: it only keeps the barriers' count
+#pragma unroll 1
+            for (int t = 0; t < (kAll ? 7 : 5); ++t) group_sync(nt);
+            continue;
+        }
+        float L[6], R[6], cost = 3.4e38f;
+        int axis = 0, item = 0;
+        bool any = false;
+        if (!kAll && e - s > 2) {   // (of two items every order gives the same split)
+            // by the centres: by the sides of the segment's box the build is 8 us shorter (198k triangles), but a
+            // 301 x 203 frame 20 us longer
             float ext = -1.0f;
 #pragma unroll
             for (int ax = 0; ax < 3; ++ax) {
                 const int i0 = S.ord[ax][s], i1 = S.ord[ax][e - 1];
                 const float x = (S.box[ax][i1] + S.box[3 + ax][i1]) - (S.box[ax][i0] + S.box[3 + ax][i0]);
-                if (x > ext) { ext = x; longaxis = ax; }
+                if (x > ext) { ext = x; axis = ax; }
             }
         }
-        const bool any = __any_sync(0xFFFFFFFFu, in);
 #pragma unroll 1
-        for (int t = 0; t < (all_axes ? 3 : 1); ++t) {
-            const int ax = all_axes ? t : longaxis;
-            if (!any) {   // no open segment in this warp
-                group_sync(nt);
-                group_sync(nt);
-                continue;
-            }
-            const int item = in ? S.ord[ax][p] : 0;
-            float b[6], f[6];
+        for (int t = 0; t < (kAll ? 3 : 1); ++t) {
+            const int ax = kAll ? t : axis;
+            float f[6], b[6];
+            item = in ? S.ord[ax][p] : 0;
 #pragma unroll
             for (int k = 0; k < 6; ++k) b[k] = f[k] = S.box[k][item];
-            run_boxes<true>(longest, p, s, e, in, f);
-            run_boxes<false>(longest, p, s, e, in, b);
+            run_boxes<true>(reach, below, f);
+            run_boxes<false>(reach, above, b);
             // across warps: a segment's part in each warp it reaches over
-            if ((p & 31) == 31)
+            if (lane == 31)
 #pragma unroll
-                for (int k = 0; k < 6; ++k) S.wup[t][p >> 5][k] = f[k];
-            if ((p & 31) == 0)
+                for (int k = 0; k < 6; ++k) S.wup[t][warp][k] = f[k];
+            if (lane == 0)
 #pragma unroll
-                for (int k = 0; k < 6; ++k) S.wdown[t][p >> 5][k] = b[k];
+                for (int k = 0; k < 6; ++k) S.wdown[t][warp][k] = b[k];
             group_sync(nt);
-            if (in) {
-                for (int v = (p >> 5) - 1; v >= 0 && 32 * v + 31 >= s; --v) grow(f, S.wup[t][v]);
-                for (int v = (p >> 5) + 1; 32 * v < e; ++v) grow(b, S.wdown[t][v]);
+            // b becomes the box of the positions behind p
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                b[k] = __shfl_down_sync(0xFFFFFFFFu, b[k], 1);
+                if (lane == 31) b[k] = k < 3 ? 3.4e38f : -3.4e38f;
             }
-            if (have)
+            if (in) {
+                for (int v = warp - 1; v >= 0 && 32 * v + 31 >= s; --v) grow(f, S.wup[t][v]);
+                for (int v = warp + 1; 32 * v < e; ++v) grow(b, S.wdown[t][v]);
+                if (p + 1 < e) {
+                    const float c = level >= sweeps ? 0.f : half_area(f) * (float)(p + 1 - s) + half_area(b) * (float)(e - 1 - p);
+                    if (!any || c < cost) {
+                        any = true;
+                        cost = c; axis = ax;
 #pragma unroll
-                for (int k = 0; k < 6; ++k) S.suf[k][p] = b[k];
-            group_sync(nt);
-            if (in && p + 1 < e) {
-                float r[6];
-#pragma unroll
-                for (int k = 0; k < 6; ++k) r[k] = S.suf[k][p + 1];
-                const float c = level >= sweeps ? 0.f : half_area(f) * (float)(p + 1 - s) + half_area(r) * (float)(e - 1 - p);
-                if (bax < 0 || c < bestc) {
-                    bestc = c; bax = ax;
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) { L[k] = f[k]; R[k] = r[k]; }
+                        for (int k = 0; k < 6; ++k) { L[k] = f[k]; R[k] = b[k]; }
+                    }
                 }
             }
         }
-        const uint32_t mid = (uint32_t)abs(2 * (p + 1 - s) - (e - s));
-        const unsigned long long key = ((unsigned long long)__float_as_uint(bestc) << 32) | (mid << 16) | (uint32_t)p;
-        if (in && bax >= 0) atomicMin(&S.best[s], key);
+        // the split's cost to 18 bits, of equals the one nearest to the middle
+        uint32_t key = 0xFFFFFFFFu;
+        if (any) key = (__float_as_uint(cost) & ~63u) | (uint32_t)min(63, abs(2 * (p + 1 - s) - (e - s)) >> (31 - __clz(e - s) > 6 ? 25 - __clz(e - s) : 0));
+        uint32_t low = key;
+#pragma unroll 1
+        for (int o = 1; o < 32 && o < reach; o <<= 1) {
+            const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, low, o);
+            if (below >= o) low = min(low, n);
+        }
+        low = __shfl_sync(0xFFFFFFFFu, low, lane + above);   // of the segment's part in this warp
+        const uint32_t same = __ballot_sync(0xFFFFFFFFu, any && key == low) & (0xFFFFFFFFu >> (31 - below - above) << (lane - below));
+        if (any && same && __ffs(same) - 1 == lane)
+            atomicMin(&S.best[s], ((unsigned long long)key << 32) | (uint32_t)(axis << 10) | (uint32_t)p);
         group_sync(nt);
-        const int cut = in ? (int)(S.best[s] & 0xFFFFu) : 0;   // the segment splits after this position
-        const bool winner = in && p == cut;
-        if (winner) {
+        const unsigned long long best = in ? S.best[s] : 0ull;
+        const int cut = (int)(best & 1023u);   // the segment splits after this position of its axis' order
+        if (in) S.side[kAll ? S.ord[(best >> 10) & 3u][p] : item] = p > cut;
+        if (in && p == cut) {
             if (level == 0) S.root_split = p;
             const int id = number(p, level == 0 ? p : S.root_split);
             nodes[4 * (size_t)id] = make_float4(L[0], L[3], L[1], L[4]);
@@ -575,53 +621,49 @@ __device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, bool all_axes, i
             }
             S.link[s] = 2 * id;        // an open left part keeps the start
             S.link[p + 1] = 2 * id + 1;
-            S.axis[s] = (uint8_t)bax;
-            const int longer = max(p + 1 - s, e - 1 - p);
-            if (longer > 1) atomicMax(&S.open, longer);
         }
-        group_sync(nt);
-        if (in) S.side[S.ord[S.axis[s]][p]] = p > cut;   // items up to the cut in the winning order go left
         group_sync(nt);
         // stable partition of the three orders
-        int item[3], before[3];
-        unsigned left = 0u;
+        int part[3];
+        uint32_t bal[3];
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
-            item[ax] = in ? S.ord[ax][p] : 0;
-            const bool l = in && S.side[item[ax]] == 0;
-            const unsigned bal = __ballot_sync(0xFFFFFFFFu, l);
-            if (l) left |= 1u << ax;
-            if ((p & 31) == 0) S.wcnt[ax][p >> 5] = __popc(bal);
-            before[ax] = __popc(bal & ((1u << (p & 31)) - 1u));
+            part[ax] = in ? S.ord[ax][p] : 0;
+            const bool l = in && S.side[part[ax]] == 0;
+            bal[ax] = __ballot_sync(0xFFFFFFFFu, l);
+            if (lane == 0) S.bal[ax][warp] = bal[ax];
         }
         group_sync(nt);
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            for (int v = 0; v < (p >> 5); ++v) before[ax] += S.wcnt[ax][v];
-            S.pre[ax][p] = (uint16_t)before[ax];
-        }
-        group_sync(nt);
-        if (in)
+        int ns = s, ne = e;
+        if (in) {
 #pragma unroll
             for (int ax = 0; ax < 3; ++ax) {
-                const int l = before[ax] - S.pre[ax][s];   // of the left side before this position
-                S.ord[ax][(left >> ax) & 1u ? s + l : cut + 1 + (p - s) - l] = (uint16_t)item[ax];
+                int l = __popc(bal[ax] & ((1u << lane) - (1u << (lane - below))));   // of the left side before this position
+                if (s < 32 * warp) {
+                    l += __popc(S.bal[ax][s >> 5] >> (s & 31));
+                    for (int v = (s >> 5) + 1; v < warp; ++v) l += __popc(S.bal[ax][v]);
+                }
+                const int dst = (bal[ax] >> lane) & 1u ? s + l : cut + 1 + (p - s) - l;
+                S.ord[ax][dst] = (uint16_t)part[ax];
+                if (ax == 0) {
+                    const int ds = dst <= cut ? s : cut + 1, de = dst <= cut ? cut + 1 : e;
+                    if (de - ds == 1) {   // one item left: a child of the node just written
+                        const int link = S.link[dst];
+                        const int code = leaf(dst, part[0]);
+                        child[link] = code;
+                        reinterpret_cast<int*>(nodes + 4 * (size_t)(link >> 1) + 3)[link & 1] = code;
+                        up(code, link >> 1);
+                    }
+                }
             }
-        group_sync(nt);
-        if (in) {
-            const int ns = p <= cut ? s : cut + 1, ne = p <= cut ? cut + 1 : e;
+            ns = p <= cut ? s : cut + 1;
+            ne = p <= cut ? cut + 1 : e;
             S.seg0[p] = (uint16_t)ns;
             S.seg1[p] = (uint16_t)ne;
-            if (ne - ns == 1) {   // one item left: a child of the node just written
-                const int link = S.link[p];
-                const int code = leaf(p, (int)S.ord[0][p]);
-                child[link] = code;
-                reinterpret_cast<int*>(nodes + 4 * (size_t)(link >> 1) + 3)[link & 1] = code;
-                up(code, link >> 1);
-            }
+            if (p == ns) S.best[p] = ~0ull;
         }
-        group_sync(nt);
-        if (!S.open) break;
+        const int most = __reduce_max_sync(0xFFFFFFFFu, in ? ne - ns : 0);
+        if (lane == 0 && most > 1) atomicMax(&S.open[(level + 1) & 1], most);
         group_sync(nt);
     }
 }
@@ -666,59 +708,81 @@ __global__ void __launch_bounds__(128) range_box_kernel(int n, const uint32_t* _
     }
 }
 
-__global__ void __launch_bounds__(kTreelet) treelet_kernel(int n, uint32_t* __restrict__ prim, const float4* __restrict__ tri,
+// one range: items p = 0 .. m - 1 are the triangles t, leaves a .. a + m - 1
+template <int N, bool kAll>
+__device__ __forceinline__ void build_range(Sweep<N>& S, int a, int m, bool last, int t, int sweeps, uint32_t* __restrict__ prim,
+                                            const float4* __restrict__ tri, float4* __restrict__ leaves, float4* __restrict__ nodes,
+                                            int* __restrict__ child, int* __restrict__ parent_int, int* __restrict__ parent_leaf) {
+    const int p = threadIdx.x;
+    if (p < m) {
+        const Box b = tri_box(tri, t);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { S.box[k][p] = b.lo[k]; S.box[3 + k][p] = b.hi[k]; }
+    }
+    __syncthreads();
+    int pos = p;   // item p's leaf within the range
+    if (m > 1) {
+        // numbers a .. a + m - 1 without the end that is not the root's
+        const int base = last ? a + 1 : a, root = last ? a + m - 1 : a, at_root = root - base;
+        sweep_build<N, kAll>(
+            S, m, sweeps, nodes, child,
+            [=](int split, int rs) { return split == rs ? root : split == at_root ? base + rs : base + split; },
+            [=](int q, int) { return ~(a + q); },
+            [=](int code, int node) {
+                if (code < 0) parent_leaf[~code] = node;
+                else parent_int[code] = node;
+            });
+        if (p < m) S.seg0[S.ord[0][p]] = (uint16_t)p;
+        __syncthreads();
+        if (p < m) pos = S.seg0[p];
+    }
+    if (p < m) {
+        const size_t l = (size_t)(a + pos);
+        prim[l] = (uint32_t)t;
+        const float4 v = tri[3 * (size_t)t];
+        leaves[3 * l] = make_float4(v.x, v.y, v.z, __int_as_float(t));
+        leaves[3 * l + 1] = tri[3 * (size_t)t + 1];
+        leaves[3 * l + 2] = tri[3 * (size_t)t + 2];
+    }
+}
+
+constexpr int kTreeletBlocks = 3;   // resident on an SM
+__global__ void __launch_bounds__(kTreelet, kTreeletBlocks) treelet_kernel(int n, uint32_t* __restrict__ prim, const float4* __restrict__ tri,
                                                            float4* __restrict__ leaves, float4* __restrict__ nodes, int* __restrict__ child,
                                                            int* __restrict__ parent_int, int* __restrict__ parent_leaf,
                                                            const uint32_t* __restrict__ cut_a, const uint32_t* __restrict__ cut_m,
                                                            const uint32_t* __restrict__ ncut) {
     extern __shared__ __align__(16) unsigned char sm[];
     Sweep<kTreelet>& S = *reinterpret_cast<Sweep<kTreelet>*>(sm);
-    const int p = threadIdx.x;
     const uint32_t R = *ncut;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // treelet_top_kernel may start beside this one
+    const int sweeps = top_by_area((int)R, n) ? kMaxSweep : kMortonSweep;
     for (uint32_t r = blockIdx.x; r < R; r += gridDim.x) {
         const int a = (int)cut_a[r], m = (int)(cut_m[r] & ~kRootLast);
-        const bool last = (cut_m[r] & kRootLast) != 0u;
-        const int t = p < m ? (int)prim[a + p] : 0;   // item p's triangle
-        if (p < m) {
-            const Box b = tri_box(tri, t);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) { S.box[k][p] = b.lo[k]; S.box[3 + k][p] = b.hi[k]; }
-        }
-        __syncthreads();
-        int pos = p;   // item p's leaf within the range
-        if (m > 1) {
-            // numbers a .. a + m - 1 without the end that is not the root's
-            const int base = last ? a + 1 : a, root = last ? a + m - 1 : a, at_root = root - base;
-            sweep_build<kTreelet>(
-                S, m, R == 1u, R == 1u || top_by_area((int)R, n) ? kMaxSweep : kMortonSweep, nodes, child,
-                [=](int split, int rs) { return split == rs ? root : split == at_root ? base + rs : base + split; },
-                [=](int q, int) { return ~(a + q); },
-                [=](int code, int node) {
-                    if (code < 0) parent_leaf[~code] = node;
-                    else parent_int[code] = node;
-                });
-            if (p < m) S.pre[0][S.ord[0][p]] = (uint16_t)p;
-            __syncthreads();
-            if (p < m) pos = S.pre[0][p];
-        }
-        if (p < m) {
-            const size_t l = (size_t)(a + pos);
-            prim[l] = (uint32_t)t;
-            const float4 v = tri[3 * (size_t)t];
-            leaves[3 * l] = make_float4(v.x, v.y, v.z, __int_as_float(t));
-            leaves[3 * l + 1] = tri[3 * (size_t)t + 1];
-            leaves[3 * l + 2] = tri[3 * (size_t)t + 2];
-        }
+        const int t = (int)threadIdx.x < m ? (int)prim[a + threadIdx.x] : 0;
+        build_range<kTreelet, false>(S, a, m, (cut_m[r] & kRootLast) != 0u, t, sweeps, prim, tri, leaves, nodes, child, parent_int, parent_leaf);
         __syncthreads();
     }
+}
+
+// A scene of at most N triangles is one range, built from the triangles as they are: no Morton codes, sort or
+// Karras pass (684 triangles: 58 us of kernels against 140 with them, 82 with the bottom-up pass).
+template <int N, bool kAll>
+__global__ void __launch_bounds__(N) whole_kernel(int n, uint32_t* __restrict__ prim, const float4* __restrict__ tri, float4* __restrict__ leaves,
+                                                  float4* __restrict__ nodes, int* __restrict__ child, int* __restrict__ parent_int,
+                                                  int* __restrict__ parent_leaf) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    Sweep<N>& S = *reinterpret_cast<Sweep<N>*>(sm);
+    const int p = threadIdx.x;
+    if (p == 0) parent_int[0] = -1;
+    build_range<N, kAll>(S, 0, n, false, p < n ? p : 0, kMaxSweep, prim, tri, leaves, nodes, child, parent_int, parent_leaf);
 }
 
 // The levels above the treelets, one block.  It starts beside treelet_kernel (programmatic launch): the ranges'
 // boxes come from range_box_kernel, which is complete when treelet_kernel starts, and the nodes, children and
 // parents that the two write are not the same ones.  It ends after treelet_kernel has (every path waits), so
-// what follows it in the stream finds both.  Both are chains of short barriers on few SMs (66k triangles: 75 and
-// 49 us), so side by side they take little more than the longer: 301 x 203 frame 1.311 -> 1.284 ms, four served
+// what follows it in the stream finds both.  Both are chains of short barriers on few SMs (66k triangles: 57 and
+// 29 us), so side by side they take little more than the longer: 301 x 203 frame 1.311 -> 1.284 ms, four served
 // streams 6.39 -> 6.28, the boxes' own launch included.
 // Of more than kTopItems ranges the Morton hierarchy's own nodes above stay, their boxes found bottom-up as in
 // refit_kernel: by treelet_top_kernel's block in a scene of up to kClimbBlock triangles, by morton_top_kernel
@@ -772,8 +836,8 @@ __global__ void __launch_bounds__(kTopItems) treelet_top_kernel(int n, const uin
         auto slot_item = [=](int split) { return split == none ? R - 1 : split; };
         auto slot_of = [=](int item) { return (cut_m[item] & kRootLast) ? (int)cut_a[item] : (int)(cut_a[item] + (cut_m[item] & ~kRootLast)) - 1; };
         const int zero_split = zero == R - 1 ? none : zero;
-        sweep_build<kTopItems>(
-            S, R, false, kMaxSweep, nodes, child,
+        sweep_build<kTopItems, false>(
+            S, R, kMaxSweep, nodes, child,
             [=](int split, int rs) { return split == rs ? 0 : slot_of(slot_item(split == zero_split ? rs : split)); },
             [=](int, int item) {
                 const int a = (int)cut_a[item], m = (int)(cut_m[item] & ~kRootLast);
@@ -867,9 +931,9 @@ __global__ void __launch_bounds__(1024) etree_top_kernel(int lowest, float4* nod
 static inline unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const uint32_t* triobj, const uint32_t* objmat,
-                         const float* xf, float4* tri_out, float4* cent, cudaStream_t s) {
+                         const float* xf, float4* tri_out, float4* cent, uint32_t* bb, cudaStream_t s) {
     note_launch();
-    xform_kernel<<<blocks(nt, 256), 256, 0, s>>>(nt, vloc, tris, triobj, objmat, xf, tri_out, cent);
+    xform_kernel<<<blocks(nt, 256), 256, 0, s>>>(nt, vloc, tris, triobj, objmat, xf, tri_out, cent, bb);
     return cudaGetLastError();
 }
 
@@ -901,10 +965,6 @@ constexpr int kAddTiles = 110, kScanTiles = 600;
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
                                   uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
                                   uint32_t* counter, uint32_t** prim_out, float4* scratch, cudaStream_t s) {
-    // centroid bounds start empty: encoded minima at 0xFFFFFFFF, maxima at 0
-    cudaError_t e = cudaMemsetAsync(bb, 0xFF, 3 * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(bb + 3, 0, 4 * sizeof(uint32_t), s);   // and the number of treelets
-    if (e != cudaSuccess) return e;
     note_launch();
     bounds_kernel<<<min(1024u, blocks(n, 256)), 256, 0, s>>>(n, cent, bb);
     note_launch();
@@ -912,14 +972,14 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
     uint32_t *ki = keys, *vi = vals, *ko = keys2, *vo = vals2;
     // the histograms (and the scans' totals) lie in the centroids' memory, which the Morton codes were the last to
     // read: at most 2 B a key and 1 KB of its 16 B a key
-    uint32_t* counts = n >= 512 ? reinterpret_cast<uint32_t*>(scratch) : hist;
+    uint32_t* counts = n > kWhole ? reinterpret_cast<uint32_t*>(scratch) : hist;
     int nt = (n + kCoopTile - 1) / kCoopTile;
     const void* sort = nt <= kAddTiles ? (const void*)radix_sort_coop_kernel<false> : (const void*)radix_sort_coop_kernel<true>;
     if (nt <= kScanTiles && nt <= sort_blocks(sort, nt <= kAddTiles ? 0 : 1)) {
         int nn = n;
         void* args[] = {&ki, &vi, &ko, &vo, &nn, &counts, &nt};
         note_launch();
-        e = cudaLaunchCooperativeKernel(sort, dim3(nt), dim3(256), args, 0, s);
+        const cudaError_t e = cudaLaunchCooperativeKernel(sort, dim3(nt), dim3(256), args, 0, s);
         if (e != cudaSuccess) return e;
     } else {
         const int ntiles = (n + kTile - 1) / kTile;
@@ -939,23 +999,45 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
     return cudaGetLastError();
 }
 
+static cudaError_t size_treelets() {
+    static std::atomic<bool> sized[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && sized[dev].load()) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(treelet_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTreelet>));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(treelet_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTopItems>));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(whole_kernel<kTreelet, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTreelet>));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(whole_kernel<kWhole, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kWhole>));
+    if (e == cudaSuccess && dev >= 0 && dev < 64) sized[dev].store(true);
+    return e;
+}
+
+// whether a full build of n triangles is launch_whole's; else launch_build_topology and launch_treelets
+bool whole_build(int n) { return n > 1 && n <= kWhole; }
+cudaError_t launch_whole(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int, int* parent_leaf,
+                         cudaStream_t s) {
+    const cudaError_t e = size_treelets();
+    if (e != cudaSuccess) return e;
+    note_launch();
+    if (n <= kTreelet)
+        whole_kernel<kTreelet, true><<<1, kTreelet, sizeof(Sweep<kTreelet>), s>>>(n, prim, tri, leaf, nodes, child, parent_int, parent_leaf);
+    else
+        whole_kernel<kWhole, false><<<1, kWhole, sizeof(Sweep<kWhole>), s>>>(n, prim, tri, leaf, nodes, child, parent_int, parent_leaf);
+    return cudaGetLastError();
+}
+
 // boxes, leaf records and the treelets' topology of a full build (n > 1), after launch_build_topology
 cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
                             int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut,
                             float4* boxes, int sms, cudaStream_t s) {
-    static std::atomic<bool> sized[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !sized[dev].load()) {
-        cudaError_t e = cudaFuncSetAttribute(treelet_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTreelet>));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(treelet_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sweep<kTopItems>));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) sized[dev].store(true);
-    }
+    cudaError_t e = size_treelets();
+    if (e != cudaSuccess) return e;
     const bool climb = n > kClimbBlock;   // by a kernel of its own
     // ranges hold at least a few leaves each, mostly hundreds: a block takes several where there are many
-    const int grid = min((int)blocks(n, 64), 4 * sms);
+    const int grid = min((int)blocks(n, 64), kTreeletBlocks * sms);
     note_launch(3);
     range_box_kernel<<<min((int)blocks(n, 64), 4 * sms), 128, 0, s>>>(n, prim, tri, boxes, cut_a, cut_m, ncut);
     treelet_kernel<<<grid, kTreelet, sizeof(Sweep<kTreelet>), s>>>(n, prim, tri, leaf, nodes, child, parent_int, parent_leaf, cut_a, cut_m, ncut);
@@ -965,8 +1047,8 @@ cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* le
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1); cfg.blockDim = dim3(kTopItems); cfg.dynamicSmemBytes = sizeof(Sweep<kTopItems>); cfg.stream = s;
     cfg.attrs = beside; cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, treelet_top_kernel, n, (const uint32_t*)prim, tri, (const float4*)boxes, nodes, child, parent_int,
-                                             parent_leaf, counter, cut_a, cut_m, ncut, !climb);
+    e = cudaLaunchKernelEx(&cfg, treelet_top_kernel, n, (const uint32_t*)prim, tri, (const float4*)boxes, nodes, child, parent_int,
+                           parent_leaf, counter, cut_a, cut_m, ncut, !climb);
     if (e != cudaSuccess) return e;
     if (climb) {
         note_launch();
