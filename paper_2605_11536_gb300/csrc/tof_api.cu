@@ -724,6 +724,7 @@ struct BatchRec {
     std::vector<GbufArgs> gbuf;
     std::vector<InitArgs> init;
     std::vector<WaveRec> wave;
+    std::vector<WaveRec> large;                // initial stages with a thread per pixel (w unused)
     std::vector<std::vector<ReuseJob>> pass;   // pass[q]: every instance's q-th reuse pass
     size_t q = 0;                              // the current instance's next pass
     long long npix = 0;                        // pixels of all instances
@@ -822,10 +823,15 @@ static tof_status ensure_tree_wave(tof_ctx* c, ViewH& V, int nc, int depth) {
 // of scratch); in a batch only views of kBatchWaveMinPix pixels and more do (small instances would
 // pay for its 2 * depth + 1 launches each).  The rest keep the single kernel, which needs no scratch.
 // Both give the same reservoirs.
+constexpr double kTreeWavePaths = 16.0 * 1024.0 * 1024.0;
 static bool use_tree_wave(const ViewH& V, int B, const tof_params* p, bool fixed) {
     if (fixed || (p->flags & TOF_FLAG_ELLIPSOID) || p->shrink_k > 1.f) return false;
-    return (double)V.W * V.H * p->n_cand <= 16.0 * 1024.0 * 1024.0;
+    return (double)V.W * V.H * p->n_cand <= kTreeWavePaths;
 }
+// the single gated kernel has a thread per path tree (initial_lanes_kernel) except in views beyond the wavefront's
+// limit, whose pixels are threads enough: 1100 x 1100 with 16 trees 6.71 (lanes) -> 6.00 ms in the box, 10.9 -> 9.7 over the
+// terrain; 2100 x 2100 with 5 trees of depth 2 over the terrain 7.79 -> 6.58 (7.47 before there was a lane form)
+static bool lanes_pay(const ViewH& V, const tof_params* p) { return (double)V.W * V.H * p->n_cand <= kTreeWavePaths; }
 
 // batches run a gated instance's initial stage as the bounce wavefront from this many pixels on:
 // smaller ones are cheaper as blocks of the batched single kernel than as 2 * depth + 1 launches
@@ -1059,7 +1065,8 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
     ia.out = (stage == stages - 1 && B == 0) ? out : nullptr;
     ia.tile_w = V.tune.tile_w;
     if (!c->sms) CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
-    initial_lanes_tile(g_rec ? g_rec->npix : (long long)V.W * V.H, params->n_cand, c->sms, &ia.lane_w, &ia.lane_h);
+    ia.lane_w = ia.lane_h = 0;
+    if (lanes_pay(V, params)) initial_lanes_tile(g_rec ? g_rec->npix : (long long)V.W * V.H, params->n_cand, c->sms, &ia.lane_w, &ia.lane_h);
     if (B == 0 && params->shrink_k > 1.f) {
         CK(launch_initial_shrink(ia, V.tune.tile_h, s));
     } else if (use_ell_wave(V, B, params, fixed_wave != nullptr)) {
@@ -1097,6 +1104,10 @@ static tof_status render(tof_ctx* c, tof_scene scene, tof_view vid, const tof_se
             CK(launch_initial_tree_wave(ia, V.tw, V.tune.tile_h, hb, vb, s));
         }
     } else if (g_rec) {
+        if (ia.lane_w == 0) {
+            ia.wave = 1;
+            g_rec->large.push_back(WaveRec{ia, TreeWaveDev(), V.tune.tile_h, 0, 0});
+        }
         g_rec->init.push_back(ia);   // staged batches hold gated views without those options only
     } else {
         CK(launch_initial(ia, V.tune.tile_h, c->d_err, s));
@@ -1346,7 +1357,7 @@ static size_t staged_layout(StagedGroup& G, size_t off) {
         const GbufArgs& g = G.rec.gbuf[j];
         const int tw = g.tile_w, th = 128 / tw;
         G.bpix[j + 1] = G.bpix[j] + ((g.F.W + tw - 1) / tw) * ((g.F.H + th - 1) / th);
-        // an instance that runs the bounce wavefront needs no blocks here
+        // an instance that runs the bounce wavefront or a thread per pixel needs no blocks here
         G.binit[j + 1] = G.binit[j] + (G.rec.init[j].wave ? 0 : initial_lanes_blocks(G.rec.init[j]));
     }
     G.o_g = off;
@@ -1399,6 +1410,7 @@ static cudaError_t staged_launch(tof_ctx* c, const StagedGroup& G, unsigned char
         const WaveRec& w = G.rec.wave[k];
         e = launch_initial_tree_wave(w.a, w.w, w.tile_h, w.hit_blocks, w.vis_blocks, q);
     }
+    for (size_t k = 0; k < G.rec.large.size() && e == cudaSuccess; ++k) e = launch_initial(G.rec.large[k].a, G.rec.large[k].tile_h, c->d_err, q);
     for (size_t k = 0; k < G.rec.pass.size() && e == cudaSuccess; ++k)
         e = launch_reuse_batch((const ReuseJob*)(d + G.o_p[k]), (int)G.rec.pass[k].size(), (const int*)(d + G.o_s[k]),
                                G.bs[k].back(), (const int*)(d + G.o_u[k]), G.bu[k].back(), c->persist_blocks, c->shift_blocks,

@@ -467,7 +467,7 @@ __device__ __forceinline__ void run_boxes(int reach, int before, float b[6]) {
 // them the running boxes) and its chain of barriers, so: the three orders are sorted together, keys in
 // registers, barriers only for exchanges between warps; a level has five barriers (eleven at first); the best
 // split of a segment is found by shuffles with one shared atomic for each warp and segment; 40 registers.
-// treelet_kernel 66k triangles 71 -> 57 us, 198k 130 -> 93, 4M 2.08 -> 1.7 ms.
+// treelet_kernel 66k triangles 71 -> 57 us, 198k 130 -> 93, 4M 2.08 -> 1.52 ms.
 constexpr int kMaxSweep = 16, kMortonSweep = 8;
 template <int N, bool kAll, class Number, class Leaf, class Up>
 __device__ __forceinline__ void sweep_build(Sweep<N>& S, int m, int sweeps, float4* __restrict__ nodes, int* __restrict__ child, Number number, Leaf leaf,

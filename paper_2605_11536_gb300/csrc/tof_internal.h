@@ -131,8 +131,8 @@ struct InitArgs {
     float* out;              // gated image if this is the last stage (else null)
     int tile_w;
     int wave;                // a staged batch runs this instance's initial stage as the bounce
-                             // wavefront: initial_lanes_batch_kernel skips it
-    int lane_w, lane_h;      // pixel tile of the lane form (initial_lanes_tile)
+                             // wavefront, or a thread per pixel: initial_lanes_batch_kernel skips it
+    int lane_w, lane_h;      // pixel tile of the lane form (initial_lanes_tile); 0: a thread per pixel
 };
 
 struct ReuseArgs {

@@ -261,9 +261,10 @@ struct GatedSink {
     }
 };
 
-// gated views with the ellipsoidal connection: the same trees, candidates, order and uniforms as
-// initial_kernel, into GatedSink
-__global__ void __launch_bounds__(128, 4) initial_gated_ell_kernel(const __grid_constant__ InitArgs a) {
+// gated views with the ellipsoidal connection, and those too large for the bounce wavefront's scratch
+// (kTreeWavePaths): the same trees, candidates, order and uniforms as initial_kernel, into GatedSink
+template <bool kEll>
+__global__ void __launch_bounds__(128, kEll ? 4 : 6) initial_gated_kernel(const __grid_constant__ InitArgs a) {
     const FrameDev& F = a.F;
     int ix, iy;
     tile_pixel(a.tile_w, ix, iy);
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(128, 4) initial_gated_ell_kernel(const __grid_
     TreeVerts T;
     for (int t = 0; t < P.n_cand; ++t) {
         sink.tree = t;
-        trace_tree<1>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
+        trace_tree<kEll ? 1 : 0>(D, P, (uint32_t)pix, F.frame, t, F.L0, F.L0 + F.dL, T, sink);
     }
     float outv = 0.f;
     uint32_t occ = 0u;
@@ -1153,7 +1154,8 @@ cudaError_t launch_initial(const InitArgs& a, int tile_h, unsigned* err, cudaStr
     const dim3 grid = tile_grid(a.F.W, a.F.H, a.tile_w, tile_h);
     const int threads = a.tile_w * tile_h;
     if (a.F.B == 0) {
-        if (a.P.flags & kFlagEllipsoid) initial_gated_ell_kernel<<<grid, threads, 0, s>>>(a);
+        if (a.P.flags & kFlagEllipsoid) initial_gated_kernel<true><<<grid, threads, 0, s>>>(a);
+        else if (a.lane_w == 0) initial_gated_kernel<false><<<grid, threads, 0, s>>>(a);
         else initial_lanes_kernel<<<tile_grid(a.F.W, a.F.H, a.lane_w, a.lane_h), kLaneThreads, 0, s>>>(a);
     } else {
         if (a.P.flags & kFlagEllipsoid) initial_kernel<true><<<grid, threads, 0, s>>>(a, err);
