@@ -183,9 +183,10 @@ tof_status tof_scene_destroy(tof_ctx* ctx, tof_scene scene);
  * LBVH (Morton codes, radix sort, hierarchy, bounds).  Not in the paper, which traces rays with
  * the GPU's ray-tracing hardware through DXR (Sec. 6); GB300 has no such units, so the library
  * builds its own hierarchy (Karras 2012 construction over 30-bit Morton codes, its ranges of up to
- * 512 leaves and the levels above them rebuilt by the surface area heuristic).  refit_only = 1 keeps the hierarchy and
+ * 512 leaves and the levels above them rebuilt by the surface area heuristic; scenes of up to 1024
+ * triangles in one range).  refit_only = 1 keeps the hierarchy and
  * refits bounds after rigid motion: cheaper to build, but the hierarchy's quality decays as objects
- * move away from where it was built (a full build of 66k triangles takes about 0.2 ms on GB300 and
+ * move away from where it was built (a full build of 66k triangles takes about 0.15 ms on GB300 and
  * pays for itself within a few frames of motion).  Call once per frame before rendering it: the library keeps
  * the geometry of the previous call resident for temporal reuse (an exact inverse shift into the
  * previous frame needs the previous scene).  Transforms identical to the current ones are a
@@ -283,16 +284,19 @@ tof_status tof_render_batch(tof_ctx* ctx, const tof_job* jobs, uint32_t n, void*
 /* Launch shapes and reservoir layout of a view (the batched form's per-instance-class tuning).
  * None of them changes a result: every pixel's random numbers are keyed by the pixel, and the
  * merges read their inputs by index, so a frame renders to the same bits under every tuning.
- *   tile_w x tile_h: pixel tile of the per-pixel kernels (G-buffer, initial candidates), one thread
- *     per pixel; tile_w a power of two in [4, 32], tile_w * tile_h = 64 or 128.
+ *   tile_w x tile_h: pixel tile of the kernels with one thread per pixel (G-buffer, the gated wavefronts'
+ *     selection, the single kernels of histograms, the shrink mapping, the ellipsoidal connection and large
+ *     gated views); tile_w a power of two in [4, 32], tile_w * tile_h = 64 or 128.  The initial stage with a
+ *     thread per path tree (allocation-free form, small views of a batch) has tiles of its own.
  *   packet: blocks of 128 threads per SM that pull shift and visibility tasks in the persistent
  *     reuse kernels (the width of the task packets in flight per SM), 1..8; 0 = as many as fit.
  *     Fewer leave room for other instances of a batch to run beside this one.
  *   layout: TOF_LAYOUT_SOA (six 16-byte planes, the default) or TOF_LAYOUT_AOS (each reservoir's
  *     96 bytes contiguous).
- * In a staged batch (tof_render_batch) the per-pixel stages run blocks of 128 threads, tiles of
- * tile_w x (128 / tile_w) pixels, and the persistent stages run as many blocks as fit: there only
- * tile_w and the layout of a view's tuning apply. */
+ * In a staged batch (tof_render_batch) the G-buffer runs blocks of 128 threads, tiles of
+ * tile_w x (128 / tile_w) pixels, and the reuse passes' persistent stages run as many blocks as fit: there
+ * tile_w and the layout of a view's tuning apply, and tile_h and packet in the initial stage of views of
+ * 256 x 256 pixels and more. */
 #define TOF_LAYOUT_SOA 0
 #define TOF_LAYOUT_AOS 1
 typedef struct {

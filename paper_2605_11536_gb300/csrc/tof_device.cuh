@@ -885,8 +885,10 @@ static __device__ __noinline__ void build_rec(const Domain& D, const TreeVerts& 
 // Fixed rounding.  The shift's functions with every multiplication and addition rounded in one given way (a
 // dot product as fma(z, z', fma(x, x', y y')), a difference of products as fma(a, b, -(c d))).  Left to the
 // compiler, which products it fuses depends on how often each is used nearby, so the same expression
-// rounds differently in code that is cut in another way; here a shift's bits do not depend on which kernel
-// runs it, and these are the roundings that the one-kernel form had.
+// rounds differently in code that is cut in another way; here these steps' bits do not depend on which kernel
+// runs them, and the roundings are those that the one-kernel form had.  Left to the compiler are the primary hit's
+// domain (make_domain_hit) and the walk to a neighbouring triangle (walk_bary, walk_corner, walk_locate): a walking
+// shift's bits may depend on its kernel.
 // ============================================================================================
 static __device__ __forceinline__ float dot3c(float3 a, float3 b) {
     return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));

@@ -368,7 +368,9 @@ __global__ void __launch_bounds__(128, kShiftBlocks) shift_fwd_kernel(const __gr
 
 // --------------------------------------------------------------------------------------------
 // visibility segments queued by a shift kernel (trace_queue); an occluded segment zeroes the result it
-// guards.  Each segment's node visits are those of traverse<true>, so the answer is the same.
+// guards.  Whether anything is hit does not depend on the order of the tests, so the answer is that of
+// traverse<true>, although a segment may visit up to kQueueRun - 1 more nodes than it: the leaves of a round are
+// tested after the round's visits.
 // stat >= 0: the stats counter that counted the guarded shifts as successes (one decrement per
 // shift, however many of its segments are occluded); ray_stat >= 0: the counter of segments.
 // --------------------------------------------------------------------------------------------
