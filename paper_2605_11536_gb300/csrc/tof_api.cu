@@ -38,7 +38,7 @@ cudaError_t launch_laser(const GeomDev& g, float3 o, float3 d, float power, Ligh
 cudaError_t launch_xform(int nt, const float* vloc, const uint32_t* tris, const uint32_t* triobj, const uint32_t* objmat,
                          const float* xf, float4* tri_out, float4* cent, uint32_t* bb, cudaStream_t s);
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
-                                  uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
+                                  uint32_t* vals2, int* child, int* parent_int, int* parent_leaf,
                                   uint32_t* counter, uint32_t** prim_out, float4* scratch, cudaStream_t s);
 cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
                             int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut, float4* boxes,
@@ -74,7 +74,7 @@ struct SceneH {
     float4* mats = nullptr;
     float* xf = nullptr;
     float4* cent = nullptr;
-    uint32_t *keys = nullptr, *vals = nullptr, *keys2 = nullptr, *vals2 = nullptr, *hist = nullptr, *bb = nullptr;
+    uint32_t *keys = nullptr, *vals = nullptr, *keys2 = nullptr, *vals2 = nullptr, *bb = nullptr;
     uint32_t* prim = nullptr;   // points into vals after a build
     int *child = nullptr, *parent_int = nullptr, *parent_leaf = nullptr;
     uint32_t* counter = nullptr;
@@ -536,8 +536,6 @@ tof_status tof_scene_upload(tof_ctx* c, const float* verts, uint32_t nv, const u
     TRY(dalloc(c, &S.vals, sizeof(uint32_t) * nt, "vals"));
     TRY(dalloc(c, &S.keys2, sizeof(uint32_t) * nt, "keys2"));
     TRY(dalloc(c, &S.vals2, sizeof(uint32_t) * nt, "vals2"));
-    int ntiles = ((int)nt + 2047) / 2048;
-    TRY(dalloc(c, &S.hist, sizeof(uint32_t) * 256 * (size_t)ntiles, "histogram"));
     TRY(dalloc(c, &S.bb, sizeof(uint32_t) * 8, "bounds"));
     TRY(dalloc(c, &S.child, sizeof(int) * 2 * nt, "children"));
     TRY(dalloc(c, &S.parent_int, sizeof(int) * nt, "parents"));
@@ -594,7 +592,7 @@ tof_status tof_scene_destroy(tof_ctx* c, tof_scene id) {
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     SceneH& S = c->scenes[id];
-    void* ps[] = {S.vloc, S.tris, S.triobj, S.objmat, S.mats, S.xf, S.cent, S.keys, S.vals, S.keys2, S.vals2, S.hist, S.bb,
+    void* ps[] = {S.vloc, S.tris, S.triobj, S.objmat, S.mats, S.xf, S.cent, S.keys, S.vals, S.keys2, S.vals2, S.bb,
                   S.child, S.parent_int, S.parent_leaf, S.counter, S.tri[0], S.tri[1], S.leaf[0], S.leaf[1], S.nodes[0], S.nodes[1],
                   S.adj, S.enode[0], S.enode[1]};
     for (void* p : ps) dfree(c, p);
@@ -620,15 +618,17 @@ tof_status tof_bvh_build(tof_ctx* c, tof_scene id, const float* xf, int refit_on
     if (full && whole_build(S.nt)) {
         S.prim = S.vals;
         CK(launch_whole(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, s));
-    } else if (full) {
-        CK(launch_build_topology(S.nt, S.cent, S.bb, S.keys, S.vals, S.keys2, S.vals2, S.hist, S.child, S.parent_int,
-                                 S.parent_leaf, S.counter, &S.prim, S.cent, s));
-    }
-    if (full && S.nt > 1 && !whole_build(S.nt)) {
+    } else if (full && S.nt > 1) {
         if (!c->sms) CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
+        CK(launch_build_topology(S.nt, S.cent, S.bb, S.keys, S.vals, S.keys2, S.vals2, S.child, S.parent_int, S.parent_leaf, S.counter, &S.prim,
+                                 S.cent, s));
         CK(launch_treelets(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, S.keys2,
                            S.vals2, S.bb + 6, S.cent, c->sms, s));
-    } else if (!full || S.nt == 1) {
+    } else {
+        if (full) {   // one triangle
+            S.prim = S.vals;
+            CK(cudaMemsetAsync(S.prim, 0, sizeof(uint32_t), s));
+        }
         CK(launch_refit(S.nt, S.prim, S.tri[slot], S.leaf[slot], S.nodes[slot], S.child, S.parent_int, S.parent_leaf, S.counter, s));
     }
     if (S.enode[slot]) CK(launch_etree(S.nt, S.eP, S.tri[slot], S.enode[slot], s));

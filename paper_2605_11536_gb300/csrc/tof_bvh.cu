@@ -341,8 +341,6 @@ __global__ void karras_kernel(int n, const uint32_t* __restrict__ keys, int* __r
     if (last - first + 1 > kTreelet) {
         if (g - first + 1 <= kTreelet) list_cut(first, g, left, cut_a, cut_m, ncut);
         if (last - g <= kTreelet) list_cut(g + 1, last, right, cut_a, cut_m, ncut);
-    } else if (i == 0) {
-        list_cut(0, n - 1, 0, cut_a, cut_m, ncut);
     }
 }
 
@@ -818,7 +816,6 @@ __global__ void __launch_bounds__(kTopItems) treelet_top_kernel(int n, const uin
     __shared__ int s_no_slot, s_slot0;   // the item without a free number; the item whose free number is 0
     const int p = threadIdx.x;
     const int R = (int)*ncut;
-    if (R == 1) { wait_for_treelets(); return; }
     if (top_by_area(R, n)) {
         if (p < R) {
             const int a = (int)cut_a[p], m = (int)(cut_m[p] & ~kRootLast);
@@ -862,7 +859,7 @@ __global__ void __launch_bounds__(256) morton_top_kernel(int n, const uint32_t* 
                                                          const uint32_t* __restrict__ cut_a, const uint32_t* __restrict__ cut_m,
                                                          const uint32_t* __restrict__ ncut) {
     const int R = (int)*ncut;
-    if (R == 1 || top_by_area(R, n)) return;
+    if (top_by_area(R, n)) return;
     for (int r = blockIdx.x * 256 + threadIdx.x; r < R; r += gridDim.x * 256)
         climb_range(r, n, prim, tri, nodes, child, parent_int, parent_leaf, counter, cut_a, cut_m);
 }
@@ -961,9 +958,9 @@ static int sort_blocks(const void* kernel, int form) {
 // tiles of 1024 with scanned rows: 400k 62, elsewhere slower than the best of these.)
 constexpr int kAddTiles = 110, kScanTiles = 600;
 
-// full build of the hierarchy (prim order, children, parents) from the centroids
+// full build of the hierarchy (prim order, children, parents) from the centroids, n > kWhole
 cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint32_t* keys, uint32_t* vals, uint32_t* keys2,
-                                  uint32_t* vals2, uint32_t* hist, int* child, int* parent_int, int* parent_leaf,
+                                  uint32_t* vals2, int* child, int* parent_int, int* parent_leaf,
                                   uint32_t* counter, uint32_t** prim_out, float4* scratch, cudaStream_t s) {
     note_launch();
     bounds_kernel<<<min(1024u, blocks(n, 256)), 256, 0, s>>>(n, cent, bb);
@@ -971,8 +968,8 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
     morton_kernel<<<blocks(n, 256), 256, 0, s>>>(n, cent, bb, keys, vals);
     uint32_t *ki = keys, *vi = vals, *ko = keys2, *vo = vals2;
     // the histograms (and the scans' totals) lie in the centroids' memory, which the Morton codes were the last to
-    // read: at most 2 B a key and 1 KB of its 16 B a key
-    uint32_t* counts = n > kWhole ? reinterpret_cast<uint32_t*>(scratch) : hist;
+    // read: at most 2 B a key and 2 KB of its 16 B a key (n > kWhole)
+    uint32_t* counts = reinterpret_cast<uint32_t*>(scratch);
     int nt = (n + kCoopTile - 1) / kCoopTile;
     const void* sort = nt <= kAddTiles ? (const void*)radix_sort_coop_kernel<false> : (const void*)radix_sort_coop_kernel<true>;
     if (nt <= kScanTiles && nt <= sort_blocks(sort, nt <= kAddTiles ? 0 : 1)) {
@@ -994,7 +991,8 @@ cudaError_t launch_build_topology(int n, const float4* cent, uint32_t* bb, uint3
         }
     }
     // after 4 passes the sorted keys / prims are back in keys / vals
-    if (n > 1) { note_launch(); karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6, n > kClimbBlock ? counter : nullptr); }
+    note_launch();
+    karras_kernel<<<blocks(n - 1, 256), 256, 0, s>>>(n, ki, child, parent_int, parent_leaf, keys2, vals2, bb + 6, n > kClimbBlock ? counter : nullptr);
     *prim_out = vi;
     return cudaGetLastError();
 }
@@ -1029,7 +1027,7 @@ cudaError_t launch_whole(int n, uint32_t* prim, const float4* tri, float4* leaf,
     return cudaGetLastError();
 }
 
-// boxes, leaf records and the treelets' topology of a full build (n > 1), after launch_build_topology
+// boxes, leaf records and the treelets' topology of a full build, after launch_build_topology
 cudaError_t launch_treelets(int n, uint32_t* prim, const float4* tri, float4* leaf, float4* nodes, int* child, int* parent_int,
                             int* parent_leaf, uint32_t* counter, const uint32_t* cut_a, const uint32_t* cut_m, const uint32_t* ncut,
                             float4* boxes, int sms, cudaStream_t s) {
