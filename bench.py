@@ -72,15 +72,15 @@ BYTES = {
 # kernel changes; the hash below ties the figures to the sources they were captured on.
 ELL_WAVE = "ell_trees_kernel + ell_place_kernel + ell_select_kernel"
 TREE_WAVE = "tw_start_kernel + 3 x (tw_hit_kernel + tw_shade_kernel) + vis_kernel + tree_select_kernel"
-NCU_TRAFFIC_SRC = "3739f9029c5b"   # _src_hash() of the sources the figures below were captured on
+NCU_TRAFFIC_SRC = "68c21e20a1c9"   # _src_hash() of the sources the figures below were captured on
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch (one stage for the initial wavefront),
 # frame 5 (profiles/kernels_dynamic_gated_512.md)
-NCU_TRAFFIC = {TREE_WAVE: 313.60e6, "shift_inv_kernel<0, 1>": 99.83e6 + 64.69e6, "shift_fwd_kernel<0, 1>": 50.43e6 + 41.61e6,
-               "vis_kernel (inverse segments)": 88.78e6 + 2.95e6, "reuse_merge_kernel": 115.74e6 + 7.46e6}
+NCU_TRAFFIC = {TREE_WAVE: 313.92e6, "shift_inv_kernel<0, 1>": 99.96e6 + 64.67e6, "shift_fwd_kernel<0, 1>": 50.35e6 + 41.37e6,
+               "vis_kernel (inverse segments)": 88.76e6 + 2.95e6, "reuse_merge_kernel": 115.77e6 + 7.39e6}
 # L1 / L2 sector hit rates (%) and active lanes per warp instruction of the traversal-bound kernels,
 # from the same capture (the initial wavefront's first closest-hit round)
-NCU_HIT = {"tw_hit_kernel": [79.7, 69.6, 14.6], "shift_fwd_kernel<0, 1>": [49.9, 58.8, 19.5],
-           "shift_inv_kernel<0, 1>": [64.4, 51.7, 21.1], "vis_kernel": [91.3, 66.0, 16.5]}
+NCU_HIT = {"tw_hit_kernel": [79.7, 69.7, 14.5], "shift_fwd_kernel<0, 1>": [49.9, 58.9, 19.5],
+           "shift_inv_kernel<0, 1>": [64.5, 51.8, 21.1], "vis_kernel": [91.5, 65.7, 16.5]}
 
 
 def _peaks():
